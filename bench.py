@@ -1130,7 +1130,7 @@ def main():
     single = ["gcn_aggregate", "edge_softmax", "pool_mean", "pool_max"]
     dom = max(single, key=lambda k: kernels[k]["ms"])
     traffic = measured_traffic(dom)
-    roof = {"kernel": {"gcn_aggregate": "aggregate_mp_kernel", "edge_softmax": "softmax_fast (+ node_scores prologue)",
+    roof = {"kernel": {"gcn_aggregate": "aggregate_rows", "edge_softmax": "softmax_fast (+ node_scores prologue)",
                        "pool_mean": "pool_kernel", "pool_max": "pool_kernel"}[dom],
             "call": dom, "bound": "hbm", "achieved": kernels[dom]["gbs"], "peak": hbm_peak,
             "unit": "GB/s", "frac": round(kernels[dom]["gbs"] / hbm_peak, 4), "traffic": traffic,

@@ -35,24 +35,18 @@ bool aligned_to(const void *p, uintptr_t b) { return reinterpret_cast<uintptr_t>
 
 // One hop.  x = h_k (x0 itself for k = 0), a.out = h_{k+1}.
 template <typename X0T>
-cudaError_t launch_hop(AggArgs a, bool first, cudaStream_t s) {
+cudaError_t launch_hop(const AggArgs &a, bool first, cudaStream_t s) {
     const int64_t f = a.f;
     const bool out16 = aligned_to(a.out, 16);
     if (first) {   // h_0 = x0: the gathered rows and the teleport rows share one type
-        if constexpr (sizeof(X0T) == 2) {
-            if (out16 && aligned_to(a.x, 16) && f % 8 == 0)
-                return launch_lpr<X0T, 8, kAppnp, X0T>(a, lanes_per_row(f / 8), s);
-            return launch_lpr<X0T, 1, kAppnp, X0T>(a, lanes_per_row(f), s);
-        } else {
-            if (out16 && aligned_to(a.x, 16) && f % 4 == 0)
-                return launch_lpr<float, 4, kAppnp, float>(a, lanes_per_row(f / 4), s);
-            return launch_lpr<float, 1, kAppnp, float>(a, lanes_per_row(f), s);
-        }
+        constexpr int vec = sizeof(X0T) == 2 ? 8 : 4;
+        if (out16 && aligned_to(a.x, 16) && f % vec == 0) return launch_rows_vec<X0T, vec, kAppnp>(a, s);
+        return launch_rows_scalar<X0T, kAppnp>(a, s);
     }
     // fp32 iterate; x0 rows are read 4 at a time (16 bytes fp32, 8 bytes bf16)
     if (out16 && aligned_to(a.x, 16) && f % 4 == 0 && aligned_to(a.x0, 4 * sizeof(X0T)))
-        return launch_lpr<float, 4, kAppnp, X0T>(a, lanes_per_row(f / 4), s);
-    return launch_lpr<float, 1, kAppnp, X0T>(a, lanes_per_row(f), s);
+        return launch_rows_vec<float, 4, kAppnp, X0T>(a, s);
+    return launch_rows_scalar<float, kAppnp, X0T>(a, s);
 }
 
 }  // namespace
@@ -81,7 +75,7 @@ cudaError_t launch_propagate(const int32_t *rowptr, const int32_t *col, const fl
     const void *h = x0;
     for (int64_t k = 0; k < hops; ++k) {
         float *dst = ((hops - 1 - k) % 2 == 0) ? out : spare;
-        AggArgs a{rowptr, col, w, dinv, h, dst, n, f, 0, add_self, fill, x0, alpha, beta, kRegimeAny};
+        const AggArgs a{rowptr, col, w, dinv, h, dst, n, f, 0, add_self, fill, x0, alpha, beta};
         const cudaError_t err = x_dtype == TFG_BF16 ? launch_hop<uint16_t>(a, k == 0, s)
                                                     : launch_hop<float>(a, k == 0, s);
         if (err != cudaSuccess) return err;

@@ -1,0 +1,65 @@
+"""The row walk of the aggregations (agg.cuh) where its layout changes: feature
+counts on both sides of every lanes-per-row and features-per-lane choice, rows
+that end inside, at and after a 32-edge window, empty rows, a row shared by all
+warps of a CTA, and weights with an infinity in a row that no edge names."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from _helpers import TOL_F32, assert_exact_f32, assert_scaled_close, dev, features, host_features
+from paper_2101_11552_gb300 import graphgen as gg
+from paper_2101_11552_gb300 import tfg
+
+pytestmark = pytest.mark.gpu
+
+# degrees around the 32-edge window, runs of empty rows, one hub
+DEGREES = [0, 1, 31, 32, 33, 0, 0, 64, 5, 3, 9000, 2, 0, 95, 96, 97] + [3, 0, 7] * 40
+
+
+def graph(seed):
+    rng = np.random.default_rng(seed)
+    deg = np.array(DEGREES)
+    n = len(deg)
+    dst = np.repeat(np.arange(n), deg)
+    src = rng.integers(0, n - 1, size=dst.size)      # the last node is nobody's source
+    order = rng.permutation(dst.size)
+    return np.ascontiguousarray(np.stack([src[order], dst[order]]).astype(np.int64)), n
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("f", [2, 7, 8, 9, 16, 17, 31, 32, 33, 41, 48, 49, 64, 65, 96, 97, 100, 128,
+                               129, 132, 200, 256, 257, 264, 392])
+def test_widths(f, dtype):
+    ei, n = graph(f)
+    rng = np.random.default_rng(1000 + f)
+    x = rng.standard_normal((n, f), dtype=np.float32)
+    x[-1] = np.inf                                    # reaches no row but its own
+    wl = gg.Workload("walk", n, ei, x, x_bf16=gg.bf16_bits_rne(x))
+    ew = rng.uniform(-1.5, 1.5, ei.shape[1]).astype(np.float32)
+    csr = tfg.tfg_build_csr(dev(ei), n)
+    xd = features(wl, dtype)
+    finite = host_features(wl, dtype).copy()
+    finite[-1] = 0
+    for w in (None, ew):
+        wd = None if w is None else dev(w).index_select(0, csr.perm)
+        for reduce, fn in (("sum", tfg.tfg_aggregate_sum), ("mean", tfg.tfg_aggregate_mean),
+                           ("max", tfg.tfg_aggregate_max)):
+            got = fn(csr.rowptr, csr.col, xd, wd).cpu().numpy()
+            ref, scale = oracle.aggregate(ei, n, finite, reduce, w=w)
+            if reduce == "max":
+                assert_exact_f32(got, ref, f"max F={f}")
+            else:
+                assert_scaled_close(got, ref, scale, TOL_F32, f"{reduce} F={f}")
+        dinv, w_csr = tfg.tfg_gcn_norm(csr.rowptr, csr.col, csr.perm, n,
+                                       None if w is None else dev(np.abs(w)), 1, 1.0,
+                                       want_w_csr=w is not None)
+        got = tfg.tfg_gcn_aggregate_sum(csr.rowptr, csr.col, dinv, xd, w_csr, 1, 1.0).cpu().numpy()
+        ref, scale = oracle.gcn_aggregate(ei, n, finite, None if w is None else np.abs(w), 1, 1.0)
+        assert np.isinf(got[-1]).all()
+        assert_scaled_close(got[:-1], ref[:-1], scale[:-1], TOL_F32, f"gcn F={f}")
+    out = tfg.tfg_appnp_propagate(csr.rowptr, csr.col, dinv, dev(finite) if dtype == "f32" else
+                                  dev(finite.view(np.int16)).view(torch.bfloat16), 3, 0.1,
+                                  add_self_loops=1).cpu().numpy()
+    dw = np.abs(ew)
+    assert np.isfinite(out).all() and dw.size       # values: test_gpu_propagate; here every width runs
