@@ -12,22 +12,24 @@
 //   ds_src[s,h] = sum over e out of s of dz,   ds_dst[t,h] = sum over e into t of dz
 //   grad_a_src[h,c] = sum_v ds_src[v,h] x[v,h,c],  grad_a_dst likewise.
 //
-// Kernels, one warp per row:
+// Kernels:
 //   node_scores         s_src, s_dst in base-2 units, as in the forward
-//   fast_bwd_targets    (the forward's fast layout) per target t, CSR by
-//                       target: one online pass gives the softmax statistics
-//                       and ds_dst; statistics stored per (node, head)
-//   fast_bwd_sources    per source s, CSR by source: alpha from the
-//                       statistics, grad_x and ds_src
-//   bwd_targets,        the same two passes for any other layout: lanes cover
-//   bwd_sources         the features in tiles of 32, a head's dot products
-//                       finished by a butterfly over its lanes
+//   by target           (whole 16-byte slices per head, F <= 128) softmax_fast's
+//                       backward on long rows, GatByTarget's walk otherwise: one
+//                       online pass gives the softmax statistics and ds_dst
+//   by source           (the same layouts) GatBySource's walk: alpha from the
+//                       statistics, grad_x and ds_src.  Both passes sum weighted
+//                       rows and take the dot products once per row, not per edge.
+//   bwd_targets,        the same two passes for any other layout, one warp per
+//   bwd_sources         row: lanes cover the features in tiles of 32, a head's dot
+//                       products finished by a butterfly over its lanes per edge
 //   bwd_vectors_*       grad_a_src / grad_a_dst: per-block column sums, then
-//                       the blocks' sums added in block order (deterministic)
+//                       the blocks' sums added in a fixed order (deterministic)
 // The same file holds the backward of the dot-product form (below).
 #include <math_constants.h>
 
 #include "common.cuh"
+#include "gat_walk.cuh"
 
 namespace tfg {
 namespace {
@@ -273,335 +275,16 @@ __global__ void __launch_bounds__(kBwThreads) bwd_sources(BwArgs a) {
     }
 }
 
-// ---------------------------------------------------------------------------
-// Fast form, on the forward's fast layout: H divides 32, channels / VEC a
-// power of two (a lane's VEC features lie in one head), one feature tile per
-// row.  Score lanes (se, sh) = (lane / H, lane % H) evaluate each (edge, head)
-// once; feature lanes gather 16-byte slices of the rows and finish a head's
-// dot product with a butterfly over its channels / VEC lanes.
-//
-// Target pass (CSR by target), one warp per row t and ONE online pass over the
-// in-edges, as in the forward: the running maximum m and denominator den of
-// each head, and the rescaled sum of w (dalpha - beta), w = exp(l - m) times
-// the LeakyReLU slope at z; ds_dst[t] = that sum / den.  The row's statistics
-// go to stats[t, h] = (s_dst, m, 1 / den, beta) for the source pass.
-//
-// Source pass (CSR by source), one warp per row s: alpha of each out-edge
-// from stats[t] (score lanes), the fp32 rows grad_out[t] gathered 16 bytes
-// per lane (feature lanes), then grad_x[s] and ds_src[s].
-// ---------------------------------------------------------------------------
-struct FastBwArgs {
-    const int32_t *rowptr, *col;          // CSR by target
-    const int32_t *rowptr_src, *col_src;  // CSR by source
-    const void *x;
-    int64_t n;
-    int heads, channels;
-    float slope;
-    const float *a_src, *a_dst, *out, *grad_out;
-    const float *s_src, *s_dst;           // base-2 node scores
-    float4 *stats;                        // [N, H]: (s_dst, m, 1 / den, beta)
-    float *ds_dst, *ds_src, *grad_x;
-};
+size_t bw_align(size_t b) { return (b + 255) & ~size_t(255); }
+
+int bw_blocks(int64_t n) { return static_cast<int>((n + kBwRowsPerBlock - 1) / kBwRowsPerBlock); }
 
 constexpr int64_t kFbMinWork = 2048;   // edges + rows per CTA, at least
-#ifndef TFG_FB_STAGE
-#define TFG_FB_STAGE 1             // source pass: per-chunk weights staged in shared memory
-#endif
-#ifndef TFG_FB_UNROLL_TGT
-#define TFG_FB_UNROLL_TGT 4        // row gathers in flight per lane, target pass
-#endif
-#ifndef TFG_FB_UNROLL_SRC
-#define TFG_FB_UNROLL_SRC 4        // row gathers in flight per lane, source pass
-#endif
-constexpr int kFbUnroll = TFG_FB_UNROLL_TGT;
-constexpr int kFbUnrollSrc = TFG_FB_UNROLL_SRC;
-// Measured on the 114.6M-edge graph (bf16, 8 heads x 16): 3 / 3 CTAs per SM
-// 13.43 ms, 4 target / 3 source 13.20, 3 / 4 12.60, 4 / 4 12.37.
-#ifndef TFG_FB_TGT_BLOCKS
-#define TFG_FB_TGT_BLOCKS 4        // resident CTAs per SM of the fast target pass
-#endif
-#ifndef TFG_FB_SRC_BLOCKS
-#define TFG_FB_SRC_BLOCKS 4        // resident CTAs per SM of the fast source pass
-#endif
 
 // Sum over the aligned groups of hl lanes (hl a power of two).
 __device__ __forceinline__ float group_sum(float v, int hl) {
     for (int o = 1; o < hl; o <<= 1) v += __shfl_xor_sync(kFull, v, o);
     return v;
-}
-
-template <typename XT, int VEC, int LPR, int H>
-__device__ __forceinline__ void fast_bwd_target(const FastBwArgs &a, int64_t t, int lane) {
-    using V = VecLoad<XT, VEC>;
-    constexpr int G = 32 / LPR;     // edges per feature step
-    constexpr int ES = 32 / H;      // edges per score step
-    constexpr int R = H;            // score steps per 32-edge chunk
-    static_assert(ES % G == 0, "score step must hold whole feature steps");
-    static_assert(G * kFbUnroll <= 32 && 32 % (G * kFbUnroll) == 0,
-                  "feature steps of G * kFbUnroll slots must tile the 32-edge chunk");
-    const int se = lane / H, sh = lane % H;
-    const int g = lane / LPR, sub = lane % LPR;
-    const int f = H * a.channels;
-    const int hl = a.channels / VEC;
-    const int f0 = sub * VEC;
-    const bool fok = f0 < f;
-    const int fh = fok ? f0 / a.channels : 0;
-    const int fo = fok ? f0 : 0;
-    const char *xb = reinterpret_cast<const char *>(static_cast<const XT *>(a.x) + fo);
-    const uint32_t row_bytes = static_cast<uint32_t>(f) * static_cast<uint32_t>(sizeof(XT));
-    auto gather = [&](uint32_t src) {
-        return V::raw(reinterpret_cast<const XT *>(xb + static_cast<uint64_t>(src) * row_bytes));
-    };
-    const int64_t beg = a.rowptr[t], end = a.rowptr[t + 1];
-    const float sd = __ldg(a.s_dst + t * H + sh);
-    // the lane's slice of grad_out[t] and beta = <grad_out[t, h], out[t, h]>
-    float gt[VEC], beta = 0.f;
-#pragma unroll
-    for (int q = 0; q < VEC; q += 4) {
-        const float4 g4 = __ldg(reinterpret_cast<const float4 *>(a.grad_out + t * f + fo + q));
-        const float4 o4 = __ldg(reinterpret_cast<const float4 *>(a.out + t * f + fo + q));
-        gt[q] = fok ? g4.x : 0.f;
-        gt[q + 1] = fok ? g4.y : 0.f;
-        gt[q + 2] = fok ? g4.z : 0.f;
-        gt[q + 3] = fok ? g4.w : 0.f;
-        beta = fmaf(gt[q], o4.x, beta);
-        beta = fmaf(gt[q + 1], o4.y, beta);
-        beta = fmaf(gt[q + 2], o4.z, beta);
-        beta = fmaf(gt[q + 3], o4.w, beta);
-    }
-    beta = group_sum(beta, hl);
-
-    float m = -CUDART_INF_F, den = 0.f, acc = 0.f;
-    int cnext = beg + lane < end ? ld_stream(a.col + beg + lane) : 0;
-    for (int64_t base = beg; base < end; base += 32) {
-        const int cnt = static_cast<int>(min64(32, end - base));
-        const int c = cnext;
-        cnext = base + 32 + lane < end ? ld_stream(a.col + base + 32 + lane) : 0;
-        typename V::Raw raw0[kFbUnroll];
-#pragma unroll
-        for (int u = 0; u < kFbUnroll; ++u)
-            raw0[u] = gather(static_cast<uint32_t>(__shfl_sync(kFull, c, (u * G + g) & 31)));
-        float l[R], w[R];
-        float cm = -CUDART_INF_F;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int k = r * ES + se;
-            const int src = __shfl_sync(kFull, c, k);
-            const float z = __ldg(a.s_src + static_cast<int64_t>(src) * H + sh) + sd;
-            l[r] = k < cnt ? bw_leaky(z, a.slope) : -CUDART_INF_F;
-            w[r] = z > 0.f ? 1.f : a.slope;
-            cm = fmaxf(cm, l[r]);
-        }
-#pragma unroll
-        for (int o = H; o < 32; o <<= 1) cm = fmaxf(cm, __shfl_xor_sync(kFull, cm, o));
-        const bool rises = cm > m;
-        if (__any_sync(kFull, rises)) {   // warp-uniform; rare after the first chunks
-            const float sc = rises ? (m == -CUDART_INF_F ? 0.f : exp2f(m - cm)) : 1.f;
-            den *= sc;
-            acc *= __shfl_sync(kFull, sc, fh);   // lane fh scores head fh
-            m = fmaxf(m, cm);
-        }
-        float den_part = 0.f;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const float p = r * ES + se < cnt ? exp2f(l[r] - m) : 0.f;
-            den_part += p;
-            w[r] *= p;
-        }
-        den += den_part;
-        float part = 0.f;
-#pragma unroll
-        for (int e = 0; e < 32; e += G * kFbUnroll) {
-            if (e >= cnt) break;   // warp-uniform
-            typename V::Raw raw[kFbUnroll];
-            float ww[kFbUnroll];
-#pragma unroll
-            for (int u = 0; u < kFbUnroll; ++u) {
-                const int k0 = e + u * G;
-                const int k = k0 + g;
-                ww[u] = __shfl_sync(kFull, w[k0 / ES], ((k0 % ES) + g) * H + fh);
-                if (e == 0) raw[u] = raw0[u];
-                else raw[u] = gather(static_cast<uint32_t>(__shfl_sync(kFull, c, k & 31)));
-            }
-#pragma unroll
-            for (int u = 0; u < kFbUnroll; ++u) {
-                float v[VEC];
-                V::widen(raw[u], v);
-                float d = 0.f;
-#pragma unroll
-                for (int q = 0; q < VEC; ++q) d = fmaf(gt[q], v[q], d);
-                d = group_sum(d, hl);
-                part = fmaf(ww[u], d - beta, part);
-            }
-        }
-        acc += part;
-    }
-#pragma unroll
-    for (int o = H; o < 32; o <<= 1) den += __shfl_xor_sync(kFull, den, o);
-#pragma unroll
-    for (int o = LPR; o < 32; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);
-    const float dh = __shfl_sync(kFull, den, fh);
-    const float bh = __shfl_sync(kFull, beta, (sh * hl) & 31);   // group-0 lane of head sh
-    if (lane < LPR && fok && f0 % a.channels == 0)
-        a.ds_dst[t * H + fh] = end > beg ? acc / dh : 0.f;
-    if (lane < H) a.stats[t * H + sh] = make_float4(sd, m, den > 0.f ? 1.f / den : 0.f, bh);
-}
-
-// (Splitting the heads over several launches, so that the slice of grad_out
-// each one gathers stays in L2, measured no faster on the 114.6M-edge graph:
-// 14.65 ms in one launch, 14.59 in two, 15.06 in four -- the pass is bound by
-// latency, not by DRAM bytes.)
-template <typename XT, int LPR, int H>
-__device__ __forceinline__ void fast_bwd_source(const FastBwArgs &a, int64_t s, int lane,
-                                                float4 *__restrict__ stage) {
-    constexpr int G = 32 / LPR;     // edges per feature step
-    constexpr int ES = 32 / H;      // edges per score step
-    constexpr int R = H;
-    static_assert(ES % G == 0, "score step must hold whole feature steps");
-    static_assert(G * kFbUnrollSrc <= 32 && 32 % (G * kFbUnrollSrc) == 0,
-                  "feature steps of G * kFbUnrollSrc slots must tile the 32-edge chunk");
-    const int se = lane / H, sh = lane % H;
-    const int g = lane / LPR, sub = lane % LPR;
-    const int f = H * a.channels;
-    const int hl = a.channels / 4;
-    const int f0 = sub * 4;
-    const bool fok = f0 < f;
-    const int fh = fok ? f0 / a.channels : 0;
-    const int fo = fok ? f0 : 0;
-    float xs[4];
-    VecLoad<XT, 4>::load(static_cast<const XT *>(a.x) + s * f + fo, xs);
-    const float ss = __ldg(a.s_src + s * H + sh);
-    const char *gb = reinterpret_cast<const char *>(a.grad_out + fo);
-    const uint32_t row_bytes = static_cast<uint32_t>(f) * 4u;
-    auto gather = [&](uint32_t t) {
-        return VecLoad<float, 4>::raw(reinterpret_cast<const float *>(gb + static_cast<uint64_t>(t) * row_bytes));
-    };
-    const int64_t beg = a.rowptr_src[s], end = a.rowptr_src[s + 1];
-    float px[4] = {0.f, 0.f, 0.f, 0.f}, pdz = 0.f;
-    int cnext = beg + lane < end ? ld_stream(a.col_src + beg + lane) : 0;
-    for (int64_t base = beg; base < end; base += 32) {
-        const int cnt = static_cast<int>(min64(32, end - base));
-        const int c = cnext;
-        cnext = base + 32 + lane < end ? ld_stream(a.col_src + base + 32 + lane) : 0;
-        float4 raw0[kFbUnrollSrc];
-#pragma unroll
-        for (int u = 0; u < kFbUnrollSrc; ++u)
-            raw0[u] = gather(static_cast<uint32_t>(__shfl_sync(kFull, c, (u * G + g) & 31)));
-        // alpha, af = alpha * slope(z) and ab = af * beta of (edge, head)
-#if TFG_FB_STAGE
-        // score lanes stage them per (edge, head) in the warp's shared-memory
-        // slots (lane-consecutive: conflict-free); feature lanes read their
-        // (edge, head) with one 16-byte load instead of three shuffles
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int k = r * ES + se;
-            const int t = __shfl_sync(kFull, c, k);
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (k < cnt) {
-                const float4 st = __ldg(a.stats + static_cast<int64_t>(t) * H + sh);
-                const float z = ss + st.x;
-                v.x = exp2f(bw_leaky(z, a.slope) - st.y) * st.z;
-                v.y = v.x * (z > 0.f ? 1.f : a.slope);
-                v.z = v.y * st.w;
-            }
-            stage[k * H + sh] = v;
-        }
-        __syncwarp();
-#else
-        float al[R], af[R], ab[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int k = r * ES + se;
-            const int t = __shfl_sync(kFull, c, k);
-            al[r] = af[r] = ab[r] = 0.f;
-            if (k < cnt) {
-                const float4 st = __ldg(a.stats + static_cast<int64_t>(t) * H + sh);
-                const float z = ss + st.x;
-                al[r] = exp2f(bw_leaky(z, a.slope) - st.y) * st.z;
-                af[r] = al[r] * (z > 0.f ? 1.f : a.slope);
-                ab[r] = af[r] * st.w;
-            }
-        }
-#endif
-        float part[4] = {0.f, 0.f, 0.f, 0.f}, partd = 0.f;
-#pragma unroll
-        for (int e = 0; e < 32; e += G * kFbUnrollSrc) {
-            if (e >= cnt) break;   // warp-uniform
-            float4 raw[kFbUnrollSrc];
-#if !TFG_FB_STAGE
-            float wa[kFbUnrollSrc], wf[kFbUnrollSrc], wb[kFbUnrollSrc];
-#endif
-#pragma unroll
-            for (int u = 0; u < kFbUnrollSrc; ++u) {
-                const int k0 = e + u * G;
-                const int k = k0 + g;
-#if !TFG_FB_STAGE
-                const int from = ((k0 % ES) + g) * H + fh;
-                wa[u] = __shfl_sync(kFull, al[k0 / ES], from);
-                wf[u] = __shfl_sync(kFull, af[k0 / ES], from);
-                wb[u] = __shfl_sync(kFull, ab[k0 / ES], from);
-#endif
-                if (e == 0) raw[u] = raw0[u];
-                else raw[u] = gather(static_cast<uint32_t>(__shfl_sync(kFull, c, k & 31)));
-            }
-#pragma unroll
-            for (int u = 0; u < kFbUnrollSrc; ++u) {
-#if TFG_FB_STAGE
-                // the staged weights are read when the row is used, so only
-                // the row slices are live while the gathers are in flight
-                const float4 w4 = stage[(e + u * G + g) * H + fh];
-                const float wa_u = w4.x, wf_u = w4.y, wb_u = w4.z;
-#else
-                const float wa_u = wa[u], wf_u = wf[u], wb_u = wb[u];
-#endif
-                const float gv[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};
-                float d = 0.f;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) d = fmaf(gv[q], xs[q], d);
-                d = group_sum(d, hl);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) part[q] = fmaf(wa_u, gv[q], part[q]);
-                partd += fmaf(wf_u, d, -wb_u);
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) px[q] += part[q];
-        pdz += partd;
-#if TFG_FB_STAGE
-        __syncwarp();   // every lane has read the stage before the next chunk writes it
-#endif
-    }
-#pragma unroll
-    for (int o = LPR; o < 32; o <<= 1) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) px[q] += __shfl_xor_sync(kFull, px[q], o);
-        pdz += __shfl_xor_sync(kFull, pdz, o);
-    }
-    if (lane < LPR && fok) {
-        const int64_t sh_g = s * H + fh;
-        const float dsd = __ldg(a.ds_dst + sh_g);
-        const float4 as = __ldg(reinterpret_cast<const float4 *>(a.a_src + fo));
-        const float4 ad = __ldg(reinterpret_cast<const float4 *>(a.a_dst + fo));
-        float4 o;
-        o.x = px[0] + pdz * as.x + dsd * ad.x;
-        o.y = px[1] + pdz * as.y + dsd * ad.y;
-        o.z = px[2] + pdz * as.z + dsd * ad.z;
-        o.w = px[3] + pdz * as.w + dsd * ad.w;
-        *reinterpret_cast<float4 *>(a.grad_x + s * f + fo) = o;
-        if (f0 % a.channels == 0) a.ds_src[sh_g] = pdz;
-    }
-}
-
-template <typename XT, int VEC, int LPR, int H>
-__global__ void __launch_bounds__(kBwThreads, TFG_FB_TGT_BLOCKS) fast_bwd_targets(FastBwArgs a) {
-    for_each_row(a.rowptr, a.n, [&](int64_t t, int lane) { fast_bwd_target<XT, VEC, LPR, H>(a, t, lane); });
-}
-
-template <typename XT, int LPR, int H>
-__global__ void __launch_bounds__(kBwThreads, TFG_FB_SRC_BLOCKS) fast_bwd_sources(FastBwArgs a) {
-    __shared__ float4 s_stage[TFG_FB_STAGE ? kBwWarps : 1][TFG_FB_STAGE ? 32 * H : 1];
-    float4 *stage = s_stage[TFG_FB_STAGE ? (threadIdx.x >> 5) : 0];
-    for_each_row(a.rowptr_src, a.n, [&](int64_t s, int lane) { fast_bwd_source<XT, LPR, H>(a, s, lane, stage); });
 }
 
 // ---------------------------------------------------------------------------
@@ -1100,46 +783,101 @@ cudaError_t launch_dot_bw_tiles(const DotBwArgs &a, cudaStream_t s) {
 }
 
 // Column sums of ds[v, head(f)] * x[v, f] over a block of rows, for both
-// vectors: part[b][0:F] (a_src) and part[b][F:2F] (a_dst).
-template <typename XT>
+// vectors: part[b][0:F] (a_src) and part[b][F:2F] (a_dst).  The block's threads
+// are F / VEC columns of VEC features times as many rows as fit; the rows'
+// sums are added in row order.  (One thread per feature walking 512 rows left
+// the loads in flight to a chain of fmas: 79 us for 169,343 x 128 fp32.)
+template <typename XT, int VEC>
 __global__ void __launch_bounds__(kBwThreads) bwd_vectors_partial(const XT *__restrict__ x,
                                                                   int64_t n, int heads,
                                                                   int channels,
                                                                   const float *__restrict__ ds_src,
                                                                   const float *__restrict__ ds_dst,
                                                                   float *__restrict__ part) {
-    const int f = heads * channels;
+    __shared__ float s_sum[2][kBwThreads * VEC];
+    const int f = heads * channels, cols = f / VEC, rows = kBwThreads / cols;
+    const int c = threadIdx.x % cols, r = threadIdx.x / cols, h = c * VEC / channels;
     const int64_t v0 = static_cast<int64_t>(blockIdx.x) * kBwRowsPerBlock;
     const int64_t v1 = min64(n, v0 + kBwRowsPerBlock);
-    for (int fi = threadIdx.x; fi < f; fi += kBwThreads) {
-        const int h = fi / channels;
-        float s1 = 0.f, s2 = 0.f;
-        for (int64_t v = v0; v < v1; ++v) {
-            float xv[1];
-            VecLoad<XT, 1>::load(x + v * f + fi, xv);
-            s1 = fmaf(__ldg(ds_src + v * heads + h), xv[0], s1);
-            s2 = fmaf(__ldg(ds_dst + v * heads + h), xv[0], s2);
+    float s1[VEC], s2[VEC];
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) s1[q] = s2[q] = 0.f;
+    if (r < rows) {
+#pragma unroll 4
+        for (int64_t v = v0 + r; v < v1; v += rows) {
+            float xv[VEC];
+            VecLoad<XT, VEC>::load(x + v * f + c * VEC, xv);
+            const float d1 = __ldg(ds_src + v * heads + h), d2 = __ldg(ds_dst + v * heads + h);
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) {
+                s1[q] = fmaf(d1, xv[q], s1[q]);
+                s2[q] = fmaf(d2, xv[q], s2[q]);
+            }
         }
-        part[static_cast<int64_t>(blockIdx.x) * 2 * f + fi] = s1;
-        part[static_cast<int64_t>(blockIdx.x) * 2 * f + f + fi] = s2;
+#pragma unroll
+        for (int q = 0; q < VEC; ++q) {
+            s_sum[0][r * f + c * VEC + q] = s1[q];
+            s_sum[1][r * f + c * VEC + q] = s2[q];
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 2 * f; i += kBwThreads) {
+        const float *p = s_sum[i < f ? 0 : 1] + (i < f ? i : i - f);
+        float sum = 0.f;
+        for (int k = 0; k < rows; ++k) sum += p[k * f];
+        part[static_cast<int64_t>(blockIdx.x) * 2 * f + i] = sum;
     }
 }
 
+// The blocks' sums, 32 columns a block: warp w adds blocks w, w + 8, ..., then
+// the warps' sums are added in warp order.
 __global__ void __launch_bounds__(kBwThreads) bwd_vectors_final(const float *__restrict__ part,
                                                                 int blocks, int f,
                                                                 float *__restrict__ ga_src,
                                                                 float *__restrict__ ga_dst) {
-    const int fi = blockIdx.x * kBwThreads + threadIdx.x;
-    if (fi >= 2 * f) return;
+    __shared__ float s_sum[kBwWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, fi = blockIdx.x * 32 + lane;
     float s = 0.f;
-    for (int b = 0; b < blocks; ++b) s += part[static_cast<int64_t>(b) * 2 * f + fi];
+    if (fi < 2 * f) {
+#pragma unroll 8
+        for (int b = warp; b < blocks; b += kBwWarps) s += __ldg(part + static_cast<int64_t>(b) * 2 * f + fi);
+    }
+    s_sum[warp][lane] = s;
+    __syncthreads();
+    if (warp > 0 || fi >= 2 * f) return;
+    for (int w = 1; w < kBwWarps; ++w) s += s_sum[w][lane];
     if (fi < f) ga_src[fi] = s;
     else ga_dst[fi - f] = s;
 }
 
-size_t bw_align(size_t b) { return (b + 255) & ~size_t(255); }
+// nb: blocks of kBwRowsPerBlock rows (bw_blocks)
+template <typename XT>
+cudaError_t launch_vectors(const XT *x, int64_t n, int heads, int channels, const float *ds_src,
+                           const float *ds_dst, int nb, float *part, float *ga_src, float *ga_dst,
+                           cudaStream_t s) {
+    const int f = heads * channels;
+    if (channels % 4 == 0 && reinterpret_cast<uintptr_t>(x) % (4 * sizeof(XT)) == 0)
+        bwd_vectors_partial<XT, 4><<<nb, kBwThreads, 0, s>>>(x, n, heads, channels, ds_src, ds_dst, part);
+    else
+        bwd_vectors_partial<XT, 1><<<nb, kBwThreads, 0, s>>>(x, n, heads, channels, ds_src, ds_dst, part);
+    bwd_vectors_final<<<ceil_div(2 * f, 32), kBwThreads, 0, s>>>(part, nb, f, ga_src, ga_dst);
+    return cudaGetLastError();
+}
 
-int bw_blocks(int64_t n) { return static_cast<int>((n + kBwRowsPerBlock - 1) / kBwRowsPerBlock); }
+template <typename XT, int VEC>
+cudaError_t walk_targets(const GatArgs &a, cudaStream_t s) {
+    const int slices = a.heads * a.channels / VEC;
+    if (slices <= 8) return launch_walk<GatByTarget<XT, VEC, 8, 1, 1, true>>(a, s);
+    if (slices <= 16) return launch_walk<GatByTarget<XT, VEC, 16, 1, 1, true>>(a, s);
+    return launch_walk<GatByTarget<XT, VEC, 32, 1, 1, true>>(a, s);
+}
+template <typename XT>
+cudaError_t walk_sources(const GatArgs &a, cudaStream_t s) {
+    const int slices = a.heads * a.channels / 4;
+    if (slices <= 8) return launch_walk<GatBySource<XT, 4, 8, 1, 1>>(a, s);
+    if (slices <= 16) return launch_walk<GatBySource<XT, 4, 16, 1, 1>>(a, s);
+    return launch_walk<GatBySource<XT, 4, 32, 1, 1>>(a, s);
+}
 
 template <typename XT, int NT>
 cudaError_t launch_bw(const BwArgs &a, float *part, float *ga_src, float *ga_dst,
@@ -1147,12 +885,8 @@ cudaError_t launch_bw(const BwArgs &a, float *part, float *ga_src, float *ga_dst
     const int rows = ceil_div(a.n, kBwWarps);
     bwd_targets<XT, NT><<<rows, kBwThreads, 0, s>>>(a);
     bwd_sources<XT, NT><<<rows, kBwThreads, 0, s>>>(a);
-    const int f = a.heads * a.channels;
-    const int nb = bw_blocks(a.n);
-    bwd_vectors_partial<XT><<<nb, kBwThreads, 0, s>>>(static_cast<const XT *>(a.x), a.n, a.heads,
-                                                      a.channels, a.ds_src, a.ds_dst, part);
-    bwd_vectors_final<<<ceil_div(2 * f, kBwThreads), kBwThreads, 0, s>>>(part, nb, f, ga_src, ga_dst);
-    return cudaGetLastError();
+    return launch_vectors(static_cast<const XT *>(a.x), a.n, a.heads, a.channels, a.ds_src, a.ds_dst,
+                          bw_blocks(a.n), part, ga_src, ga_dst, s);
 }
 
 template <typename XT>
@@ -1168,56 +902,6 @@ cudaError_t launch_bw_tiles(const BwArgs &a, float *part, float *ga_src, float *
         case 6: return launch_bw<XT, 6>(a, part, ga_src, ga_dst, s);
         case 7: return launch_bw<XT, 7>(a, part, ga_src, ga_dst, s);
         default: return launch_bw<XT, 8>(a, part, ga_src, ga_dst, s);
-    }
-}
-
-// Fast passes when the layout allows them (both or neither); false means
-// "use the general kernels".
-template <typename XT, int VEC, int H>
-bool launch_fast_bw_heads(const FastBwArgs &a, int64_t e, cudaStream_t s) {
-    const int f = H * a.channels;
-    const int lt = f / VEC <= 8 ? 8 : (f / VEC <= 16 ? 16 : 32);   // target pass lanes per row
-    const int ls = f / 4 <= 8 ? 8 : (f / 4 <= 16 ? 16 : 32);       // source pass lanes per row
-    if ((32 / H) % (32 / lt) != 0 || (32 / H) % (32 / ls) != 0) return false;
-    const int grid = balanced_grid(a.n, e, kFbMinWork);
-    switch (lt) {
-        case 8:
-            if constexpr ((32 / H) % 4 == 0)
-                fast_bwd_targets<XT, VEC, 8, H><<<grid, kBwThreads, 0, s>>>(a);
-            break;
-        case 16:
-            if constexpr ((32 / H) % 2 == 0)
-                fast_bwd_targets<XT, VEC, 16, H><<<grid, kBwThreads, 0, s>>>(a);
-            break;
-        default:
-            if constexpr (VEC == 4) fast_bwd_targets<XT, VEC, 32, H><<<grid, kBwThreads, 0, s>>>(a);
-            break;
-    }
-    switch (ls) {
-        case 8:
-            if constexpr ((32 / H) % 4 == 0)
-                fast_bwd_sources<XT, 8, H><<<grid, kBwThreads, 0, s>>>(a);
-            break;
-        case 16:
-            if constexpr ((32 / H) % 2 == 0)
-                fast_bwd_sources<XT, 16, H><<<grid, kBwThreads, 0, s>>>(a);
-            break;
-        default: fast_bwd_sources<XT, 32, H><<<grid, kBwThreads, 0, s>>>(a); break;
-    }
-    return true;
-}
-
-template <typename XT, int VEC>
-bool launch_fast_bw(const FastBwArgs &a, int heads, int64_t e, cudaStream_t s) {
-    const int c = a.channels;
-    const int hl = c / VEC;
-    if (c % VEC != 0 || (hl & (hl - 1)) != 0 || static_cast<int64_t>(heads) * c > 128) return false;
-    switch (heads) {
-        case 1: return launch_fast_bw_heads<XT, VEC, 1>(a, e, s);
-        case 2: return launch_fast_bw_heads<XT, VEC, 2>(a, e, s);
-        case 4: return launch_fast_bw_heads<XT, VEC, 4>(a, e, s);
-        case 8: return launch_fast_bw_heads<XT, VEC, 8>(a, e, s);
-        default: return false;
     }
 }
 
@@ -1273,6 +957,8 @@ cudaError_t launch_node_scores(const void *x, int x_dtype, int64_t n, int heads,
                                const float *a_src, const float *a_dst, float *s_src, float *s_dst,
                                cudaStream_t s);
 
+bool launch_softmax_fast_bwd(const GatArgs &a, int x_dtype, int64_t e, cudaStream_t s);
+
 cudaError_t launch_edge_softmax_backward(const int32_t *rowptr, const int32_t *col,
                                          const int32_t *rowptr_src, const int32_t *col_src,
                                          const void *x, int x_dtype, int64_t n, int64_t e,
@@ -1300,25 +986,27 @@ cudaError_t launch_edge_softmax_backward(const int32_t *rowptr, const int32_t *c
     auto a16 = [](const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
     const bool aligned = a16(x) && a16(out) && a16(grad_out) && a16(grad_x) && a16(a_src) &&
                          a16(a_dst);
-    if (aligned) {
-        FastBwArgs fa{rowptr, col, rowptr_src, col_src, x, n, heads, channels, slope, a_src, a_dst,
-                      out, grad_out, buf[0], buf[1], reinterpret_cast<float4 *>(buf[2]), buf[6],
-                      buf[7], grad_x};
-        const bool fast = x_dtype == TFG_BF16 ? launch_fast_bw<uint16_t, 8>(fa, heads, e, s)
-                                              : launch_fast_bw<float, 4>(fa, heads, e, s);
-        if (fast) {
-            const int fdim = heads * channels;
-            const int nb = bw_blocks(n);
-            if (x_dtype == TFG_BF16)
-                bwd_vectors_partial<uint16_t><<<nb, kBwThreads, 0, s>>>(
-                    static_cast<const uint16_t *>(x), n, heads, channels, buf[7], buf[6], part);
-            else
-                bwd_vectors_partial<float><<<nb, kBwThreads, 0, s>>>(
-                    static_cast<const float *>(x), n, heads, channels, buf[7], buf[6], part);
-            bwd_vectors_final<<<ceil_div(2 * fdim, kBwThreads), kBwThreads, 0, s>>>(
-                part, nb, fdim, grad_a_src, grad_a_dst);
-            return cudaGetLastError();
-        }
+    // Whole 16-byte gradient slices in one head each, a power of two of them per
+    // head, and one feature tile per row: softmax_fast's backward or the walk by
+    // target, then the walk by source.
+    const int hl4 = channels / 4;
+    if (aligned && channels % 4 == 0 && (hl4 & (hl4 - 1)) == 0 && f <= 128) {
+        GatArgs ga{rowptr, col, x, n, heads, channels, slope, buf[0], buf[1], nullptr, nullptr, out,
+                   grad_out, reinterpret_cast<float4 *>(buf[2]), buf[6], buf[7], grad_x, a_src, a_dst};
+        const bool bf16 = x_dtype == TFG_BF16;
+        if (launch_softmax_fast_bwd(ga, x_dtype, e, s)) err = cudaGetLastError();
+        else if (bf16) err = channels % 8 == 0 ? walk_targets<uint16_t, 8>(ga, s) : walk_targets<uint16_t, 4>(ga, s);
+        else err = walk_targets<float, 4>(ga, s);
+        if (err != cudaSuccess) return err;
+        ga.rowptr = rowptr_src;
+        ga.col = col_src;
+        err = bf16 ? walk_sources<uint16_t>(ga, s) : walk_sources<float>(ga, s);
+        if (err != cudaSuccess) return err;
+        if (bf16)
+            return launch_vectors(static_cast<const uint16_t *>(x), n, heads, channels, buf[7], buf[6],
+                                  bw_blocks(n), part, grad_a_src, grad_a_dst, s);
+        return launch_vectors(static_cast<const float *>(x), n, heads, channels, buf[7], buf[6],
+                              bw_blocks(n), part, grad_a_src, grad_a_dst, s);
     }
     BwArgs a{rowptr, col, rowptr_src, col_src, x, n, heads, channels, slope, a_src, a_dst,
              out, grad_out, buf[0], buf[1], buf[2], buf[3], buf[4], buf[5], buf[6], grad_x};

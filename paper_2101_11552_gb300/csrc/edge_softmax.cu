@@ -8,16 +8,14 @@
 //   aggregate    out[t,h,:] = sum over row t of alpha * x[src,h,:]
 //
 // The paper's workflow runs map, reduce and map as separate passes over the
-// edges.  Here one warp owns a target row and makes a single pass with the
-// running-maximum form of the softmax: when an edge raises the row maximum m
-// of a head, the running denominator and weighted sum are rescaled by
-// exp(m_old - m_new), which leaves alpha and out mathematically unchanged.
-// A row is split among G = 32 / LPR lane groups (each group covers LPR * VEC
-// features and takes every G-th edge); the groups' (m, den, acc) triples are
-// merged by a butterfly at the end.  Sums are blocked per 32-edge chunk to
-// keep fp32 chains short.  Every lane of a head evaluates the same logits in
-// the same order, so the lanes agree and results are deterministic.  With
-// alpha requested, a second pass over the row writes the normalised weights.
+// edges.  Here a row is read in a single pass with the running-maximum form of
+// the softmax: when an edge raises the row maximum m of a head, the running
+// denominator and weighted sum are rescaled by exp(m_old - m_new), which leaves
+// alpha and out mathematically unchanged.  Two forms: softmax_fast (this file)
+// on graphs of long rows whose layout it takes, the row walk of gat_walk.cuh
+// otherwise.  Sums are blocked per 32 edges to keep fp32 chains short, in a
+// fixed order (deterministic).  With alpha requested, a second pass over a row
+// writes its normalised weights.
 //
 // Logits are kept in base-2 units: the node scores are multiplied by log2(e)
 // once, and since LeakyReLU(c v) = c LeakyReLU(v) for c > 0 every logit,
@@ -32,6 +30,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "gat_walk.cuh"
 
 namespace tfg {
 namespace {
@@ -40,7 +39,7 @@ constexpr int kSmThreads = 256;
 #ifndef TFG_SM_UNROLL
 #define TFG_SM_UNROLL 4   // gathers in flight per lane (tuning knob)
 #endif
-constexpr int kSmUnroll = TFG_SM_UNROLL;   // fast kernel
+constexpr int kSmUnroll = TFG_SM_UNROLL;
 // 1: the next chunk's column ids are requested one chunk ahead; 2: also its
 // node scores s_src, gathered while this chunk's rows are summed (measured on
 // the 114.6M-edge graph: 2.29 ms with 2, 2.40-2.50 ms with 1, 2.44-2.57 ms with 0)
@@ -51,7 +50,6 @@ constexpr int kSmUnroll = TFG_SM_UNROLL;   // fast kernel
 #define TFG_SM_FULL_CHUNKS 1   // separate code for full 32-edge chunks (no slot tests)
 #endif
 constexpr bool kSmFullChunks = TFG_SM_FULL_CHUNKS != 0;
-constexpr int kGenUnroll = 4;               // generic kernel
 constexpr float kLog2e = 1.4426950408889634f;   // log2(e): natural-log units -> base-2 units
 
 // Compensated dot product (the "Dot2" scheme of Ogita, Rump and Oishi,
@@ -75,132 +73,37 @@ struct Dot2 {
     __device__ __forceinline__ float value() const { return s + c; }
 };
 
-template <typename XT>
+// One thread per (node, head), VEC channels a load (VEC > 1: channels a multiple
+// of VEC, x, a_src and a_dst 16-byte aligned); the additions run channel by
+// channel whatever VEC is.  Single-channel loads made the kernel LSU-bound:
+// 169,343 nodes x 8 x 16 fp32 55 us against 13 us for its 87 MB.
+template <typename XT, int VEC>
 __global__ void node_scores(const XT *__restrict__ x, int64_t n, int heads, int channels,
                             const float *__restrict__ a_src, const float *__restrict__ a_dst,
                             float *__restrict__ s_src, float *__restrict__ s_dst) {
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= n * heads) return;
-    const int64_t v = i / heads;
     const int h = static_cast<int>(i % heads);
-    const XT *xr = x + v * heads * channels + static_cast<int64_t>(h) * channels;
+    const XT *xr = x + i * channels;
     const float *as = a_src + h * channels, *ad = a_dst + h * channels;
     Dot2 a, b;
-    for (int c = 0; c < channels; ++c) {
-        float xv[1];
-        VecLoad<XT, 1>::load(xr + c, xv);
-        a.add(xv[0], __ldg(as + c));
-        b.add(xv[0], __ldg(ad + c));
+#pragma unroll 2
+    for (int c = 0; c < channels; c += VEC) {
+        float xv[VEC], av[VEC], bv[VEC];
+        VecLoad<XT, VEC>::load(xr + c, xv);
+        gw_load(as + c, av);
+        gw_load(ad + c, bv);
+#pragma unroll
+        for (int q = 0; q < VEC; ++q) {
+            a.add(xv[q], av[q]);
+            b.add(xv[q], bv[q]);
+        }
     }
     s_src[i] = a.value() * kLog2e;
     s_dst[i] = b.value() * kLog2e;
 }
 
 __device__ __forceinline__ float leaky(float v, float slope) { return v > 0.f ? v : slope * v; }
-
-// 2^(m_old - m_new) for base-2 maxima, with 2^(-inf - anything) = 0 (an
-// empty group has m = -inf).
-__device__ __forceinline__ float rescale(float m_old, float m_new) {
-    return m_old == -CUDART_INF_F ? 0.f : exp2f(m_old - m_new);
-}
-
-template <typename XT, int VEC, int LPR>
-__device__ __forceinline__ void generic_row(const int32_t *__restrict__ rowptr,
-                                            const int32_t *__restrict__ col,
-                                            const XT *__restrict__ x, int heads, int channels,
-                                            float slope, const float *__restrict__ s_src,
-                                            const float *__restrict__ s_dst,
-                                            float *__restrict__ out, float *__restrict__ alpha,
-                                            int64_t t, int lane) {
-    using V = VecLoad<XT, VEC>;
-    constexpr int G = 32 / LPR;
-    const int g = lane / LPR, sub = lane % LPR;
-    const int64_t f = static_cast<int64_t>(heads) * channels;
-    const int64_t beg = rowptr[t], end = col ? rowptr[t + 1] : rowptr[t];
-    for (int64_t ft = 0; ft < f; ft += LPR * VEC) {
-        const int64_t f0 = ft + sub * VEC;
-        const bool fok = f0 < f;
-        const int h = fok ? static_cast<int>(f0 / channels) : 0;
-        const float sd = __ldg(s_dst + t * heads + h);
-
-        float m = -CUDART_INF_F, den = 0.f;
-        float acc[VEC];
-#pragma unroll
-        for (int q = 0; q < VEC; ++q) acc[q] = 0.f;
-        for (int64_t base = beg; base < end; base += 32) {
-            const int cnt = static_cast<int>(min64(32, end - base));
-            const int c = lane < cnt ? ld_stream(col + base + lane) : 0;
-            float den_part = 0.f, part[VEC];
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) part[q] = 0.f;
-            for (int j = 0; j < cnt; j += G * kGenUnroll) {
-                float l[kGenUnroll];
-                typename V::Raw raw[kGenUnroll];
-#pragma unroll
-                for (int u = 0; u < kGenUnroll; ++u) {
-                    const int k = j + u * G + g;
-                    const int src = __shfl_sync(kFull, c, k & 31);
-                    const bool ok = k < cnt;
-                    l[u] = ok ? leaky(__ldg(s_src + static_cast<int64_t>(src) * heads + h) + sd, slope)
-                              : -CUDART_INF_F;
-                    raw[u] = (ok && fok) ? V::raw(x + static_cast<int64_t>(src) * f + f0) : V::zero();
-                }
-#pragma unroll
-                for (int u = 0; u < kGenUnroll; ++u) {
-                    if (l[u] == -CUDART_INF_F) continue;   // empty slot
-                    if (l[u] > m) {                        // new running maximum
-                        const float sc = rescale(m, l[u]);
-                        den *= sc;
-                        den_part *= sc;
-#pragma unroll
-                        for (int q = 0; q < VEC; ++q) {
-                            acc[q] *= sc;
-                            part[q] *= sc;
-                        }
-                        m = l[u];
-                    }
-                    const float p = exp2f(l[u] - m);
-                    den_part += p;
-                    float v[VEC];
-                    V::widen(raw[u], v);
-#pragma unroll
-                    for (int q = 0; q < VEC; ++q) part[q] = fmaf(p, v[q], part[q]);
-                }
-            }
-            den += den_part;
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) acc[q] += part[q];
-        }
-        // merge the G groups: (m, den, acc) in a fixed butterfly order
-#pragma unroll
-        for (int s = LPR; s < 32; s <<= 1) {
-            const float mo = __shfl_xor_sync(kFull, m, s);
-            const float dn = __shfl_xor_sync(kFull, den, s);
-            const float mm = fmaxf(m, mo);
-            const float a = rescale(m, mm), b = rescale(mo, mm);
-            den = den * a + dn * b;
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) {
-                const float ao = __shfl_xor_sync(kFull, acc[q], s);
-                acc[q] = acc[q] * a + ao * b;
-            }
-            m = mm;
-        }
-        if (lane < LPR && fok) {
-            float *o = out + t * f + f0;
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) o[q] = end > beg ? acc[q] / den : 0.f;
-        }
-        // normalised attention weights, one writer per (edge, head)
-        if (alpha && lane < LPR && fok && (f0 % channels) == 0) {
-            for (int64_t k = beg; k < end; ++k) {
-                const int src = __ldg(col + k);
-                const float l = leaky(__ldg(s_src + static_cast<int64_t>(src) * heads + h) + sd, slope);
-                alpha[k * heads + h] = exp2f(l - m) / den;
-            }
-        }
-    }
-}
 
 // Fast form for the common layout: H divides 32, every lane's VEC features
 // lie in one head, and one feature tile covers the row (F <= LPR * VEC).
@@ -214,13 +117,21 @@ __device__ __forceinline__ void generic_row(const int32_t *__restrict__ rowptr,
 //  * feature lanes: group g = lane / LPR gathers every G-th edge, fetches the
 //    p of its (edge, head) from the score lane holding it with one shuffle,
 //    and accumulates p * x into fp32 per-chunk partials.
-template <typename XT, int VEC, int LPR, int H>
+//
+// BWD: the backward by target, as in GatByTarget: the rows are weighted with
+// p times the LeakyReLU's slope at the edge, whose sum the score lanes keep in
+// ph; out is then the forward's output, and grad_out, stats and ds_dst are set
+// (114.6M edges, 8 x 16 bf16: 2.66 ms against 3.46 ms for a pass that finished
+// <grad_out[t], x[src]> per edge with a butterfly).
+template <typename XT, int VEC, int LPR, int H, bool BWD>
 __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
                                          const int32_t *__restrict__ col,
                                          const XT *__restrict__ x, int channels, float slope,
                                          const float *__restrict__ s_src,
                                          const float *__restrict__ s_dst, float *__restrict__ out,
-                                         float *__restrict__ alpha, int64_t t, int lane) {
+                                         float *__restrict__ alpha, const float *__restrict__ grad_out,
+                                         float4 *__restrict__ stats, float *__restrict__ ds_dst,
+                                         int64_t t, int lane) {
     using V = VecLoad<XT, VEC>;
     constexpr int G = 32 / LPR;     // edges per feature step
     constexpr int ES = 32 / H;      // edges per score step
@@ -249,7 +160,7 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
     // chunk's logits, the running maximum m of each head absorbs the chunk's
     // maximum (earlier sums are rescaled by exp(m_old - m_new) when it rises),
     // then p = exp(l - m) weights the chunk's gathered rows
-    float m = -CUDART_INF_F, den = 0.f, acc[VEC];
+    float m = -CUDART_INF_F, den = 0.f, ph = 0.f, acc[VEC];
 #pragma unroll
     for (int q = 0; q < VEC; ++q) acc[q] = 0.f;
 #if TFG_SM_PREFETCH
@@ -287,19 +198,25 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
         if (__any_sync(kFull, rises)) {   // warp-uniform; rare after the first chunks
             const float sc = rises ? (m == -CUDART_INF_F ? 0.f : exp2f(m - cm)) : 1.f;
             den *= sc;
+            if (BWD) ph *= sc;
             const float fsc = __shfl_sync(kFull, sc, fh);   // lane fh scores head fh
 #pragma unroll
             for (int q = 0; q < VEC; ++q) acc[q] *= fsc;
             m = fmaxf(m, cm);
         }
-        float den_part = 0.f;
+        float den_part = 0.f, ph_part = 0.f;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int k = r * ES + se;
             p[r] = (FULL || k < cnt) ? exp2f(p[r] - m) : 0.f;
             den_part += p[r];
+            if (BWD) {
+                p[r] = sv[r] + sd > 0.f ? p[r] : slope * p[r];
+                ph_part += p[r];
+            }
         }
         den += den_part;
+        if (BWD) ph += ph_part;
 #if TFG_SM_PREFETCH >= 2
         // the next chunk's node scores, requested before this chunk's rows
 #pragma unroll
@@ -372,6 +289,31 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
 #pragma unroll
         for (int q = 0; q < VEC; ++q) acc[q] += __shfl_xor_sync(kFull, acc[q], o);
     const float dh = __shfl_sync(kFull, den, fh);   // lane fh holds head fh's denominator
+    if constexpr (BWD) {
+#pragma unroll
+        for (int o = H; o < 32; o <<= 1) ph += __shfl_xor_sync(kFull, ph, o);
+        const float phh = __shfl_sync(kFull, ph, fh), mh = __shfl_sync(kFull, m, fh), sdh = __shfl_sync(kFull, sd, fh);
+        float b = 0.f, d = 0.f;
+        if (fok) {
+            float gv[VEC], ov[VEC];
+            gw_load(grad_out + t * f + f0, gv);
+            gw_load(out + t * f + f0, ov);
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) {
+                b = fmaf(gv[q], ov[q], b);
+                d = fmaf(gv[q], acc[q], d);
+            }
+        }
+        for (int o = 1; o < channels / VEC; o <<= 1) {
+            b += __shfl_xor_sync(kFull, b, o);
+            d += __shfl_xor_sync(kFull, d, o);
+        }
+        if (lane < LPR && fok && f0 % channels == 0) {
+            ds_dst[t * H + fh] = end > beg ? (d - b * phh) / dh : 0.f;
+            stats[t * H + fh] = make_float4(sdh, mh, end > beg ? 1.f / dh : 0.f, b);
+        }
+        return;
+    }
     if (lane < LPR && fok) {
         float *o = out + t * f + f0;
 #pragma unroll
@@ -394,305 +336,13 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
     }
 }
 
-// ---------------------------------------------------------------------------
-// Merge-path form of the fast kernel (same layout conditions).  The work is
-// split as in aggregate_mp_kernel: whole rows per CTA, an equal number of
-// edges + row ends per warp inside it, so a hub row is shared by the warps it
-// spans; the next chunk's column ids are loaded before this chunk is
-// gathered.  A warp's part of a row is the running state (m, den, acc) of
-// fast_row; the owner of a row begun by earlier warps merges their parts and
-// its own in warp order after the CTA's one barrier:
-//   m = max(m1, m2),  den = den1 2^(m1 - m) + den2 2^(m2 - m),  acc likewise.
-// ---------------------------------------------------------------------------
-#ifndef TFG_SM_MP
-#define TFG_SM_MP 1          // 0: the fast layout takes softmax_fast (side-by-side timing)
-#endif
-#ifndef TFG_SMP_BLOCKS
-#define TFG_SMP_BLOCKS 3     // resident CTAs per SM
-#endif
-constexpr int kSmpBlocks = TFG_SMP_BLOCKS;
-// Measured: on the 169,343-node graph (mean in-degree 6.9) the merge-path form
-// takes 0.24 ms against 0.26 ms; on the 114.6M-edge graph (mean 492) 3.15 ms
-// against 2.62 ms for softmax_fast, whose per-row work is already balanced
-// by its long rows.  Graphs with a mean in-degree below this take it.
-constexpr int64_t kSmpMaxDegree = 32;
-constexpr int kSmWarps = kSmThreads / 32;
-
-// (M, D, A) absorbs another part (m2, d2, a2) of the same row and head.
-template <int VEC>
-__device__ __forceinline__ void merge_state(float &M, float &D, float (&A)[VEC], float m2,
-                                            float d2, const float *a2) {
-    const float mn = fmaxf(M, m2);
-    const float sa = M == -CUDART_INF_F ? 0.f : exp2f(M - mn);
-    const float sb = m2 == -CUDART_INF_F ? 0.f : exp2f(m2 - mn);
-    D = D * sa + d2 * sb;
-#pragma unroll
-    for (int q = 0; q < VEC; ++q) A[q] = A[q] * sa + (a2 ? a2[q] * sb : 0.f);
-    M = mn;
-}
-
-template <typename XT, int VEC, int LPR, int H>
-struct SmMp {
-    using V = VecLoad<XT, VEC>;
-    static constexpr int G = 32 / LPR;     // edges per feature step
-    static constexpr int ES = 32 / H;      // edges per score step
-    static constexpr int R = 32 / ES;      // score steps per 32-edge chunk (= H)
-    static constexpr int kF = LPR * VEC;
-    static_assert(ES % G == 0, "score step must hold whole feature steps");
-    static_assert(G * kSmUnroll <= 32 && 32 % (G * kSmUnroll) == 0,
-                  "steps of G * kSmUnroll slots must tile the 32-edge chunk");
-
-    // One chunk of up to 32 edges of one row (ids in c, lane j holds edge j):
-    // the logits of the chunk (score lanes), the running maximum, then the
-    // weighted rows (feature lanes), exactly as in fast_row.
-    static __device__ __forceinline__ void chunk(const XT *xf, uint32_t fs,
-                                                 const float *__restrict__ s_src, float sd,
-                                                 float slope, int c, int cnt, int lane, int fh,
-                                                 float &m, float &den, float (&acc)[VEC]) {
-        const int se = lane / H, sh = lane % H, g = lane / LPR;
-        typename V::Raw raw0[kSmUnroll];
-#pragma unroll
-        for (int u = 0; u < kSmUnroll; ++u) {
-            const uint32_t src = static_cast<uint32_t>(__shfl_sync(kFull, c, u * G + g));
-            raw0[u] = V::raw(xf + static_cast<uint64_t>(src) * fs);
-        }
-        float p[R];
-        float cm = -CUDART_INF_F;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int k = r * ES + se;
-            const uint32_t src = static_cast<uint32_t>(__shfl_sync(kFull, c, k));
-            p[r] = k < cnt ? leaky(__ldg(s_src + static_cast<uint64_t>(src) * H + sh) + sd, slope)
-                           : -CUDART_INF_F;
-            cm = fmaxf(cm, p[r]);
-        }
-#pragma unroll
-        for (int o = H; o < 32; o <<= 1) cm = fmaxf(cm, __shfl_xor_sync(kFull, cm, o));
-        const bool rises = cm > m;
-        if (__any_sync(kFull, rises)) {   // warp-uniform; rare after the first chunks
-            const float sc = rises ? (m == -CUDART_INF_F ? 0.f : exp2f(m - cm)) : 1.f;
-            den *= sc;
-            const float fsc = __shfl_sync(kFull, sc, fh);   // lane fh scores head fh
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) acc[q] *= fsc;
-            m = fmaxf(m, cm);
-        }
-        float den_part = 0.f;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int k = r * ES + se;
-            p[r] = k < cnt ? exp2f(p[r] - m) : 0.f;
-            den_part += p[r];
-        }
-        den += den_part;
-        float part[VEC];
-#pragma unroll
-        for (int q = 0; q < VEC; ++q) part[q] = 0.f;
-#pragma unroll
-        for (int e = 0; e < 32; e += G * kSmUnroll) {
-            if (e >= cnt) break;   // warp-uniform
-            typename V::Raw raw[kSmUnroll];
-            float pw[kSmUnroll];
-#pragma unroll
-            for (int u = 0; u < kSmUnroll; ++u) {
-                const int k0 = e + u * G;              // edge of group 0 in this step
-                // p of (edge k0 + g, head fh) sits in lane ((k0 + g) % ES) * H + fh, register k0 / ES
-                pw[u] = __shfl_sync(kFull, p[k0 / ES], ((k0 % ES) + g) * H + fh);
-                if (e == 0) {
-                    raw[u] = raw0[u];
-                } else {
-                    const uint32_t src = static_cast<uint32_t>(__shfl_sync(kFull, c, k0 + g));
-                    raw[u] = V::raw(xf + static_cast<uint64_t>(src) * fs);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kSmUnroll; ++u) {
-                float v[VEC];
-                V::widen(raw[u], v);
-                if constexpr (VEC % 2 == 0) {
-                    const float2 w2 = make_float2(pw[u], pw[u]);
-#pragma unroll
-                    for (int q = 0; q < VEC; q += 2) {
-                        const float2 r2 = fma2(make_float2(v[q], v[q + 1]), w2,
-                                               make_float2(part[q], part[q + 1]));
-                        part[q] = r2.x;
-                        part[q + 1] = r2.y;
-                    }
-                } else {
-#pragma unroll
-                    for (int q = 0; q < VEC; ++q) part[q] = fmaf(pw[u], v[q], part[q]);
-                }
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < VEC; ++q) acc[q] += part[q];
-    }
-
-    // Normalised weights of every edge of row t, given the row's final
-    // maximum M and denominator D of this lane's score head.
-    static __device__ void write_alpha(const int32_t *__restrict__ rowptr,
-                                       const int32_t *__restrict__ col,
-                                       const float *__restrict__ s_src, float sd, float slope,
-                                       float M, float D, float *__restrict__ alpha, int32_t t,
-                                       int lane) {
-        const int se = lane / H, sh = lane % H;
-        const int32_t beg = __ldg(rowptr + t), end = __ldg(rowptr + t + 1);
-        for (int32_t base = beg; base < end; base += 32) {
-            const int cnt = min(32, end - base);
-            const int c = lane < cnt ? __ldg(col + base + lane) : 0;
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int k = r * ES + se;
-                const uint32_t src = static_cast<uint32_t>(__shfl_sync(kFull, c, k));
-                if (k < cnt) {
-                    const float l = leaky(__ldg(s_src + static_cast<uint64_t>(src) * H + sh) + sd, slope);
-                    alpha[(static_cast<int64_t>(base) + k) * H + sh] = exp2f(l - M) / D;
-                }
-            }
-        }
-    }
-};
-
-template <typename XT, int VEC, int LPR, int H>
-__global__ void __launch_bounds__(kSmThreads, kSmpBlocks)
-softmax_mp(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col,
-           const XT *__restrict__ x, int64_t n, int channels, float slope,
-           const float *__restrict__ s_src, const float *__restrict__ s_dst,
-           float *__restrict__ out, float *__restrict__ alpha) {
-    using S = SmMp<XT, VEC, LPR, H>;
-    constexpr int kF = S::kF;
-    __shared__ float s_tacc[kSmWarps][kF], s_hacc[kSmWarps][kF];
-    __shared__ float s_tm[kSmWarps][H], s_tden[kSmWarps][H], s_hm[kSmWarps][H], s_hden[kSmWarps][H];
-    __shared__ int32_t s_tail_row[kSmWarps], s_head_row[kSmWarps];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int sh = lane % H, sub = lane % LPR;
-    const int f = H * channels;
-    const int f0 = sub * VEC;
-    const bool fok = f0 < f;
-    const int fh = fok ? f0 / channels : 0;
-    const XT *xf = x + (fok ? f0 : 0);
-    const uint32_t fs = static_cast<uint32_t>(f);
-
-    // node ids and edge positions fit int32 (the ABI caps N and E below 2^31)
-    int64_t r0l, r1l;
-    balanced_rows(rowptr, n, gridDim.x, blockIdx.x, r0l, r1l);
-    const int32_t r0 = static_cast<int32_t>(r0l), r1 = static_cast<int32_t>(r1l);
-    const int64_t q0 = static_cast<int64_t>(__ldg(rowptr + r0)) + r0;
-    const int64_t q1 = static_cast<int64_t>(__ldg(rowptr + r1)) + r1;
-    const int64_t per = (q1 - q0 + kSmWarps - 1) / kSmWarps;
-    const int64_t qa = min64(q1, q0 + warp * per), qb = min64(q1, qa + per);
-    const int32_t ta = last_row_at(rowptr, r0, r1, qa);
-    const int32_t tb = last_row_at(rowptr, ta, r1, qb);
-    const int32_t ka = static_cast<int32_t>(qa - ta), kb = static_cast<int32_t>(qb - tb);
-    const bool head_split = ka > __ldg(rowptr + ta);   // row ta begun by an earlier warp
-    if (lane == 0) s_head_row[warp] = -1;
-
-    float m = -CUDART_INF_F, den = 0.f, acc[VEC];
-#pragma unroll
-    for (int q = 0; q < VEC; ++q) acc[q] = 0.f;
-    int32_t t = ta, k = ka;                            // this warp's edges are [ka, kb)
-    int32_t rend = t < tb ? __ldg(rowptr + t + 1) : kb;
-    float sd = t < n ? __ldg(s_dst + static_cast<int64_t>(t) * H + sh) : 0.f;
-    int cnext = (col && k + lane < kb) ? __ldg(col + k + lane) : 0;
-    for (;;) {
-        while (k >= rend) {                            // row t has no edges left here
-            if (t >= tb) break;
-#pragma unroll
-            for (int o = H; o < 32; o <<= 1) den += __shfl_xor_sync(kFull, den, o);
-#pragma unroll
-            for (int o = LPR; o < 32; o <<= 1)
-#pragma unroll
-                for (int q = 0; q < VEC; ++q) acc[q] += __shfl_xor_sync(kFull, acc[q], o);
-            if (t == ta && head_split) {               // parts of it sit with earlier warps
-                if (lane < H) {
-                    s_hm[warp][lane] = m;
-                    s_hden[warp][lane] = den;
-                }
-                if (lane < LPR) {
-#pragma unroll
-                    for (int q = 0; q < VEC; ++q) s_hacc[warp][f0 + q] = acc[q];
-                }
-                if (lane == 0) s_head_row[warp] = t;
-            } else {
-                const float dh = __shfl_sync(kFull, den, fh);   // lane fh: head fh's denominator
-                const bool any = __ldg(rowptr + t + 1) > __ldg(rowptr + t);
-                if (lane < LPR && fok) {
-                    float *o = out + static_cast<int64_t>(t) * f + f0;
-#pragma unroll
-                    for (int q = 0; q < VEC; ++q) o[q] = any ? acc[q] / dh : 0.f;
-                }
-                if (alpha && any) S::write_alpha(rowptr, col, s_src, sd, slope, m, den, alpha, t, lane);
-            }
-            m = -CUDART_INF_F;
-            den = 0.f;
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) acc[q] = 0.f;
-            ++t;
-            rend = t < tb ? __ldg(rowptr + t + 1) : kb;
-            sd = t < n ? __ldg(s_dst + static_cast<int64_t>(t) * H + sh) : 0.f;
-        }
-        if (k >= rend) break;                          // t == tb and its edges are done
-        const int cnt = min(32, rend - k);
-        const int c = cnext;
-        const int32_t kn = k + cnt;                    // the next chunk starts here
-        cnext = (kn + lane < kb) ? __ldg(col + kn + lane) : 0;
-        S::chunk(xf, fs, s_src, sd, slope, c, cnt, lane, fh, m, den, acc);
-        k = kn;
-    }
-    // this warp's part of row tb (empty when the range ends on a row end)
-#pragma unroll
-    for (int o = H; o < 32; o <<= 1) den += __shfl_xor_sync(kFull, den, o);
-#pragma unroll
-    for (int o = LPR; o < 32; o <<= 1)
-#pragma unroll
-        for (int q = 0; q < VEC; ++q) acc[q] += __shfl_xor_sync(kFull, acc[q], o);
-    if (lane < H) {
-        s_tm[warp][lane] = m;
-        s_tden[warp][lane] = den;
-    }
-    if (lane < LPR) {
-#pragma unroll
-        for (int q = 0; q < VEC; ++q) s_tacc[warp][f0 + q] = acc[q];
-    }
-    if (lane == 0) s_tail_row[warp] = tb;
-    __syncthreads();
-    const int32_t hr = s_head_row[warp];
-    if (hr < 0) return;
-    // earlier warps' parts in warp order, then ours: (Ms, Ds) for the score
-    // head sh, (Mf, Df, A) for the feature head fh
-    float Ms = -CUDART_INF_F, Ds = 0.f, Mf = -CUDART_INF_F, Df = 0.f, A[VEC];
-    float none[1] = {0.f};
-#pragma unroll
-    for (int q = 0; q < VEC; ++q) A[q] = 0.f;
-    for (int w = 0; w < warp; ++w) {
-        if (s_tail_row[w] != hr) continue;
-        merge_state<1>(Ms, Ds, none, s_tm[w][sh], s_tden[w][sh], nullptr);
-        merge_state<VEC>(Mf, Df, A, s_tm[w][fh], s_tden[w][fh], &s_tacc[w][fok ? f0 : 0]);
-    }
-    merge_state<1>(Ms, Ds, none, s_hm[warp][sh], s_hden[warp][sh], nullptr);
-    merge_state<VEC>(Mf, Df, A, s_hm[warp][fh], s_hden[warp][fh], &s_hacc[warp][fok ? f0 : 0]);
-    if (lane < LPR && fok) {
-        float *o = out + static_cast<int64_t>(hr) * f + f0;
-#pragma unroll
-        for (int q = 0; q < VEC; ++q) o[q] = A[q] / Df;   // a split row has edges
-    }
-    if (alpha) {
-        const float sdr = __ldg(s_dst + static_cast<int64_t>(hr) * H + sh);
-        S::write_alpha(rowptr, col, s_src, sdr, slope, Ms, Ds, alpha, hr, lane);
-    }
-}
-
-template <typename XT, int VEC, int LPR>
-__global__ void __launch_bounds__(kSmThreads, 3)
-softmax_aggregate(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col,
-                  const XT *__restrict__ x, int64_t n, int heads, int channels, float slope,
-                  const float *__restrict__ s_src, const float *__restrict__ s_dst,
-                  float *__restrict__ out, float *__restrict__ alpha) {
-    for_each_row(rowptr, n, [&](int64_t t, int lane) {
-        generic_row<XT, VEC, LPR>(rowptr, col, x, heads, channels, slope, s_src, s_dst, out,
-                                  alpha, t, lane);
-    });
-}
+// Graphs of a mean in-degree below this take the row walk (gat_walk.cuh), whose
+// warps share hub rows and whose windows cross row ends; longer rows take
+// softmax_fast, whose score lanes evaluate each (edge, head) once.  Measured:
+// 169,343 nodes, mean in-degree 6.9, 8 x 16 fp32: walk 145 us, softmax_fast's
+// earlier merge-path form 164 us; 114.6M edges, mean 492, bf16: walk 2.64-2.68
+// ms, softmax_fast 2.20 ms.
+constexpr int64_t kWalkMaxDegree = 32;
 
 // Measured on the 114.6M-edge graph (bf16, 8 heads x 16), ids and scores
 // requested one chunk ahead: 3 CTAs per SM with 4 gathers in flight per lane
@@ -709,8 +359,21 @@ softmax_fast(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col
              const float *__restrict__ s_src, const float *__restrict__ s_dst,
              float *__restrict__ out, float *__restrict__ alpha) {
     for_each_row(rowptr, n, [&](int64_t t, int lane) {
-        fast_row<XT, VEC, LPR, H>(rowptr, col, x, channels, slope, s_src, s_dst, out, alpha, t,
-                                  lane);
+        fast_row<XT, VEC, LPR, H, false>(rowptr, col, x, channels, slope, s_src, s_dst, out, alpha, nullptr,
+                                         nullptr, nullptr, t, lane);
+    });
+}
+
+template <typename XT, int VEC, int LPR, int H>
+__global__ void __launch_bounds__(kSmThreads, TFG_SMF_BLOCKS)
+softmax_fast_bwd(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col,
+                 const XT *__restrict__ x, int64_t n, int channels, float slope,
+                 const float *__restrict__ s_src, const float *__restrict__ s_dst,
+                 float *__restrict__ out, const float *__restrict__ grad_out, float4 *__restrict__ stats,
+                 float *__restrict__ ds_dst) {
+    for_each_row(rowptr, n, [&](int64_t t, int lane) {
+        fast_row<XT, VEC, LPR, H, true>(rowptr, col, x, channels, slope, s_src, s_dst, out, nullptr, grad_out,
+                                        stats, ds_dst, t, lane);
     });
 }
 
@@ -718,24 +381,23 @@ constexpr int64_t kSmMinWork = 2048;   // edges + rows per CTA, at least
 
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
-// Launch the fast form when the layout allows it; false means "use the generic one".
+// Launch softmax_fast (or its backward) when the layout allows it; false means
+// "take the walk".
 template <typename XT, int VEC, int LPR>
-bool launch_fast_lpr(const int32_t *rowptr, const int32_t *col, const void *x, int64_t n, int64_t e,
-                     int heads, int channels, float slope, const float *s_src, const float *s_dst,
-                     float *out, float *alpha, cudaStream_t s) {
+bool launch_fast_lpr(const GatArgs &a, int64_t e, bool bwd, cudaStream_t s) {
     constexpr int G = 32 / LPR;
-    const int grid = balanced_grid(n, e, kSmMinWork);
-    const XT *xp = static_cast<const XT *>(x);
-    const int mp_grid = static_cast<int>(min64(n, static_cast<int64_t>(sm_count()) * kSmpBlocks));
+    const int grid = balanced_grid(a.n, e, kSmMinWork);
+    const XT *xp = static_cast<const XT *>(a.x);
 #define TFG_FAST(HH)                                                                              \
-    if (heads == HH) {                                                                            \
+    if (a.heads == HH) {                                                                          \
         if constexpr ((32 / HH) % G == 0) {                                                       \
-            if (TFG_SM_MP && e < kSmpMaxDegree * n)                                              \
-                softmax_mp<XT, VEC, LPR, HH><<<mp_grid, kSmThreads, 0, s>>>(                      \
-                    rowptr, col, xp, n, channels, slope, s_src, s_dst, out, alpha);               \
+            if (bwd)                                                                              \
+                softmax_fast_bwd<XT, VEC, LPR, HH><<<grid, kSmThreads, 0, s>>>(                   \
+                    a.rowptr, a.col, xp, a.n, a.channels, a.slope, a.s_src, a.s_dst,              \
+                    const_cast<float *>(a.fwd_out), a.grad_out, a.stats, a.ds_dst);               \
             else                                                                                  \
                 softmax_fast<XT, VEC, LPR, HH><<<grid, kSmThreads, 0, s>>>(                       \
-                    rowptr, col, xp, n, channels, slope, s_src, s_dst, out, alpha);               \
+                    a.rowptr, a.col, xp, a.n, a.channels, a.slope, a.s_src, a.s_dst, a.out, a.alpha); \
             return true;                                                                          \
         }                                                                                         \
         return false;                                                                             \
@@ -750,33 +412,14 @@ bool launch_fast_lpr(const int32_t *rowptr, const int32_t *col, const void *x, i
 }
 
 template <typename XT, int VEC>
-bool launch_fast(const int32_t *rowptr, const int32_t *col, const void *x, int64_t n, int64_t e,
-                 int heads, int channels, float slope, const float *s_src, const float *s_dst,
-                 float *out, float *alpha, cudaStream_t s) {
-    const int64_t f = static_cast<int64_t>(heads) * channels;
-    if (channels % VEC != 0 || f > 32 * VEC) return false;
+bool launch_fast(const GatArgs &a, int64_t e, bool bwd, cudaStream_t s) {
+    const int64_t f = static_cast<int64_t>(a.heads) * a.channels;
+    if (a.channels % VEC != 0 || f > 32 * VEC || e < kWalkMaxDegree * a.n) return false;
+    if (bwd && a.heads > 8) return false;   // 16 score steps a chunk and the backward's sums spill
     const int64_t chunks = f / VEC;
-    if (chunks > 16) return launch_fast_lpr<XT, VEC, 32>(rowptr, col, x, n, e, heads, channels, slope, s_src, s_dst, out, alpha, s);
-    if (chunks > 8) return launch_fast_lpr<XT, VEC, 16>(rowptr, col, x, n, e, heads, channels, slope, s_src, s_dst, out, alpha, s);
-    return launch_fast_lpr<XT, VEC, 8>(rowptr, col, x, n, e, heads, channels, slope, s_src, s_dst, out, alpha, s);
-}
-
-template <typename XT, int VEC>
-void launch_main(const int32_t *rowptr, const int32_t *col, const void *x, int64_t n, int64_t e,
-                 int heads, int channels, float slope, const float *s_src, const float *s_dst,
-                 float *out, float *alpha, cudaStream_t s) {
-    const int64_t chunks = static_cast<int64_t>(heads) * channels / VEC;
-    const int grid = balanced_grid(n, e, kSmMinWork);
-    const XT *xp = static_cast<const XT *>(x);
-    if (chunks >= 32)
-        softmax_aggregate<XT, VEC, 32><<<grid, kSmThreads, 0, s>>>(rowptr, col, xp, n, heads, channels,
-                                                                   slope, s_src, s_dst, out, alpha);
-    else if (chunks > 8)
-        softmax_aggregate<XT, VEC, 16><<<grid, kSmThreads, 0, s>>>(rowptr, col, xp, n, heads, channels,
-                                                                   slope, s_src, s_dst, out, alpha);
-    else
-        softmax_aggregate<XT, VEC, 8><<<grid, kSmThreads, 0, s>>>(rowptr, col, xp, n, heads, channels,
-                                                                  slope, s_src, s_dst, out, alpha);
+    if (chunks > 16) return launch_fast_lpr<XT, VEC, 32>(a, e, bwd, s);
+    if (chunks > 8) return launch_fast_lpr<XT, VEC, 16>(a, e, bwd, s);
+    return launch_fast_lpr<XT, VEC, 8>(a, e, bwd, s);
 }
 
 // Scratch of tfg_edge_softmax_aggregate_noalloc: the node scores s_src and
@@ -818,18 +461,58 @@ cudaError_t noalloc_softmax_scratch(void **ptr, size_t *bytes) {
 cudaError_t launch_node_scores(const void *x, int x_dtype, int64_t n, int heads, int channels,
                                const float *a_src, const float *a_dst, float *s_src, float *s_dst,
                                cudaStream_t s) {
-    const int sgrid = ceil_div(n * heads, 256);
-    if (x_dtype == TFG_BF16)
-        node_scores<uint16_t><<<sgrid, 256, 0, s>>>(static_cast<const uint16_t *>(x), n, heads,
-                                                    channels, a_src, a_dst, s_src, s_dst);
+    const int grid = ceil_div(n * heads, 256);
+    const uint16_t *xh = static_cast<const uint16_t *>(x);
+    const float *xf = static_cast<const float *>(x);
+    auto a16 = [](const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
+    const bool aligned = a16(x) && a16(a_src) && a16(a_dst);
+    if (x_dtype == TFG_BF16 && aligned && channels % 8 == 0)
+        node_scores<uint16_t, 8><<<grid, 256, 0, s>>>(xh, n, heads, channels, a_src, a_dst, s_src, s_dst);
+    else if (x_dtype == TFG_BF16)
+        node_scores<uint16_t, 1><<<grid, 256, 0, s>>>(xh, n, heads, channels, a_src, a_dst, s_src, s_dst);
+    else if (aligned && channels % 4 == 0)
+        node_scores<float, 4><<<grid, 256, 0, s>>>(xf, n, heads, channels, a_src, a_dst, s_src, s_dst);
     else
-        node_scores<float><<<sgrid, 256, 0, s>>>(static_cast<const float *>(x), n, heads, channels,
-                                                 a_src, a_dst, s_src, s_dst);
+        node_scores<float, 1><<<grid, 256, 0, s>>>(xf, n, heads, channels, a_src, a_dst, s_src, s_dst);
     return cudaGetLastError();
 }
 
+namespace {
+// 16-byte slices (or 8-byte bf16 ones) that lie in one head: one slice per lane
+template <typename XT, int VEC>
+cudaError_t walk_vec(const GatArgs &a, cudaStream_t s) {
+    const int64_t slices = static_cast<int64_t>(a.heads) * a.channels / VEC;
+    if (slices <= 8) return launch_walk<GatByTarget<XT, VEC, 8, 1, 1, false>>(a, s);
+    if (slices <= 16) return launch_walk<GatByTarget<XT, VEC, 16, 1, 1, false>>(a, s);
+    return launch_walk<GatByTarget<XT, VEC, 32, 1, 1, false>>(a, s);
+}
+template <typename XT, int LPR, int T>
+cudaError_t walk_lanes(const GatArgs &a, cudaStream_t s) {
+    if (T == 1 || a.heads == 1) return launch_walk<GatByTarget<XT, 1, LPR, T, 1, false>>(a, s);
+    return launch_walk<GatByTarget<XT, 1, LPR, T, T, false>>(a, s);
+}
+template <typename XT>
+cudaError_t walk_scalar(const GatArgs &a, cudaStream_t s) {
+    const int64_t f = static_cast<int64_t>(a.heads) * a.channels;
+    if (f <= 8) return walk_lanes<XT, 8, 1>(a, s);
+    if (f <= 16) return walk_lanes<XT, 16, 1>(a, s);
+    if (f <= 32) return walk_lanes<XT, 16, 2>(a, s);
+    if (f <= 48) return walk_lanes<XT, 16, 3>(a, s);
+    const int64_t passes = (f + 127) / 128, per = (f + passes - 1) / passes;
+    if (per <= 64) return walk_lanes<XT, 32, 2>(a, s);
+    if (per <= 96) return walk_lanes<XT, 32, 3>(a, s);
+    return walk_lanes<XT, 32, 4>(a, s);
+}
+}  // namespace
+
 size_t softmax_workspace_bytes(int64_t n, int heads) {
     return 2 * align256(sizeof(float) * size_t(n > 0 ? n : 1) * size_t(heads));
+}
+
+// Softmax statistics and ds_dst of the backward (attention_backward.cu), when
+// softmax_fast takes the layout; false means "take the walk".
+bool launch_softmax_fast_bwd(const GatArgs &a, int x_dtype, int64_t e, cudaStream_t s) {
+    return x_dtype == TFG_BF16 ? launch_fast<uint16_t, 8>(a, e, true, s) : launch_fast<float, 4>(a, e, true, s);
 }
 
 cudaError_t launch_edge_softmax(const int32_t *rowptr, const int32_t *col, const void *x,
@@ -840,29 +523,20 @@ cudaError_t launch_edge_softmax(const int32_t *rowptr, const int32_t *col, const
     float *s_src = static_cast<float *>(ws);
     float *s_dst = reinterpret_cast<float *>(static_cast<char *>(ws) +
                                              align256(sizeof(float) * size_t(n) * size_t(heads)));
-    const int sgrid = ceil_div(n * heads, 256);
+    const cudaError_t err = launch_node_scores(x, x_dtype, n, heads, channels, a_src, a_dst, s_src, s_dst, s);
+    if (err != cudaSuccess) return err;
     const bool aligned = (reinterpret_cast<uintptr_t>(x) % 16 == 0) &&
                          (reinterpret_cast<uintptr_t>(out) % 16 == 0);
+    const GatArgs a{rowptr, col, x, n, heads, channels, slope, s_src, s_dst, out, alpha};
     if (x_dtype == TFG_BF16) {
-        node_scores<uint16_t><<<sgrid, 256, 0, s>>>(static_cast<const uint16_t *>(x), n, heads,
-                                                    channels, a_src, a_dst, s_src, s_dst);
-        if (aligned && channels % 8 == 0) {
-            if (!launch_fast<uint16_t, 8>(rowptr, col, x, n, e, heads, channels, slope, s_src, s_dst, out, alpha, s))
-                launch_main<uint16_t, 8>(rowptr, col, x, n, e, heads, channels, slope, s_src, s_dst, out, alpha, s);
-        } else {
-            launch_main<uint16_t, 1>(rowptr, col, x, n, e, heads, channels, slope, s_src, s_dst, out, alpha, s);
-        }
-    } else {
-        node_scores<float><<<sgrid, 256, 0, s>>>(static_cast<const float *>(x), n, heads, channels,
-                                                 a_src, a_dst, s_src, s_dst);
-        if (aligned && channels % 4 == 0) {
-            if (!launch_fast<float, 4>(rowptr, col, x, n, e, heads, channels, slope, s_src, s_dst, out, alpha, s))
-                launch_main<float, 4>(rowptr, col, x, n, e, heads, channels, slope, s_src, s_dst, out, alpha, s);
-        } else {
-            launch_main<float, 1>(rowptr, col, x, n, e, heads, channels, slope, s_src, s_dst, out, alpha, s);
-        }
+        if (aligned && launch_fast<uint16_t, 8>(a, e, false, s)) return cudaGetLastError();
+        if (aligned && channels % 8 == 0) return walk_vec<uint16_t, 8>(a, s);
+        if (aligned && channels % 4 == 0) return walk_vec<uint16_t, 4>(a, s);
+        return walk_scalar<uint16_t>(a, s);
     }
-    return cudaGetLastError();
+    if (aligned && launch_fast<float, 4>(a, e, false, s)) return cudaGetLastError();
+    if (aligned && channels % 4 == 0) return walk_vec<float, 4>(a, s);
+    return walk_scalar<float>(a, s);
 }
 
 }  // namespace tfg

@@ -1,0 +1,597 @@
+// The three edge passes of the additive (GAT) attention as row-walk policies:
+// forward, backward by target, backward by source.  Lane layout as in the
+// aggregation: LPR lanes cover a row in 16-byte slices (T = 1, a slice lies in one
+// head), or with T single features a lane, feature i * LPR + sub in turn; G = 32 /
+// LPR lane groups take every G-th edge.  Every lane forms the logits of its own
+// heads (NH of them: 1 when all its features share a head), so no weight passes
+// between lanes.  Logits are in base-2 units.
+#pragma once
+#include <math_constants.h>
+
+#include "row_walk.cuh"
+
+namespace tfg {
+
+struct GatArgs {
+    const int32_t *rowptr, *col;         // CSR of the pass
+    const void *x;
+    int64_t n;
+    int heads, channels;
+    float slope;
+    const float *s_src, *s_dst;          // base-2 node scores [N, H]
+    float *out, *alpha;                  // forward
+    const float *fwd_out, *grad_out;     // backward by target
+    float4 *stats;                       // [N, H]: (s_dst, m, 1 / den, beta)
+    float *ds_dst, *ds_src, *grad_x;
+    const float *a_src, *a_dst;          // backward by source
+};
+
+namespace {
+
+// What bounds it: instructions on short rows (169,343 nodes, mean in-degree 6.9, 8
+// x 16 fp32: forward 145, by target 164, by source 161 us, against 36-45 us for
+// the gathered bytes at the L2 rate), the gathers and the weights' arithmetic on
+// long ones (by source at 114.6M edges: 640 bytes an edge, 5.43 ms, 13.5 TB/s;
+// 7.93 ms when each edge's dot product was finished by a butterfly).  One head of
+// 41 channels on the first graph, alpha written: 1,753 us in a row-per-warp
+// kernel whose hub rows one warp walked, 196 us.
+//
+// Tuning knobs.  Warps per CTA (one CTA per SM), measured on the two graphs:
+// by target 28 (forward 146 us / 2.68 ms), 24 160 / 2.84, 32 136 / 2.64; by source
+// 24 161 us / 5.43 ms, 28 168 / 5.50, 20 203 / 5.42.
+#ifndef TFG_GW_WARPS
+#define TFG_GW_WARPS 28
+#endif
+#ifndef TFG_GW_SRC_WARPS
+#define TFG_GW_SRC_WARPS 24
+#endif
+// Gathers in flight per lane: 4 against 2 (forward 147 us / 3.20 ms) and 8 with
+// 16 warps (239 us / 2.99 ms).
+#ifndef TFG_GW_DEPTH
+#define TFG_GW_DEPTH 4
+#endif
+// The same by source, and how many of its steps unroll in a full window (1:
+// 5.53 ms, 2: 6.12, 8: 5.43 at 114.6M edges).
+#ifndef TFG_GW_SRC_DEPTH
+#define TFG_GW_SRC_DEPTH 4
+#endif
+#ifndef TFG_GW_SRC_UNROLL
+#define TFG_GW_SRC_UNROLL 8
+#endif
+
+template <int VEC>
+__device__ __forceinline__ void gw_axpy(float (&acc)[VEC], float w, const float (&v)[VEC]) {
+    if constexpr (VEC % 2 == 0) {
+        const float2 w2 = make_float2(w, w);
+#pragma unroll
+        for (int q = 0; q < VEC; q += 2) {
+            const float2 r = fma2(make_float2(v[q], v[q + 1]), w2, make_float2(acc[q], acc[q + 1]));
+            acc[q] = r.x;
+            acc[q + 1] = r.y;
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < VEC; ++q) acc[q] = fmaf(w, v[q], acc[q]);
+    }
+}
+
+template <int VEC>
+__device__ __forceinline__ void gw_load(const float *p, float (&r)[VEC]) {
+    if constexpr (VEC % 4 == 0) {
+#pragma unroll
+        for (int q = 0; q < VEC; q += 4) {
+            const float4 v = __ldg(reinterpret_cast<const float4 *>(p + q));
+            r[q] = v.x; r[q + 1] = v.y; r[q + 2] = v.z; r[q + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < VEC; ++q) r[q] = __ldg(p + q);
+    }
+}
+
+template <int VEC>
+__device__ __forceinline__ void gw_store(float *p, const float (&r)[VEC]) {
+    if constexpr (VEC % 4 == 0) {
+#pragma unroll
+        for (int q = 0; q < VEC; q += 4)
+            *reinterpret_cast<float4 *>(p + q) = make_float4(r[q], r[q + 1], r[q + 2], r[q + 3]);
+    } else {
+#pragma unroll
+        for (int q = 0; q < VEC; ++q) p[q] = r[q];
+    }
+}
+
+// 2^(m_old - m_new) for base-2 maxima; 0 for an empty state (m_old = -inf).
+__device__ __forceinline__ float gw_rescale(float m_old, float m_new) {
+    return m_old == -CUDART_INF_F ? 0.f : exp2f(m_old - m_new);
+}
+
+// A lane's place in a row of heads * channels features.
+template <int VEC, int LPR, int T, int NH>
+struct GatLane {
+    int sub, g, own;                 // own: features i < own of this lane exist
+    uint32_t f, f0;
+    int head[NH];
+    __device__ __forceinline__ void place(uint32_t ft, int heads, int channels) {
+        const int lane = threadIdx.x & 31;
+        sub = lane % LPR;
+        g = lane / LPR;
+        f = static_cast<uint32_t>(heads) * static_cast<uint32_t>(channels);
+        f0 = ft + sub * VEC;
+        own = f0 < f ? min(T, static_cast<int>((f - f0 + LPR * VEC - 1) / (LPR * VEC))) : 0;
+#pragma unroll
+        for (int i = 0; i < NH; ++i) head[i] = i < own ? static_cast<int>((f0 + i * LPR * VEC) / channels) : 0;
+    }
+};
+
+// Softmax passes by target.  TARGET_BWD = false: out = sum of alpha x, and alpha
+// if wanted.  TARGET_BWD = true: the row's statistics for the source pass and
+//   ds_dst = sum of alpha phi (dalpha - beta) = <grad_out[t], sum of alpha phi x> - beta sum of alpha phi,
+// phi the LeakyReLU's slope at the edge, dalpha = <grad_out[t], x[src]>: the sum
+// of the weighted rows is taken first, so an edge costs what it does in the
+// forward and the dot products are taken once per row.
+template <typename XT, int VEC, int LPR, int T, int NH, bool TARGET_BWD>
+struct GatByTarget {
+    using V = VecLoad<XT, VEC>;
+    static constexpr int kWarps = TFG_GW_WARPS, kLpr = LPR, G = 32 / LPR;
+    static constexpr int kTile = LPR * VEC * T, kHeadsPerLane = T;
+    static constexpr int kState = T * VEC + NH * (TARGET_BWD ? 3 : 2);
+    static constexpr int D = TFG_GW_DEPTH * G > 32 ? 32 / G : TFG_GW_DEPTH;   // gathers in flight per lane
+    const GatArgs &a;
+    GatLane<VEC, LPR, T, NH> at;
+    const char *xb;
+    uint32_t row_bytes;
+    float *scratch;                      // [warp][heads of the tile] (m, den), for alpha
+    float sd[NH], m[NH], den[NH], phi[NH], acc[T][VEC];
+
+    __device__ __forceinline__ GatByTarget(const GatArgs &args, uint32_t ft, float *scr) : a(args), scratch(scr) {
+        at.place(ft, a.heads, a.channels);
+        xb = reinterpret_cast<const char *>(static_cast<const XT *>(a.x) + (at.own > 0 ? at.f0 : 0));
+        row_bytes = at.f * static_cast<uint32_t>(sizeof(XT));
+    }
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int i = 0; i < NH; ++i) {
+            m[i] = -CUDART_INF_F;
+            den[i] = phi[i] = 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) acc[i][q] = 0.f;
+    }
+    __device__ __forceinline__ void open(int32_t t) {
+#pragma unroll
+        for (int i = 0; i < NH; ++i)
+            sd[i] = __ldg(a.s_dst + static_cast<uint64_t>(static_cast<uint32_t>(t)) * a.heads + at.head[i]);
+        clear();
+    }
+    template <bool CHECK>
+    __device__ __forceinline__ void add(const int32_t *ids, int cnt) {
+        float part[T][VEC], dpart[NH], ppart[NH];           // sums are blocked per window
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) part[i][q] = 0.f;
+#pragma unroll
+        for (int i = 0; i < NH; ++i) dpart[i] = ppart[i] = 0.f;
+        const int32_t *sp = ids + at.g;
+        int left = cnt - at.g;                              // this group's edges: sp[0], sp[G], ... below left
+#pragma unroll 1
+        for (int e = 0; e < cnt; e += G * D) {
+            typename V::Raw raw[D][T];
+            float z[D][NH];
+#pragma unroll
+            for (int u = 0; u < D; ++u) {
+                const uint32_t id = static_cast<uint32_t>(sp[u * G]);
+                const bool ok = !CHECK || left > u * G;
+                const XT *row = reinterpret_cast<const XT *>(xb + static_cast<uint64_t>(id) * row_bytes);
+#pragma unroll
+                for (int i = 0; i < NH; ++i)
+                    z[u][i] = ok ? __ldg(a.s_src + static_cast<uint64_t>(id) * a.heads + at.head[i]) : 0.f;
+#pragma unroll
+                for (int i = 0; i < T; ++i)
+                    raw[u][i] = (T == 1 ? ok : ok && i < at.own) ? V::raw(row + i * LPR * VEC) : V::zero();
+            }
+            float l[D][NH], w[D][NH];
+#pragma unroll
+            for (int i = 0; i < NH; ++i) {
+                float top = m[i];
+#pragma unroll
+                for (int u = 0; u < D; ++u) {
+                    z[u][i] += sd[i];
+                    l[u][i] = z[u][i] > 0.f ? z[u][i] : a.slope * z[u][i];
+                    if (CHECK && left <= u * G) l[u][i] = -CUDART_INF_F;
+                    top = fmaxf(top, l[u][i]);
+                }
+                if (top > m[i]) {                           // a new running maximum: rescale the sums so far
+                    const float sc = gw_rescale(m[i], top);
+                    den[i] *= sc;
+                    dpart[i] *= sc;
+                    if (TARGET_BWD) {
+                        phi[i] *= sc;
+                        ppart[i] *= sc;
+                    }
+#pragma unroll
+                    for (int j = 0; j < T; ++j) {
+                        if (NH > 1 && j != i) continue;
+#pragma unroll
+                        for (int q = 0; q < VEC; ++q) {
+                            acc[j][q] *= sc;
+                            part[j][q] *= sc;
+                        }
+                    }
+                    m[i] = top;
+                }
+#pragma unroll
+                for (int u = 0; u < D; ++u) {
+                    const float p = !CHECK || left > u * G ? exp2f(l[u][i] - m[i]) : 0.f;
+                    dpart[i] += p;
+                    w[u][i] = p;
+                    if (TARGET_BWD) {
+                        w[u][i] = z[u][i] > 0.f ? p : a.slope * p;
+                        ppart[i] += w[u][i];
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < D; ++u)
+#pragma unroll
+                for (int i = 0; i < T; ++i) {
+                    float v[VEC];
+                    V::widen(raw[u][i], v);
+                    gw_axpy(part[i], w[u][NH > 1 ? i : 0], v);
+                }
+            sp += G * D;
+            left -= G * D;
+        }
+#pragma unroll
+        for (int i = 0; i < NH; ++i) {
+            den[i] += dpart[i];
+            if (TARGET_BWD) phi[i] += ppart[i];
+        }
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) acc[i][q] += part[i][q];
+    }
+    // this state and (m2, den2, phi2, acc2), element by element
+    template <class Get>
+    __device__ __forceinline__ void fold(Get get) {
+        float sa[NH], sb[NH];
+#pragma unroll
+        for (int i = 0; i < NH; ++i) {
+            const float m2 = get(m[i], T * VEC + i), mm = fmaxf(m[i], m2);
+            sa[i] = gw_rescale(m[i], mm);
+            sb[i] = gw_rescale(m2, mm);
+            den[i] = den[i] * sa[i] + get(den[i], T * VEC + NH + i) * sb[i];
+            if (TARGET_BWD) phi[i] = phi[i] * sa[i] + get(phi[i], T * VEC + 2 * NH + i) * sb[i];
+            m[i] = mm;
+        }
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int q = 0; q < VEC; ++q)
+                acc[i][q] = acc[i][q] * sa[NH > 1 ? i : 0] + get(acc[i][q], i * VEC + q) * sb[NH > 1 ? i : 0];
+    }
+    __device__ __forceinline__ void join() {
+#pragma unroll
+        for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return __shfl_xor_sync(kFull, mine, o); });
+    }
+    __device__ __forceinline__ void merge(const float *slot) {
+        fold([&](float, int q) { return slot[q * LPR + at.sub]; });
+    }
+    __device__ __forceinline__ void park(float *slot) const {
+        if (at.g != 0) return;
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) slot[(i * VEC + q) * LPR + at.sub] = acc[i][q];
+#pragma unroll
+        for (int i = 0; i < NH; ++i) {
+            slot[(T * VEC + i) * LPR + at.sub] = m[i];
+            slot[(T * VEC + NH + i) * LPR + at.sub] = den[i];
+            if (TARGET_BWD) slot[(T * VEC + 2 * NH + i) * LPR + at.sub] = phi[i];
+        }
+    }
+    __device__ __forceinline__ void close(int32_t t, int32_t beg, int32_t end, bool shared) {
+        const uint64_t row = static_cast<uint64_t>(static_cast<uint32_t>(t)) * at.f + at.f0;
+        const bool any = end > beg;
+        if constexpr (!TARGET_BWD) {
+            if (at.g == 0) {
+#pragma unroll
+                for (int i = 0; i < T; ++i) {
+                    if (i >= at.own) continue;
+                    float r[VEC];
+#pragma unroll
+                    for (int q = 0; q < VEC; ++q) r[q] = any ? acc[i][q] / den[NH > 1 ? i : 0] : 0.f;
+                    gw_store(a.out + row + i * LPR * VEC, r);
+                }
+            }
+            if (a.alpha) {
+                const int warp = threadIdx.x >> 5;
+                put_statistics(warp);
+                if (!shared) weights(warp, t, beg, end, threadIdx.x & 31, 32);
+            }
+        } else {
+            // beta = <grad_out[t], out[t]> and <grad_out[t], acc> per head: this
+            // lane's share, then over the lanes of the head (a power of two of them)
+            const int hl = a.channels / VEC;
+            const uint64_t th = static_cast<uint64_t>(static_cast<uint32_t>(t)) * a.heads;
+#pragma unroll
+            for (int i = 0; i < T; ++i) {
+                float b = 0.f, d = 0.f;
+                if (i < at.own) {
+                    float g[VEC], o[VEC];
+                    gw_load(a.grad_out + row + i * LPR * VEC, g);
+                    gw_load(a.fwd_out + row + i * LPR * VEC, o);
+#pragma unroll
+                    for (int q = 0; q < VEC; ++q) {
+                        b = fmaf(g[q], o[q], b);
+                        d = fmaf(g[q], acc[i][q], d);
+                    }
+                }
+                for (int o = 1; o < hl; o <<= 1) {
+                    b += __shfl_xor_sync(kFull, b, o);
+                    d += __shfl_xor_sync(kFull, d, o);
+                }
+                if (at.g == 0 && i < at.own && (at.f0 + i * LPR * VEC) % a.channels == 0) {
+                    const int k = NH > 1 ? i : 0;
+                    const int h = static_cast<int>((at.f0 + i * LPR * VEC) / a.channels);
+                    a.ds_dst[th + h] = any ? (d - b * phi[k]) / den[k] : 0.f;
+                    a.stats[th + h] = make_float4(sd[k], m[k], any ? 1.f / den[k] : 0.f, b);
+                }
+            }
+        }
+    }
+    // alpha of the row's edges: after the row (by its warp), or for a row that
+    // several warps held by all warps of the CTA together
+    __device__ __forceinline__ bool wants_after() const { return !TARGET_BWD && a.alpha != nullptr; }
+    __device__ __forceinline__ void after(int w, int32_t t, int32_t beg, int32_t end) {
+        weights(w, t, beg, end, threadIdx.x, kWarps * 32);
+    }
+    // heads whose first feature lies in this tile
+    __device__ __forceinline__ int first_head() const {
+        return static_cast<int>((at.f0 - at.sub * VEC + a.channels - 1) / a.channels);
+    }
+    __device__ __forceinline__ float2 *statistics(int w) const {
+        return reinterpret_cast<float2 *>(scratch) + w * (LPR * T);
+    }
+    __device__ __forceinline__ void put_statistics(int warp) {
+        const int h0 = first_head();
+        __syncwarp();
+        if (at.g == 0) {
+#pragma unroll
+            for (int i = 0; i < T; ++i)
+                if (i < at.own && (at.f0 + i * LPR * VEC) % a.channels == 0)
+                    statistics(warp)[static_cast<int>((at.f0 + i * LPR * VEC) / a.channels) - h0] =
+                        make_float2(m[NH > 1 ? i : 0], den[NH > 1 ? i : 0]);
+        }
+        __syncwarp();
+    }
+    // threads id, id + stride, ... over (edge, head): coalesced, four in flight
+    __device__ __forceinline__ void weights(int w, int32_t t, int32_t beg, int32_t end, int id, int stride) {
+        const uint32_t ft = at.f0 - at.sub * VEC;
+        const int h0 = first_head();
+        const int nh = static_cast<int>((min(ft + LPR * VEC * T, at.f) + a.channels - 1) / a.channels) - h0;
+        const float *sdt = a.s_dst + static_cast<uint64_t>(static_cast<uint32_t>(t)) * a.heads + h0;
+        const float *ssh = a.s_src + h0;
+        const int64_t total = static_cast<int64_t>(end - beg) * nh;
+        for (int64_t i0 = id; i0 < total; i0 += 4 * stride) {
+            int64_t at_e[4];
+            int h[4];
+            uint64_t src[4];
+            float z[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t i = min64(i0 + u * stride, total - 1), e = nh == 1 ? i : i / nh;
+                h[u] = static_cast<int>(i - e * nh);
+                at_e[u] = beg + e;
+                src[u] = static_cast<uint32_t>(__ldg(a.col + at_e[u]));
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) z[u] = __ldg(ssh + src[u] * a.heads + h[u]) + __ldg(sdt + h[u]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (i0 + u * stride >= total) break;
+                const float2 st = statistics(w)[h[u]];
+                const float l = z[u] > 0.f ? z[u] : a.slope * z[u];
+                a.alpha[at_e[u] * a.heads + h0 + h[u]] = exp2f(l - st.x) / st.y;
+            }
+        }
+    }
+};
+
+// Backward by source (CSR by source: ids are targets).  With P = sum of alpha
+// grad_out[t] and Q = sum of alpha phi grad_out[t] over the out-edges,
+//   ds_src = sum of alpha phi (dalpha - beta) = <x[s], Q> - sum of alpha phi beta,
+//   grad_x = P + ds_src a_src + ds_dst a_dst:
+// no dot product per edge.  Every lane forms alpha of its head from the target's
+// statistics.
+template <typename XT, int VEC, int LPR, int T, int NH>
+struct GatBySource {
+    using V = VecLoad<float, VEC>;
+    static constexpr int kWarps = TFG_GW_SRC_WARPS, kLpr = LPR, G = 32 / LPR;
+    static constexpr int kTile = LPR * VEC * T, kHeadsPerLane = T;
+    static constexpr int kState = 2 * T * VEC + NH;
+    static constexpr int D = TFG_GW_SRC_DEPTH * G > 32 ? 32 / G : TFG_GW_SRC_DEPTH;
+    static constexpr int kUnroll = 32 / (G * D) < TFG_GW_SRC_UNROLL ? 32 / (G * D) : TFG_GW_SRC_UNROLL;
+    const GatArgs &a;
+    GatLane<VEC, LPR, T, NH> at;
+    const char *gb;
+    uint32_t row_bytes;
+    float ss[NH], sb[NH], P[T][VEC], Q[T][VEC];
+
+    __device__ __forceinline__ GatBySource(const GatArgs &args, uint32_t ft, float *) : a(args) {
+        at.place(ft, a.heads, a.channels);
+        gb = reinterpret_cast<const char *>(a.grad_out + (at.own > 0 ? at.f0 : 0));
+        row_bytes = at.f * 4u;
+    }
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int i = 0; i < NH; ++i) sb[i] = 0.f;
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) P[i][q] = Q[i][q] = 0.f;
+    }
+    __device__ __forceinline__ void open(int32_t s) {
+#pragma unroll
+        for (int i = 0; i < NH; ++i)
+            ss[i] = __ldg(a.s_src + static_cast<uint64_t>(static_cast<uint32_t>(s)) * a.heads + at.head[i]);
+        clear();
+    }
+    template <bool CHECK>
+    __device__ __forceinline__ void add(const int32_t *ids, int cnt) {
+        float p[T][VEC], r[T][VEC], bpart[NH];
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) p[i][q] = r[i][q] = 0.f;
+#pragma unroll
+        for (int i = 0; i < NH; ++i) bpart[i] = 0.f;
+        const int32_t *sp = ids + at.g;
+        int left = cnt - at.g;
+#pragma unroll CHECK ? 1 : kUnroll
+        for (int e = 0; e < (CHECK ? cnt : 32); e += G * D) {
+            typename V::Raw raw[D][T];
+            float4 st[D][NH];
+#pragma unroll
+            for (int u = 0; u < D; ++u) {
+                const uint32_t id = static_cast<uint32_t>(sp[u * G]);
+                const bool ok = !CHECK || left > u * G;
+                const float *row = reinterpret_cast<const float *>(gb + static_cast<uint64_t>(id) * row_bytes);
+#pragma unroll
+                for (int i = 0; i < NH; ++i)
+                    st[u][i] = ok ? __ldg(a.stats + static_cast<uint64_t>(id) * a.heads + at.head[i])
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int i = 0; i < T; ++i)
+                    raw[u][i] = (T == 1 ? ok : ok && i < at.own) ? V::raw(row + i * LPR * VEC) : V::zero();
+            }
+#pragma unroll
+            for (int u = 0; u < D; ++u) {
+                float al[NH], af[NH];
+#pragma unroll
+                for (int i = 0; i < NH; ++i) {
+                    const float z = ss[i] + st[u][i].x;
+                    const float l = z > 0.f ? z : a.slope * z;
+                    al[i] = exp2f(l - st[u][i].y) * st[u][i].z;
+                    if (CHECK) al[i] = left > u * G ? al[i] : 0.f;
+                    af[i] = z > 0.f ? al[i] : a.slope * al[i];
+                    bpart[i] = fmaf(af[i], st[u][i].w, bpart[i]);
+                }
+#pragma unroll
+                for (int i = 0; i < T; ++i) {
+                    float v[VEC];
+                    V::widen(raw[u][i], v);
+                    gw_axpy(p[i], al[NH > 1 ? i : 0], v);
+                    gw_axpy(r[i], af[NH > 1 ? i : 0], v);
+                }
+            }
+            sp += G * D;
+            left -= G * D;
+        }
+#pragma unroll
+        for (int i = 0; i < NH; ++i) sb[i] += bpart[i];
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) {
+                P[i][q] += p[i][q];
+                Q[i][q] += r[i][q];
+            }
+    }
+    template <class Get>
+    __device__ __forceinline__ void fold(Get get) {
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) {
+                P[i][q] += get(P[i][q], i * VEC + q);
+                Q[i][q] += get(Q[i][q], (T + i) * VEC + q);
+            }
+#pragma unroll
+        for (int i = 0; i < NH; ++i) sb[i] += get(sb[i], 2 * T * VEC + i);
+    }
+    __device__ __forceinline__ void join() {
+#pragma unroll
+        for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return __shfl_xor_sync(kFull, mine, o); });
+    }
+    __device__ __forceinline__ void merge(const float *slot) {
+        fold([&](float, int q) { return slot[q * LPR + at.sub]; });
+    }
+    __device__ __forceinline__ void park(float *slot) const {
+        if (at.g != 0) return;
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) {
+                slot[(i * VEC + q) * LPR + at.sub] = P[i][q];
+                slot[((T + i) * VEC + q) * LPR + at.sub] = Q[i][q];
+            }
+#pragma unroll
+        for (int i = 0; i < NH; ++i) slot[(2 * T * VEC + i) * LPR + at.sub] = sb[i];
+    }
+    __device__ __forceinline__ bool wants_after() const { return false; }
+    __device__ __forceinline__ void after(int, int32_t, int32_t, int32_t) {}
+    __device__ __forceinline__ void close(int32_t s, int32_t, int32_t, bool) {
+        const uint64_t row = static_cast<uint64_t>(static_cast<uint32_t>(s)) * at.f + at.f0;
+        const uint64_t sh = static_cast<uint64_t>(static_cast<uint32_t>(s)) * a.heads;
+        const int hl = a.channels / VEC;
+#pragma unroll
+        for (int i = 0; i < T; ++i) {
+            float d = 0.f;
+            if (i < at.own) {
+                float xs[VEC];
+                VecLoad<XT, VEC>::load(static_cast<const XT *>(a.x) + row + i * LPR * VEC, xs);
+#pragma unroll
+                for (int q = 0; q < VEC; ++q) d = fmaf(xs[q], Q[i][q], d);
+            }
+            for (int o = 1; o < hl; o <<= 1) d += __shfl_xor_sync(kFull, d, o);
+            if (at.g == 0 && i < at.own) {
+                const uint32_t fi = at.f0 + i * LPR * VEC;
+                const int h = static_cast<int>(fi / a.channels);
+                const float ds = d - sb[NH > 1 ? i : 0], dd = __ldg(a.ds_dst + sh + h);
+                float as[VEC], ad[VEC], r[VEC];
+                gw_load(a.a_src + fi, as);
+                gw_load(a.a_dst + fi, ad);
+#pragma unroll
+                for (int q = 0; q < VEC; ++q) r[q] = P[i][q] + ds * as[q] + dd * ad[q];
+                gw_store(a.grad_x + row + i * LPR * VEC, r);
+                if (fi % a.channels == 0) a.ds_src[sh + h] = ds;
+            }
+        }
+    }
+};
+
+template <class Policy>
+__global__ void __launch_bounds__(Policy::kWarps * 32, 1) gat_walk(GatArgs a) {
+    extern __shared__ __align__(16) float s_parts[];
+    __shared__ WalkShared<Policy::kWarps> s_walk;
+    const uint32_t f = static_cast<uint32_t>(a.heads) * static_cast<uint32_t>(a.channels);
+    for (uint32_t ft = blockIdx.y * Policy::kTile; ft < f; ft += gridDim.y * Policy::kTile) {
+        Policy p(a, ft, s_parts + 2 * Policy::kWarps * Policy::kState * Policy::kLpr);
+        walk_rows<Policy::kWarps>(a.rowptr, a.col, a.n, p, s_walk, s_parts);
+        __syncthreads();                   // before the next tile reuses the shared memory
+    }
+}
+
+template <class Policy>
+cudaError_t launch_walk(const GatArgs &a, cudaStream_t s) {
+    constexpr int parts = 2 * Policy::kWarps * Policy::kState * Policy::kLpr * static_cast<int>(sizeof(float));
+    constexpr int stats = Policy::kWarps * Policy::kLpr * Policy::kHeadsPerLane * static_cast<int>(sizeof(float2));
+    const int smem = parts + (a.alpha ? stats : 0);
+    if (smem > 32 * 1024) {   // with the static part above the 48 KB every launch may use
+        const cudaError_t err = cudaFuncSetAttribute(gat_walk<Policy>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     parts + stats);
+        if (err != cudaSuccess) return err;
+    }
+    const int64_t tiles = (static_cast<int64_t>(a.heads) * a.channels + Policy::kTile - 1) / Policy::kTile;
+    const dim3 grid(static_cast<unsigned>(min64(a.n, static_cast<int64_t>(sm_count()))), static_cast<unsigned>(min64(tiles, 65535)));
+    gat_walk<Policy><<<grid, Policy::kWarps * 32, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+}  // namespace tfg

@@ -1,0 +1,122 @@
+// Row walk with a policy: the attention passes' version of the walk that
+// aggregate_rows (agg.cuh) makes.  Equal shares of edges and row ends per warp
+// (row_share.cuh), edges taken in windows of 32 whose ids are requested a window
+// ahead and staged in shared memory, rows taking their edges from the window
+// one after the other, parts of a row shared by several warps merged in warp
+// order after the CTA's one barrier.
+//
+// A policy P holds one lane's state of one row and provides
+//   kLpr, kState          lanes per row, floats a lane parks for another warp
+//   open(t)               start row t (loads what the row needs, clears the state)
+//   add<CHECK>(ids, cnt)  edges ids[0 .. cnt) (whole warp; ids in shared memory,
+//                         readable up to 32 entries past them)
+//   join()                combine the warp's lane groups (every lane ends with
+//                         the state of the warp's edges)
+//   park(slot) / merge(slot)  this lane's state to / combined with a parked one,
+//                         float q of lane sub at slot[q * kLpr + sub]
+//   close(t, beg, end, shared)  write row t, whose edges are [beg, end); shared:
+//                         it was held by several warps
+//   after(w, t, beg, end)  called by every warp of the CTA for each shared row t,
+//                         closed by warp w, when wants_after() says so
+#pragma once
+
+#include "row_share.cuh"
+
+namespace tfg {
+
+template <int WARPS>
+struct WalkShared {
+    int64_t row[2];
+    int32_t tail_row[WARPS], head_row[WARPS];
+    int32_t ids[WARPS][64];
+};
+
+constexpr int kWalkMinWork = 8;   // work (edges + kRowCost per row) a warp should have, at least
+
+// parts: [2 * WARPS][kState * kLpr] floats of shared memory
+template <int WARPS, class P>
+__device__ __forceinline__ void walk_rows(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col,
+                                          int64_t n, P &p, WalkShared<WARPS> &s, float *parts) {
+    WarpShare<WARPS> sh;
+    if (!sh.init(rowptr, n, kWalkMinWork, s.row)) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int32_t *ids = s.ids[warp];
+    constexpr int kSlot = P::kState * P::kLpr;
+    if (lane == 0) s.head_row[warp] = -1;
+    const int32_t kb = sh.kb, tb = sh.tb;
+    uint32_t ahead = static_cast<uint32_t>(sh.ka);          // the window after the staged one
+    auto col_at = [&](uint32_t k) { return k + lane < static_cast<uint32_t>(kb) ? ld_stream(col + k + lane) : 0; };
+    int32_t c1 = col_at(ahead);
+    auto next_window = [&]() {
+        __syncwarp();                                       // the previous window's reads are done
+        ids[lane] = c1;
+        __syncwarp();
+        ahead += 32;
+        c1 = col_at(ahead);
+    };
+    int32_t t = sh.ta, rwin;
+    int tl = 0;                                             // row t is lane tl of the row ends held
+    auto row_window = [&]() {
+        const int64_t r = static_cast<int64_t>(t) + lane;
+        rwin = r < n ? __ldg(rowptr + r + 1) : 0;
+        tl = 0;
+    };
+    row_window();
+    next_window();
+    int32_t k = sh.ka, rbeg = __ldg(rowptr + t);
+    int j = 0;                                              // position in the staged window
+    for (;;) {
+        const bool closes = t < tb;
+        const int32_t rend = closes ? __shfl_sync(kFull, rwin, tl) : kb;
+        int rem = rend - k;
+        k = rend;
+        if (closes || rem > 0) {
+            p.open(t);
+            while (rem > 0) {
+                if (j == 32) {
+                    next_window();
+                    j = 0;
+                }
+                const int cnt = min(rem, 32 - j);
+                if (cnt == 32) p.template add<false>(ids, 32);
+                else p.template add<true>(ids + j, cnt);
+                rem -= cnt;
+                j += cnt;
+            }
+            p.join();
+        } else {
+            p.clear();
+        }
+        if (!closes) break;
+        if (t == sh.ta && sh.head_split) {                  // parts of it sit with earlier warps
+            p.park(parts + (WARPS + warp) * kSlot);
+            if (lane == 0) s.head_row[warp] = t;
+        } else {
+            p.close(t, rbeg, rend, false);
+        }
+        rbeg = rend;
+        ++t;
+        if (++tl == 32) row_window();
+    }
+    p.park(parts + warp * kSlot);                           // this warp's part of row tb
+    if (lane == 0) s.tail_row[warp] = tb;
+    __syncthreads();
+    const int32_t hr = s.head_row[warp];
+    if (hr >= 0) {                                          // earlier parts in warp order, then ours
+        int first = warp;
+        while (first > 0 && s.tail_row[first - 1] == hr) --first;
+        p.open(hr);
+        for (int w = first; w < warp; ++w) p.merge(parts + w * kSlot);
+        p.merge(parts + (WARPS + warp) * kSlot);
+        p.close(hr, __ldg(rowptr + hr), __ldg(rowptr + hr + 1), true);
+    }
+    if (p.wants_after()) {
+        __syncthreads();
+        for (int w = 0; w < WARPS; ++w) {
+            const int32_t r = s.head_row[w];
+            if (r >= 0) p.after(w, r, __ldg(rowptr + r), __ldg(rowptr + r + 1));
+        }
+    }
+}
+
+}  // namespace tfg

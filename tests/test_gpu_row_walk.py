@@ -7,7 +7,8 @@ import pytest
 import torch
 
 import oracle
-from _helpers import TOL_F32, assert_exact_f32, assert_scaled_close, dev, features, host_features
+from _helpers import (KAPPA_GAT, TOL_F32, assert_alpha_close, assert_exact_f32, assert_scaled_close,
+                      csr_rows, dev, features, gat_logit_mag, host_features)
 from paper_2101_11552_gb300 import graphgen as gg
 from paper_2101_11552_gb300 import tfg
 
@@ -17,9 +18,9 @@ pytestmark = pytest.mark.gpu
 DEGREES = [0, 1, 31, 32, 33, 0, 0, 64, 5, 3, 9000, 2, 0, 95, 96, 97] + [3, 0, 7] * 40
 
 
-def graph(seed):
+def graph(seed, more=0):
     rng = np.random.default_rng(seed)
-    deg = np.array(DEGREES)
+    deg = np.array(DEGREES + [3, 0, 7] * more)
     n = len(deg)
     dst = np.repeat(np.arange(n), deg)
     src = rng.integers(0, n - 1, size=dst.size)      # the last node is nobody's source
@@ -63,3 +64,44 @@ def test_widths(f, dtype):
                                   add_self_loops=1).cpu().numpy()
     dw = np.abs(ew)
     assert np.isfinite(out).all() and dw.size       # values: test_gpu_propagate; here every width runs
+
+
+# layouts of one slice per lane, several features per lane (one head and many),
+# and more than one feature tile; backward where the layout has one
+LAYOUTS = [(1, 3), (1, 41), (1, 100), (3, 5), (2, 9), (5, 13), (1, 130), (7, 20), (8, 16), (4, 8),
+           (1, 32), (2, 64), (3, 4), (16, 4), (6, 32), (12, 4)]
+
+
+@pytest.mark.parametrize("more", [0, 1000])     # mean in-degree 72 and 6
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("heads,channels", LAYOUTS)
+def test_gat_layouts(heads, channels, dtype, more):
+    f = heads * channels
+    ei, n = graph(f, more)
+    rng = np.random.default_rng(2000 + f)
+    x = rng.standard_normal((n, f), dtype=np.float32)
+    wl = gg.Workload("walk", n, ei, x, x_bf16=gg.bf16_bits_rne(x))
+    a_s, a_d = (0.5 * rng.standard_normal((2, f))).astype(np.float32)
+    csr = tfg.tfg_build_csr(dev(ei), n)
+    xd, xh = features(wl, dtype), host_features(wl, dtype)
+    out, alpha = tfg.tfg_edge_softmax_aggregate(csr.rowptr, csr.col, xd, heads, channels, dev(a_s),
+                                                dev(a_d), 0.2, want_alpha=True)
+    ref, ref_alpha, scale = oracle.edge_softmax(ei, n, xh, heads, channels, a_s, a_d, 0.2)
+    what = f"{dtype} H={heads} C={channels} more={more}"
+    assert_scaled_close(out.cpu().numpy(), ref, scale, TOL_F32, "out " + what)
+    rowptr, col, perm, _ = oracle.build_csr(ei, n)
+    row = csr_rows(rowptr)
+    lam = gat_logit_mag(oracle.widen(xh), col, row, heads, channels, a_s, a_d)
+    assert_alpha_close(alpha.cpu().numpy(), ref_alpha[perm], lam, row, KAPPA_GAT, "alpha " + what)
+    if f > 256 or not (32 % channels == 0 if channels <= 32 else channels % 32 == 0):
+        return
+    src = tfg.tfg_build_csr_by_source(dev(ei), n)
+    g = rng.standard_normal((n, f)).astype(np.float32)
+    got = tfg.tfg_edge_softmax_aggregate_backward(csr.rowptr, csr.col, src.rowptr, src.col, xd, heads,
+                                                  channels, dev(a_s), dev(a_d), 0.2, out, dev(g))
+    want = oracle.edge_softmax_backward(ei, n, xh, heads, channels, a_s, a_d, 0.2, g)
+    lam_max = np.zeros((n, heads))
+    np.maximum.at(lam_max, row, lam)
+    tol = TOL_F32 + KAPPA_GAT * float(np.max(lam + lam_max[row]))
+    for name, a, b, sc in zip(("grad_x", "grad_a_src", "grad_a_dst"), got, want[:3], want[3]):
+        assert_scaled_close(a.cpu().numpy(), b, sc, tol, f"{name} {what}")
