@@ -71,6 +71,9 @@ namespace {
 #ifndef TFG_AGG_DEPTH
 #define TFG_AGG_DEPTH 8
 #endif
+#ifndef TFG_AGG_PART4
+#define TFG_AGG_PART4 2
+#endif
 constexpr int kAggWarps = TFG_AGG_WARPS;
 constexpr int kAggThreads = kAggWarps * 32;
 // Work (edges + kRowCost per row) a warp should have, at least: 8 against 32 on
@@ -106,7 +109,7 @@ struct RowAgg {
     static constexpr int kTile = LPR * VEC * T;               // features of one pass
     static constexpr int D0 = T > 1 || VEC == 8 ? 4 : TFG_AGG_DEPTH;
     static constexpr int D = D0 * G > 32 ? 32 / G : D0;       // gathers in flight per lane, full windows
-    static constexpr int P = 4;                               // the same, partial windows
+    static constexpr int P = G >= 4 ? TFG_AGG_PART4 : 4;       // the same, partial windows: about 8 edges a step
     static_assert(32 % (G * D) == 0 && G * P <= 32, "steps of G * D slots must tile the 32-edge window");
 
     static __device__ __forceinline__ float combine(float a, float b) { return kIsMax ? fmaxf(a, b) : a + b; }

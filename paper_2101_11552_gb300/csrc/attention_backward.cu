@@ -28,7 +28,7 @@
 // The same file holds the backward of the dot-product form (below).
 #include <math_constants.h>
 
-#include "common.cuh"
+#include "dot_walk.cuh"
 #include "gat_walk.cuh"
 
 namespace tfg {
@@ -279,14 +279,6 @@ size_t bw_align(size_t b) { return (b + 255) & ~size_t(255); }
 
 int bw_blocks(int64_t n) { return static_cast<int>((n + kBwRowsPerBlock - 1) / kBwRowsPerBlock); }
 
-constexpr int64_t kFbMinWork = 2048;   // edges + rows per CTA, at least
-
-// Sum over the aligned groups of hl lanes (hl a power of two).
-__device__ __forceinline__ float group_sum(float v, int hl) {
-    for (int o = 1; o < hl; o <<= 1) v += __shfl_xor_sync(kFull, v, o);
-    return v;
-}
-
 // ---------------------------------------------------------------------------
 // Backward of the dot-product attention (l = scale <q[t], k[s]> per head):
 //   dalpha = <grad_out[t,h,:], v[s,h,:]>,  beta[t,h] = <grad_out[t,h,:], out[t,h,:]>
@@ -462,304 +454,6 @@ __global__ void __launch_bounds__(kBwThreads) dot_bwd_sources(DotBwArgs a) {
     }
 }
 
-// Fast form of the dot-product backward, on the forward's fast layout
-// (channels = lh * VEC, lh a power of two, 16-byte aligned rows): a lane
-// holds VEC features of one head, the lh lanes of a head finish each dot
-// product with a butterfly, G = 32 / LPR lane groups take every G-th edge
-// and merge their states at the end; tiles of LPR * VEC features loop.
-//  * target pass (CSR by target): per row t the running maximum m and
-//    denominator den of each head and the rescaled sum
-//    acc = sum of exp(l - m) (dalpha - beta) k[s], in one pass;
-//    grad_q[t] = scale * acc / den; stats[t, h] = (m, 1 / den, beta, 0).
-//  * source pass (CSR by source): per row s, alpha of each out-edge from
-//    stats[t]; grad_k[s] = scale * sum dl q[t], grad_v[s] = sum alpha grad_out[t].
-// Measured on the 114.6M-edge graph (bf16, 8 x 16): 4 / 2 edges in flight
-// (target / source) at 2 CTAs per SM 21.60 ms, 4 / 4 20.95 ms (kept), 2 / 2
-// 23.32 ms, 2 / 1 at 3 CTAs 23.23 ms, 8 / 2 at 1 CTA 35.65 ms.
-#ifndef TFG_DB_UNROLL_TGT
-#define TFG_DB_UNROLL_TGT 4       // edges in flight per lane, target pass
-#endif
-#ifndef TFG_DB_UNROLL_SRC
-#define TFG_DB_UNROLL_SRC 4       // edges in flight per lane, source pass
-#endif
-constexpr int kDbUnroll = TFG_DB_UNROLL_TGT;
-constexpr int kDbUnrollSrc = TFG_DB_UNROLL_SRC;
-#ifndef TFG_DB_BLOCKS
-#define TFG_DB_BLOCKS 3           // resident CTAs per SM of the fast passes, fp32
-#endif
-#ifndef TFG_DB_BLOCKS16
-#define TFG_DB_BLOCKS16 2         // the same for bf16 (8 features a lane: 3 spill)
-#endif
-
-struct DotFastBwArgs {
-    const int32_t *rowptr, *col, *rowptr_src, *col_src;
-    const void *q, *k, *v;
-    int64_t n;
-    int heads, channels, lh;
-    float scale, scale2;              // natural and base-2 (scale * log2 e)
-    const float *out, *grad_out;
-    float4 *stats;                    // [N, H]: (m, 1 / den, beta, 0)
-    float *grad_q, *grad_k, *grad_v;
-};
-
-template <int VEC>
-__device__ __forceinline__ float vec_dot(const float (&a)[VEC], const float (&b)[VEC]) {
-    float2 d = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int i = 0; i < VEC; i += 2) d = fma2(make_float2(a[i], a[i + 1]), make_float2(b[i], b[i + 1]), d);
-    return d.x + d.y;
-}
-
-template <int VEC>
-__device__ __forceinline__ void vec_axpy(float (&acc)[VEC], float w, const float (&v)[VEC]) {
-    const float2 w2 = make_float2(w, w);
-#pragma unroll
-    for (int i = 0; i < VEC; i += 2) {
-        const float2 r = fma2(make_float2(v[i], v[i + 1]), w2, make_float2(acc[i], acc[i + 1]));
-        acc[i] = r.x;
-        acc[i + 1] = r.y;
-    }
-}
-
-template <int VEC>
-__device__ __forceinline__ void load_f32(const float *p, float (&r)[VEC]) {
-#pragma unroll
-    for (int i = 0; i < VEC; i += 4) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(p + i));
-        r[i] = v.x; r[i + 1] = v.y; r[i + 2] = v.z; r[i + 3] = v.w;
-    }
-}
-
-template <typename XT, int VEC, int LPR>
-__device__ __forceinline__ void dot_fast_bwd_target(const DotFastBwArgs &a, int64_t t, int lane) {
-    using V = VecLoad<XT, VEC>;
-    constexpr int G = 32 / LPR;
-    static_assert(G * kDbUnroll <= 32, "a step must stay inside the 32-edge chunk");
-    const int g = lane / LPR, sub = lane % LPR;
-    const int64_t f = static_cast<int64_t>(a.heads) * a.channels;
-    const XT *qp = static_cast<const XT *>(a.q), *kp = static_cast<const XT *>(a.k),
-             *vp = static_cast<const XT *>(a.v);
-    const int64_t beg = a.rowptr[t], end = a.rowptr[t + 1];
-    const uint32_t row_bytes = static_cast<uint32_t>(f) * static_cast<uint32_t>(sizeof(XT));
-    for (int64_t ft = 0; ft < f; ft += LPR * VEC) {
-        const int64_t f0 = ft + sub * VEC;
-        const bool fok = f0 < f;
-        const int64_t fl = fok ? f0 : 0;
-        float qv[VEC], gt[VEC], ov[VEC];
-        V::load(qp + t * f + fl, qv);
-        load_f32<VEC>(a.grad_out + t * f + fl, gt);
-        load_f32<VEC>(a.out + t * f + fl, ov);
-        if (!fok) {
-#pragma unroll
-            for (int i = 0; i < VEC; ++i) qv[i] = gt[i] = 0.f;
-        }
-        const float beta = group_sum(vec_dot(gt, ov), a.lh);
-        const char *kb = reinterpret_cast<const char *>(kp + fl);
-        const char *vb = reinterpret_cast<const char *>(vp + fl);
-        float m = -CUDART_INF_F, den = 0.f, acc[VEC];
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) acc[i] = 0.f;
-        int cnext = beg + lane < end ? ld_stream(a.col + beg + lane) : 0;
-        for (int64_t base = beg; base < end; base += 32) {
-            const int cnt = static_cast<int>(min64(32, end - base));
-            const int c = cnext;
-            cnext = base + 32 + lane < end ? ld_stream(a.col + base + 32 + lane) : 0;
-            float den_part = 0.f, part[VEC];
-#pragma unroll
-            for (int i = 0; i < VEC; ++i) part[i] = 0.f;
-            for (int j = 0; j < cnt; j += G * kDbUnroll) {
-                typename V::Raw rk[kDbUnroll], rv[kDbUnroll];
-                bool ok[kDbUnroll];
-#pragma unroll
-                for (int u = 0; u < kDbUnroll; ++u) {
-                    const int k = j + u * G + g;
-                    const uint64_t off = static_cast<uint64_t>(
-                        static_cast<uint32_t>(__shfl_sync(kFull, c, k & 31))) * row_bytes;
-                    ok[u] = k < cnt;
-                    rk[u] = ok[u] ? V::raw(reinterpret_cast<const XT *>(kb + off)) : V::zero();
-                    rv[u] = ok[u] ? V::raw(reinterpret_cast<const XT *>(vb + off)) : V::zero();
-                }
-                float l[kDbUnroll], da[kDbUnroll];
-                float mc = -CUDART_INF_F;
-#pragma unroll
-                for (int u = 0; u < kDbUnroll; ++u) {
-                    float kv[VEC], vv[VEC];
-                    V::widen(rk[u], kv);
-                    V::widen(rv[u], vv);
-                    l[u] = group_sum(vec_dot(qv, kv), a.lh);
-                    da[u] = group_sum(vec_dot(gt, vv), a.lh);
-                    l[u] = ok[u] ? l[u] * a.scale2 : -CUDART_INF_F;
-                    mc = fmaxf(mc, l[u]);
-                }
-                if (mc > m) {   // new running maximum for this lane's head
-                    const float sc = m == -CUDART_INF_F ? 0.f : exp2f(m - mc);
-                    den *= sc;
-                    den_part *= sc;
-#pragma unroll
-                    for (int i = 0; i < VEC; ++i) {
-                        acc[i] *= sc;
-                        part[i] *= sc;
-                    }
-                    m = mc;
-                }
-#pragma unroll
-                for (int u = 0; u < kDbUnroll; ++u) {
-                    const float p = ok[u] ? exp2f(l[u] - m) : 0.f;
-                    den_part += p;
-                    float kv[VEC];
-                    V::widen(rk[u], kv);
-                    vec_axpy(part, p * (da[u] - beta), kv);
-                }
-            }
-            den += den_part;
-#pragma unroll
-            for (int i = 0; i < VEC; ++i) acc[i] += part[i];
-        }
-        // merge the G groups' states in a fixed butterfly order
-#pragma unroll
-        for (int o = LPR; o < 32; o <<= 1) {
-            const float mo = __shfl_xor_sync(kFull, m, o);
-            const float dn = __shfl_xor_sync(kFull, den, o);
-            const float mm = fmaxf(m, mo);
-            const float x = m == -CUDART_INF_F ? 0.f : exp2f(m - mm);
-            const float y = mo == -CUDART_INF_F ? 0.f : exp2f(mo - mm);
-            den = den * x + dn * y;
-#pragma unroll
-            for (int i = 0; i < VEC; ++i) {
-                const float ao = __shfl_xor_sync(kFull, acc[i], o);
-                acc[i] = acc[i] * x + ao * y;
-            }
-            m = mm;
-        }
-        if (lane < LPR && fok) {
-            const float w = end > beg ? a.scale / den : 0.f;
-#pragma unroll
-            for (int i = 0; i < VEC; i += 4)
-                *reinterpret_cast<float4 *>(a.grad_q + t * f + f0 + i) =
-                    make_float4(acc[i] * w, acc[i + 1] * w, acc[i + 2] * w, acc[i + 3] * w);
-            if (sub % a.lh == 0)
-                a.stats[t * a.heads + f0 / a.channels] =
-                    make_float4(m, den > 0.f ? 1.f / den : 0.f, beta, 0.f);
-        }
-    }
-}
-
-template <typename XT, int VEC, int LPR>
-__device__ __forceinline__ void dot_fast_bwd_source(const DotFastBwArgs &a, int64_t s, int lane) {
-    using V = VecLoad<XT, VEC>;
-    constexpr int G = 32 / LPR;
-    static_assert(G * kDbUnrollSrc <= 32, "a step must stay inside the 32-edge chunk");
-    const int g = lane / LPR, sub = lane % LPR;
-    const int64_t f = static_cast<int64_t>(a.heads) * a.channels;
-    const XT *qp = static_cast<const XT *>(a.q), *kp = static_cast<const XT *>(a.k),
-             *vp = static_cast<const XT *>(a.v);
-    const int64_t beg = a.rowptr_src[s], end = a.rowptr_src[s + 1];
-    const uint32_t row_bytes = static_cast<uint32_t>(f) * static_cast<uint32_t>(sizeof(XT));
-    const uint32_t grow_bytes = static_cast<uint32_t>(f) * 4u;
-    for (int64_t ft = 0; ft < f; ft += LPR * VEC) {
-        const int64_t f0 = ft + sub * VEC;
-        const bool fok = f0 < f;
-        const int64_t fl = fok ? f0 : 0;
-        const int h = static_cast<int>(fl / a.channels);
-        float ks[VEC], vs[VEC];
-        V::load(kp + s * f + fl, ks);
-        V::load(vp + s * f + fl, vs);
-        const char *qb = reinterpret_cast<const char *>(qp + fl);
-        const char *gb = reinterpret_cast<const char *>(a.grad_out + fl);
-        float dk[VEC], dv[VEC];
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) dk[i] = dv[i] = 0.f;
-        int cnext = beg + lane < end ? ld_stream(a.col_src + beg + lane) : 0;
-        for (int64_t base = beg; base < end; base += 32) {
-            const int cnt = static_cast<int>(min64(32, end - base));
-            const int c = cnext;
-            cnext = base + 32 + lane < end ? ld_stream(a.col_src + base + 32 + lane) : 0;
-            float pk[VEC], pv[VEC];
-#pragma unroll
-            for (int i = 0; i < VEC; ++i) pk[i] = pv[i] = 0.f;
-            for (int j = 0; j < cnt; j += G * kDbUnrollSrc) {
-                typename V::Raw rq[kDbUnrollSrc];
-                float gr[kDbUnrollSrc][VEC];
-                float4 st[kDbUnrollSrc];
-                bool ok[kDbUnrollSrc];
-#pragma unroll
-                for (int u = 0; u < kDbUnrollSrc; ++u) {
-                    const int k = j + u * G + g;
-                    const uint32_t t = static_cast<uint32_t>(__shfl_sync(kFull, c, k & 31));
-                    ok[u] = k < cnt;
-                    rq[u] = ok[u] ? V::raw(reinterpret_cast<const XT *>(qb + uint64_t(t) * row_bytes)) : V::zero();
-                    if (ok[u]) {
-                        load_f32<VEC>(reinterpret_cast<const float *>(gb + uint64_t(t) * grow_bytes), gr[u]);
-                        st[u] = __ldg(a.stats + static_cast<int64_t>(t) * a.heads + h);
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < VEC; ++i) gr[u][i] = 0.f;
-                        st[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < kDbUnrollSrc; ++u) {
-                    float qv[VEC];
-                    V::widen(rq[u], qv);
-                    const float l = group_sum(vec_dot(qv, ks), a.lh) * a.scale2;
-                    const float da = group_sum(vec_dot(gr[u], vs), a.lh);
-                    const float alpha = ok[u] ? exp2f(l - st[u].x) * st[u].y : 0.f;
-                    vec_axpy(pk, alpha * (da - st[u].z), qv);
-                    vec_axpy(pv, alpha, gr[u]);
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < VEC; ++i) {
-                dk[i] += pk[i];
-                dv[i] += pv[i];
-            }
-        }
-#pragma unroll
-        for (int o = LPR; o < 32; o <<= 1)
-#pragma unroll
-            for (int i = 0; i < VEC; ++i) {
-                dk[i] += __shfl_xor_sync(kFull, dk[i], o);
-                dv[i] += __shfl_xor_sync(kFull, dv[i], o);
-            }
-        if (lane < LPR && fok) {
-#pragma unroll
-            for (int i = 0; i < VEC; i += 4) {
-                *reinterpret_cast<float4 *>(a.grad_k + s * f + f0 + i) =
-                    make_float4(dk[i] * a.scale, dk[i + 1] * a.scale, dk[i + 2] * a.scale,
-                                dk[i + 3] * a.scale);
-                *reinterpret_cast<float4 *>(a.grad_v + s * f + f0 + i) =
-                    make_float4(dv[i], dv[i + 1], dv[i + 2], dv[i + 3]);
-            }
-        }
-    }
-}
-
-template <typename XT, int VEC, int LPR>
-__global__ void __launch_bounds__(kBwThreads, VEC >= 8 ? TFG_DB_BLOCKS16 : TFG_DB_BLOCKS) dot_fast_bwd_targets(DotFastBwArgs a) {
-    for_each_row(a.rowptr, a.n, [&](int64_t t, int lane) { dot_fast_bwd_target<XT, VEC, LPR>(a, t, lane); });
-}
-
-template <typename XT, int VEC, int LPR>
-__global__ void __launch_bounds__(kBwThreads, VEC >= 8 ? TFG_DB_BLOCKS16 : TFG_DB_BLOCKS) dot_fast_bwd_sources(DotFastBwArgs a) {
-    for_each_row(a.rowptr_src, a.n, [&](int64_t s, int lane) { dot_fast_bwd_source<XT, VEC, LPR>(a, s, lane); });
-}
-
-template <typename XT, int VEC>
-void launch_dot_fast_bw(const DotFastBwArgs &a, int64_t e, cudaStream_t s) {
-    const int64_t chunks = static_cast<int64_t>(a.heads) * a.channels / VEC;
-    const int grid = balanced_grid(a.n, e, kFbMinWork);
-    if (chunks >= 32 || a.lh > 16) {
-        dot_fast_bwd_targets<XT, VEC, 32><<<grid, kBwThreads, 0, s>>>(a);
-        dot_fast_bwd_sources<XT, VEC, 32><<<grid, kBwThreads, 0, s>>>(a);
-    } else if (chunks > 8 || a.lh > 8) {
-        dot_fast_bwd_targets<XT, VEC, 16><<<grid, kBwThreads, 0, s>>>(a);
-        dot_fast_bwd_sources<XT, VEC, 16><<<grid, kBwThreads, 0, s>>>(a);
-    } else {
-        dot_fast_bwd_targets<XT, VEC, 8><<<grid, kBwThreads, 0, s>>>(a);
-        dot_fast_bwd_sources<XT, VEC, 8><<<grid, kBwThreads, 0, s>>>(a);
-    }
-}
-
 template <typename XT, int NT>
 cudaError_t launch_dot_bw(const DotBwArgs &a, cudaStream_t s) {
     const int rows = ceil_div(a.n, kBwWarps);
@@ -923,6 +617,9 @@ size_t dot_attention_backward_workspace_bytes(int64_t n, int heads) {
     return 4 * bw_align(sizeof(float) * size_t(n > 0 ? n : 1) * size_t(heads));
 }
 
+cudaError_t launch_dot_walk_targets(const DotArgs &a, int x_dtype, cudaStream_t s);
+cudaError_t launch_dot_walk_sources(const DotArgs &a, int x_dtype, cudaStream_t s);
+
 cudaError_t launch_dot_softmax_backward(const int32_t *rowptr, const int32_t *col,
                                         const int32_t *rowptr_src, const int32_t *col_src,
                                         const void *q, const void *k, const void *v, int x_dtype,
@@ -938,12 +635,13 @@ cudaError_t launch_dot_softmax_backward(const int32_t *rowptr, const int32_t *co
     if (a16(q) && a16(k) && a16(v) && a16(out) && a16(grad_out) && a16(grad_q) && a16(grad_k) &&
         a16(grad_v) && channels % vec == 0 && lh >= 1 && lh <= 32 && (lh & (lh - 1)) == 0) {
         // workspace: the [N, H] float4 statistics (4 * nh bytes)
-        const DotFastBwArgs fa{rowptr, col, rowptr_src, col_src, q, k, v, n, heads, channels, lh,
-                               scale, scale * 1.4426950408889634f, out, grad_out,
-                               reinterpret_cast<float4 *>(w), grad_q, grad_k, grad_v};
-        if (x_dtype == TFG_BF16) launch_dot_fast_bw<uint16_t, 8>(fa, e, s);
-        else launch_dot_fast_bw<float, 4>(fa, e, s);
-        return cudaGetLastError();
+        DotArgs da{rowptr, col, q, k, v, n, heads, channels, lh, scale, scale * 1.4426950408889634f, nullptr,
+                   nullptr, out, grad_out, reinterpret_cast<float4 *>(w), grad_q, grad_k, grad_v};
+        const cudaError_t err = launch_dot_walk_targets(da, x_dtype, s);
+        if (err != cudaSuccess) return err;
+        da.rowptr = rowptr_src;
+        da.col = col_src;
+        return launch_dot_walk_sources(da, x_dtype, s);
     }
     DotBwArgs a{rowptr, col, rowptr_src, col_src, q, k, v, n, heads, channels, scale,
                 scale * 1.4426950408889634f, out, grad_out,

@@ -9,40 +9,30 @@
 //
 // Unlike the additive form there is no per-node score to precompute: every
 // logit is a dot product of a gathered key row with the target's query row,
-// so each edge gathers a key row and a value row.  One warp owns a target row
-// and makes one pass with the running-maximum softmax (the running sums are
-// rescaled by exp(m_old - m_new) when the maximum rises; the result is
-// unchanged), blocked per 32-edge chunk to keep fp32 chains short.
+// so each edge gathers a key row and a value row.  A row is read in one pass
+// with the running-maximum softmax (the running sums are rescaled by exp(m_old -
+// m_new) when the maximum rises; the result is unchanged), blocked per 32 edges
+// to keep fp32 chains short.
 //
-//  * fast form (channels = LH * VEC with LH a power of two <= 32, 16-byte
-//    aligned rows): a row tile of LPR * VEC features holds whole heads; a
-//    lane holds VEC features of one head, the LH lanes of a head finish the
-//    dot product with a butterfly, so every lane of a head sees the same
-//    logit.  G = 32 / LPR lane groups take every G-th edge and merge their
-//    (m, den, acc) states at the end.  Tiles loop when F > LPR * VEC.
-//  * general form (any channels <= 256, any alignment): the warp walks the
-//    heads of the row one at a time, lanes striding over the channels of the
+//  * channels = LH * VEC with LH a power of two <= 32, 16-byte aligned rows: on
+//    short rows the row walk (dot_walk.cuh), on long ones dot_fast: a row tile of
+//    LPR * VEC features holds whole heads; a lane holds VEC features of one head,
+//    the LH lanes of a head finish the dot product with a butterfly, so every lane
+//    of a head sees the same logit.  G = 32 / LPR lane groups take every G-th edge
+//    and merge their (m, den, acc) states at the end.
+//  * general form (any channels <= 256, any alignment): one warp per row walks
+//    the heads of the row one at a time, lanes striding over the channels of the
 //    head (NCH chunks of 32), the logit finished by a full-warp butterfly.
 #include <math_constants.h>
 
 #include <type_traits>
 
-#include "common.cuh"
+#include "dot_walk.cuh"
 
 namespace tfg {
 namespace {
 
 constexpr int kDotThreads = 256;
-// Tuning knobs (compile-time; the defaults are the measured best on GB300).
-#ifndef TFG_DOT_UNROLL
-#define TFG_DOT_UNROLL 8   // edges gathered per lane per step (key + value rows)
-#endif
-#ifndef TFG_DOT_MINB
-#define TFG_DOT_MINB 2     // resident CTAs per SM asked of the compiler, 16-byte bf16 path
-#endif
-// (the fp32 path, with half the features per load, keeps 4 in flight: 8 spill there)
-template <int VEC>
-__host__ __device__ constexpr int dot_unroll() { return VEC >= 8 ? TFG_DOT_UNROLL : 4; }
 constexpr int64_t kDotMinWork = 2048;      // edges + rows per CTA, at least
 constexpr int kDotMaxChannels = 256;
 
@@ -57,17 +47,6 @@ constexpr float kDotLog2e = 1.4426950408889634f;
 __device__ __forceinline__ float dot_rescale(float m_old, float m_new) {
     return m_old == -CUDART_INF_F ? 0.f : exp2f(m_old - m_new);
 }
-
-struct DotArgs {
-    const int32_t *rowptr;
-    const int32_t *col;
-    const void *q, *k, *v;
-    int64_t n;
-    int heads, channels;
-    float scale;
-    float *out;
-    float *alpha;
-};
 
 // Rows of a work-balanced range (edges + rows split evenly across CTAs),
 // taken one at a time by the CTA's warps from a shared counter.
@@ -88,40 +67,19 @@ __device__ __forceinline__ void dot_rows(const int32_t *rowptr, int64_t n, RowFn
     }
 }
 
-// This lane's share of a head's dot product: two interleaved fp32 chains
-// through the packed fma (even and odd channels), added at the end.
+// Long rows (a mean in-degree of 32 and more): a row per warp from a shared
+// counter, 8 edges' key and value rows in flight per lane.  At 114.6M edges, 8 x
+// 16 bf16, it takes 3.97 ms, the row walk 4.27 (24 warps, 4 in flight) to 5.17; on
+// short rows the walk is faster (169,343 nodes, mean in-degree 6.9, 8 x 16 fp32:
+// 170 us against 481).
+#ifndef TFG_DOT_WALK_DEGREE
+#define TFG_DOT_WALK_DEGREE 32
+#endif
+constexpr int64_t kDotWalkDegree = TFG_DOT_WALK_DEGREE;
+// edges gathered per lane per step (the fp32 form, with half the features per
+// load, keeps 4: 8 spill there)
 template <int VEC>
-__device__ __forceinline__ float lane_dot(const float (&q)[VEC], const float (&k)[VEC]) {
-    if constexpr (VEC % 2 == 0) {
-        float2 d = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < VEC; i += 2)
-            d = fma2(make_float2(q[i], q[i + 1]), make_float2(k[i], k[i + 1]), d);
-        return d.x + d.y;
-    } else {
-        float d = 0.f;
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) d = fmaf(q[i], k[i], d);
-        return d;
-    }
-}
-
-// part += p * v through the packed fma.
-template <int VEC>
-__device__ __forceinline__ void axpy_vec(float (&part)[VEC], float p, const float (&v)[VEC]) {
-    if constexpr (VEC % 2 == 0) {
-        const float2 p2 = make_float2(p, p);
-#pragma unroll
-        for (int i = 0; i < VEC; i += 2) {
-            const float2 r = fma2(make_float2(v[i], v[i + 1]), p2, make_float2(part[i], part[i + 1]));
-            part[i] = r.x;
-            part[i + 1] = r.y;
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) part[i] = fmaf(p, v[i], part[i]);
-    }
-}
+__host__ __device__ constexpr int dot_unroll() { return VEC >= 8 ? 8 : 4; }
 
 // LH > 0: lanes per head fixed at compile time (the butterfly unrolls);
 // LH = 0 takes lh_arg.
@@ -185,14 +143,14 @@ __device__ __forceinline__ void dot_fast_row(const DotArgs &a, int lh_arg, int64
                 for (int u = 0; u < kDotUnroll; ++u) {
                     float kv[VEC];
                     V::widen(rk[u], kv);
-                    float d = lane_dot(qv, kv);
+                    float d = dw_dot(qv, kv);
 #pragma unroll
                     for (int o = 1; o < lh; o <<= 1) d += __shfl_xor_sync(kFull, d, o);
-                    l[u] = ok[u] ? d * a.scale : -CUDART_INF_F;
+                    l[u] = ok[u] ? d * a.scale2 : -CUDART_INF_F;
                     mc = fmaxf(mc, l[u]);
                 }
                 if (mc > m) {   // new running maximum for this lane's head
-                    const float sc = dot_rescale(m, mc);
+                    const float sc = dw_rescale(m, mc);
                     den *= sc;
                     den_part *= sc;
 #pragma unroll
@@ -208,7 +166,7 @@ __device__ __forceinline__ void dot_fast_row(const DotArgs &a, int lh_arg, int64
                     den_part += p;
                     float vv[VEC];
                     V::widen(rv[u], vv);
-                    axpy_vec(part, p, vv);
+                    dw_axpy(part, p, vv);
                 }
             }
             den += den_part;
@@ -230,7 +188,7 @@ __device__ __forceinline__ void dot_fast_row(const DotArgs &a, int lh_arg, int64
             const float mo = __shfl_xor_sync(kFull, m, s);
             const float dn = __shfl_xor_sync(kFull, den, s);
             const float mm = fmaxf(m, mo);
-            const float x = dot_rescale(m, mm), y = dot_rescale(mo, mm);
+            const float x = dw_rescale(m, mm), y = dw_rescale(mo, mm);
             den = den * x + dn * y;
 #pragma unroll
             for (int q = 0; q < VEC; ++q) {
@@ -253,10 +211,10 @@ __device__ __forceinline__ void dot_fast_row(const DotArgs &a, int lh_arg, int64
                 const int64_t src = ok ? __ldg(a.col + k) : 0;
                 float kv[VEC];
                 V::load(kp + src * f + fl, kv);
-                float d = lane_dot(qv, kv);
+                float d = dw_dot(qv, kv);
                 for (int o = 1; o < lh; o <<= 1) d += __shfl_xor_sync(kFull, d, o);
                 if (ok && fok && sub % lh == 0)
-                    a.alpha[k * a.heads + h] = exp2f(d * a.scale - m) / den;
+                    a.alpha[k * a.heads + h] = exp2f(d * a.scale2 - m) / den;
             }
         }
     }
@@ -310,7 +268,7 @@ __device__ __forceinline__ void dot_general_row(const DotArgs &a, int64_t t, int
                 for (int j = 0; j < NCH; ++j) d = fmaf(qv[j], kv[j], d);
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) d += __shfl_xor_sync(kFull, d, o);
-                const float l = d * a.scale;
+                const float l = d * a.scale2;
                 if (l > m) {
                     const float sc = dot_rescale(m, l);
                     den *= sc;
@@ -349,7 +307,7 @@ __device__ __forceinline__ void dot_general_row(const DotArgs &a, int64_t t, int
                 }
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) d += __shfl_xor_sync(kFull, d, o);
-                if (lane == 0) a.alpha[k * a.heads + h] = exp2f(d * a.scale - m) / den;
+                if (lane == 0) a.alpha[k * a.heads + h] = exp2f(d * a.scale2 - m) / den;
             }
         }
     }
@@ -358,7 +316,7 @@ __device__ __forceinline__ void dot_general_row(const DotArgs &a, int64_t t, int
 // 16-byte bf16 rows hold twice the features per gather: two resident CTAs
 // per SM leave the registers for kDotUnroll key + value gathers in flight.
 template <typename XT, int VEC, int LPR, int LH>
-__global__ void __launch_bounds__(kDotThreads, VEC >= 8 ? TFG_DOT_MINB : 3) dot_fast(DotArgs a, int lh) {
+__global__ void __launch_bounds__(kDotThreads, VEC >= 8 ? 2 : 3) dot_fast(DotArgs a, int lh) {
     dot_rows(a.rowptr, a.n, [&](int64_t t, int lane) { dot_fast_row<XT, VEC, LPR, LH>(a, lh, t, lane); });
 }
 
@@ -367,17 +325,9 @@ __global__ void __launch_bounds__(kDotThreads, 3) dot_general(DotArgs a) {
     dot_rows(a.rowptr, a.n, [&](int64_t t, int lane) { dot_general_row<XT, NCH>(a, t, lane); });
 }
 
-#ifndef TFG_DOT_STATIC_LH
-#define TFG_DOT_STATIC_LH 1   // one kernel per lanes-per-head count
-#endif
-
 // lh (a power of two <= LPR) picks the kernel with that many lanes per head.
 template <typename XT, int VEC, int LPR>
 void launch_fast_lpr(const DotArgs &a, int lh, int grid, cudaStream_t s) {
-    if constexpr (!TFG_DOT_STATIC_LH) {
-        dot_fast<XT, VEC, LPR, 0><<<grid, kDotThreads, 0, s>>>(a, lh);
-        return;
-    }
     switch (lh) {
         case 1: dot_fast<XT, VEC, LPR, 1><<<grid, kDotThreads, 0, s>>>(a, lh); break;
         case 2: dot_fast<XT, VEC, LPR, 2><<<grid, kDotThreads, 0, s>>>(a, lh); break;
@@ -403,6 +353,9 @@ void launch_fast_vec(const DotArgs &a, int lh, int grid, cudaStream_t s) {
     else launch_fast_lpr<XT, VEC, 8>(a, lh, grid, s);
 }
 
+template <typename XT, int VEC, int LPR, int LH>
+using DotForward = DotByTarget<XT, VEC, LPR, LH, false>;
+
 template <typename XT>
 void launch_general(const DotArgs &a, int grid, cudaStream_t s) {
     const int nch = (a.channels + 31) / 32;
@@ -423,18 +376,22 @@ cudaError_t launch_dot_softmax(const int32_t *rowptr, const int32_t *col, const 
                                int heads, int channels, float scale, float *out, float *alpha,
                                cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    const DotArgs a{rowptr, col, q, k, v, n, heads, channels, scale * kDotLog2e, out, alpha};
+    const int vec = x_dtype == TFG_BF16 ? 8 : 4;
+    const DotArgs a{rowptr, col, q, k, v, n, heads, channels, channels / vec, scale, scale * kDotLog2e, out, alpha};
     const int grid = balanced_grid(n, e, kDotMinWork);
     auto a16 = [](const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
     const bool aligned = a16(q) && a16(k) && a16(v) && a16(out);
-    const int vec = x_dtype == TFG_BF16 ? 8 : 4;
     if (aligned && channels % vec == 0 && is_pow2_upto32(channels / vec)) {
-        if (x_dtype == TFG_BF16) launch_fast_vec<uint16_t, 8>(a, channels / 8, grid, s);
-        else launch_fast_vec<float, 4>(a, channels / 4, grid, s);
-    } else {
-        if (x_dtype == TFG_BF16) launch_general<uint16_t>(a, grid, s);
-        else launch_general<float>(a, grid, s);
+        if (e < kDotWalkDegree * n) {
+            if (x_dtype == TFG_BF16) return launch_dot_pass<DotForward, uint16_t, 8>(a, s);
+            return launch_dot_pass<DotForward, float, 4>(a, s);
+        }
+        if (x_dtype == TFG_BF16) launch_fast_vec<uint16_t, 8>(a, a.lh, grid, s);
+        else launch_fast_vec<float, 4>(a, a.lh, grid, s);
+        return cudaGetLastError();
     }
+    if (x_dtype == TFG_BF16) launch_general<uint16_t>(a, grid, s);
+    else launch_general<float>(a, grid, s);
     return cudaGetLastError();
 }
 

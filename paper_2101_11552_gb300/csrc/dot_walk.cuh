@@ -1,0 +1,481 @@
+// The three edge passes of the dot-product attention as row-walk policies
+// (row_walk.cuh): forward, backward by target, backward by source.  A row's head
+// is LH lanes of VEC features (LH a power of two; LH = 0 takes the count at run
+// time), which finish a dot product with a butterfly, so every lane of a head
+// holds the same logit; LPR lanes cover whole heads of a row (wider rows loop
+// over tiles), G = 32 / LPR lane groups take every G-th edge.  Logits are in base-2
+// units (scale2 = scale log2 e).
+#pragma once
+#include <math_constants.h>
+
+#include "row_walk.cuh"
+
+namespace tfg {
+
+struct DotArgs {
+    const int32_t *rowptr, *col;          // CSR of the pass
+    const void *q, *k, *v;
+    int64_t n;
+    int heads, channels, lh;
+    float scale, scale2;
+    float *out, *alpha;                   // forward
+    const float *fwd_out, *grad_out;      // backward
+    float4 *stats;                        // [N, H]: (m, 1 / den, beta, 0)
+    float *grad_q, *grad_k, *grad_v;
+};
+
+namespace {
+
+// What bounds it: instructions on short rows (169,343 nodes, mean in-degree 6.9, 8
+// x 16 fp32: forward 166, by target 206, by source 253 us); on long ones (114.6M
+// edges, 8 x 16 bf16) the gathers, 896 bytes an edge by source (7.6 ms, 13.5 TB/s)
+// and 512 by target (5.4 ms, 11 TB/s), with one CTA of few, register-rich warps.
+// Before: a row per warp, the lanes of a head a run-time count and every slot
+// tested, 141 instructions for two edges by source: 12.4 ms, by target 8.9 ms.
+//
+// Tuning knobs, measured there: by target 20 warps 5.54 ms, 16 5.66, 24 6.29; four
+// steps of a full window unrolled 5.35, one 5.54.  By source 16 warps with 4 edges
+// in flight 7.6 ms, 20 with 2 8.8, 12 with 4 9.1; before the earlier windows' sums
+// waited in shared memory 8.9.  Forward (short rows; fp32) 24 warps 166 us, 20 183.
+#ifndef TFG_DW_FWD_WARPS
+#define TFG_DW_FWD_WARPS 24
+#endif
+#ifndef TFG_DW_TGT_WARPS
+#define TFG_DW_TGT_WARPS 20
+#endif
+#ifndef TFG_DW_SRC_WARPS
+#define TFG_DW_SRC_WARPS 16
+#endif
+#ifndef TFG_DW_DEPTH
+#define TFG_DW_DEPTH 4        // edges in flight per lane group, full windows
+#endif
+#ifndef TFG_DW_UNROLL
+#define TFG_DW_UNROLL 4       // by target: steps of a full window unrolled
+#endif
+
+template <int VEC>
+__device__ __forceinline__ float dw_dot(const float (&a)[VEC], const float (&b)[VEC]) {
+    float2 d = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < VEC; i += 2) d = fma2(make_float2(a[i], a[i + 1]), make_float2(b[i], b[i + 1]), d);
+    return d.x + d.y;
+}
+template <int VEC>
+__device__ __forceinline__ void dw_axpy(float (&acc)[VEC], float w, const float (&v)[VEC]) {
+    const float2 w2 = make_float2(w, w);
+#pragma unroll
+    for (int i = 0; i < VEC; i += 2) {
+        const float2 r = fma2(make_float2(v[i], v[i + 1]), w2, make_float2(acc[i], acc[i + 1]));
+        acc[i] = r.x;
+        acc[i + 1] = r.y;
+    }
+}
+template <int VEC>
+__device__ __forceinline__ void dw_load(const float *p, float (&r)[VEC]) {
+#pragma unroll
+    for (int i = 0; i < VEC; i += 4) {
+        const float4 v = __ldg(reinterpret_cast<const float4 *>(p + i));
+        r[i] = v.x; r[i + 1] = v.y; r[i + 2] = v.z; r[i + 3] = v.w;
+    }
+}
+template <int VEC>
+__device__ __forceinline__ void dw_store(float *p, const float (&r)[VEC], float w) {
+#pragma unroll
+    for (int i = 0; i < VEC; i += 4)
+        *reinterpret_cast<float4 *>(p + i) = make_float4(r[i] * w, r[i + 1] * w, r[i + 2] * w, r[i + 3] * w);
+}
+template <int VEC>
+__device__ __forceinline__ void dw_clear(float (&r)[VEC]) {
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) r[i] = 0.f;
+}
+__device__ __forceinline__ float dw_rescale(float m_old, float m_new) {
+    return m_old == -CUDART_INF_F ? 0.f : exp2f(m_old - m_new);
+}
+
+// A lane's place and the sum over its head's lanes.
+template <typename XT, int VEC, int LPR, int LH>
+struct DotLane {
+    using V = VecLoad<XT, VEC>;
+    int sub, g, head, lh;
+    bool own;                             // the lane holds features
+    uint32_t f, f0, row_bytes;
+    __device__ __forceinline__ DotLane(const DotArgs &a, uint32_t ft) {
+        const int lane = threadIdx.x & 31;
+        sub = lane % LPR;
+        g = lane / LPR;
+        f = static_cast<uint32_t>(a.heads) * static_cast<uint32_t>(a.channels);
+        own = ft + sub * VEC < f;
+        f0 = own ? ft + sub * VEC : 0;    // lanes past F read (and never store) feature 0
+        head = static_cast<int>(f0 / a.channels);
+        lh = LH > 0 ? LH : a.lh;
+        row_bytes = f * static_cast<uint32_t>(sizeof(XT));
+    }
+    __device__ __forceinline__ float head_sum(float v) const {
+        if constexpr (LH > 0) {
+#pragma unroll
+            for (int o = 1; o < LH; o <<= 1) v += __shfl_xor_sync(kFull, v, o);
+        } else {
+            for (int o = 1; o < lh; o <<= 1) v += __shfl_xor_sync(kFull, v, o);
+        }
+        return v;
+    }
+    __device__ __forceinline__ const char *base(const void *p) const {
+        return reinterpret_cast<const char *>(static_cast<const XT *>(p) + f0);
+    }
+    __device__ __forceinline__ const XT *row(const char *b, uint32_t id) const {
+        return reinterpret_cast<const XT *>(b + static_cast<uint64_t>(id) * row_bytes);
+    }
+    __device__ __forceinline__ uint64_t at(int32_t r) const {   // element f0 of row r
+        return static_cast<uint64_t>(static_cast<uint32_t>(r)) * f + f0;
+    }
+    __device__ __forceinline__ uint64_t stat(uint32_t r, int heads) const {
+        return static_cast<uint64_t>(r) * heads + head;
+    }
+};
+
+// Sums are blocked per window of 32 edges.  The sums of a row's earlier windows wait
+// in shared memory (element q of a lane at q * 32), so that the registers hold
+// one set of accumulators and more rows in flight; a row of one window never
+// goes there.
+template <int N>
+struct DotHeld {
+    float *at;
+    bool begun, used;
+    __device__ __forceinline__ explicit DotHeld(float *warp_slots) : at(warp_slots + (threadIdx.x & 31)) {}
+    __device__ __forceinline__ void clear() { begun = used = false; }
+    // before a window: the previous window's sums join the earlier ones
+    __device__ __forceinline__ void next(float (&acc)[N]) {
+        if (begun) {
+#pragma unroll
+            for (int q = 0; q < N; ++q) {
+                at[q * 32] = (used ? at[q * 32] : 0.f) + acc[q];
+                acc[q] = 0.f;
+            }
+            used = true;
+        }
+        begun = true;
+    }
+    __device__ __forceinline__ void scale(float sc) {
+        if (used) {
+#pragma unroll
+            for (int q = 0; q < N; ++q) at[q * 32] *= sc;
+        }
+    }
+    __device__ __forceinline__ void last(float (&acc)[N]) {
+        if (used) {
+#pragma unroll
+            for (int q = 0; q < N; ++q) acc[q] += at[q * 32];
+            used = false;
+        }
+    }
+};
+
+// Softmax over the in-edges of a target.  BWD = false: acc = sum of p v[src];
+// BWD = true: acc = sum of p (dalpha - beta) k[src], dalpha = <grad_out[t], v[src]>.
+template <typename XT, int VEC, int LPR, int LH, bool BWD>
+struct DotByTarget {
+    using L = DotLane<XT, VEC, LPR, LH>;
+    using V = VecLoad<XT, VEC>;
+    static constexpr int kWarps = BWD ? TFG_DW_TGT_WARPS : TFG_DW_FWD_WARPS, kLpr = LPR, G = 32 / LPR;
+    static constexpr int kTile = LPR * VEC, kHeadsPerLane = 1;
+    static constexpr int kState = VEC + 2, kHeld = VEC;
+    static constexpr int kFull = TFG_DW_DEPTH * G > 32 ? 32 / G : TFG_DW_DEPTH, kUnroll = TFG_DW_UNROLL;
+    static constexpr int kPart = walk_part(G) < kFull ? walk_part(G) : kFull;
+    const DotArgs &a;
+    L ln;
+    const char *kb, *vb;
+    float2 *scratch;                      // [warp][heads of the tile] (m, den), for alpha
+    DotHeld<VEC> held;                    // the sums of the row's earlier windows
+    float qv[VEC], gt[BWD ? VEC : 1], beta, m, den, acc[VEC];
+
+    __device__ __forceinline__ DotByTarget(const DotArgs &args, uint32_t ft, float *hold, float *scr)
+        : a(args), ln(args, ft), scratch(reinterpret_cast<float2 *>(scr)), held(hold) {
+        kb = ln.base(a.k);
+        vb = ln.base(a.v);
+        beta = 0.f;
+    }
+    __device__ __forceinline__ void clear() {
+        m = -CUDART_INF_F;
+        den = 0.f;
+        dw_clear(acc);
+        held.clear();
+    }
+    __device__ __forceinline__ void load_query(int32_t t) {
+        V::load(static_cast<const XT *>(a.q) + ln.at(t), qv);
+        if (!ln.own) dw_clear(qv);
+    }
+    __device__ __forceinline__ void open(int32_t t) {
+        load_query(t);
+        if constexpr (BWD) {
+            float ov[VEC];
+            dw_load(a.grad_out + ln.at(t), gt);
+            dw_load(a.fwd_out + ln.at(t), ov);
+            if (!ln.own) dw_clear(gt);
+            beta = ln.head_sum(dw_dot(gt, ov));
+        }
+        clear();
+    }
+    // D edges of the group, sp[0], sp[G], ... (CHECK: those below left)
+    template <int D, bool CHECK>
+    __device__ __forceinline__ void step(const int32_t *sp, int left, float &dpart) {
+        typename V::Raw rk[D], rv[D];
+#pragma unroll
+        for (int u = 0; u < D; ++u) {
+            const uint32_t id = static_cast<uint32_t>(sp[u * G]);
+            const bool ok = !CHECK || left > u * G;
+            rk[u] = ok ? V::raw(ln.row(kb, id)) : V::zero();
+            rv[u] = ok ? V::raw(ln.row(vb, id)) : V::zero();
+        }
+        float l[D], w[D], top = m;
+#pragma unroll
+        for (int u = 0; u < D; ++u) {
+            float x[VEC];
+            V::widen(rk[u], x);
+            l[u] = ln.head_sum(dw_dot(qv, x)) * a.scale2;
+            if (CHECK && left <= u * G) l[u] = -CUDART_INF_F;
+            top = fmaxf(top, l[u]);
+            if constexpr (BWD) {
+                V::widen(rv[u], x);
+                w[u] = ln.head_sum(dw_dot(gt, x)) - beta;
+            }
+        }
+        if (top > m) {                                           // a new running maximum: rescale the sums so far
+            const float sc = dw_rescale(m, top);
+            den *= sc;
+            dpart *= sc;
+#pragma unroll
+            for (int i = 0; i < VEC; ++i) acc[i] *= sc;
+            held.scale(sc);
+            m = top;
+        }
+#pragma unroll
+        for (int u = 0; u < D; ++u) {
+            const float p = !CHECK || left > u * G ? exp2f(l[u] - m) : 0.f;
+            dpart += p;
+            float x[VEC];
+            V::widen(BWD ? rk[u] : rv[u], x);
+            dw_axpy(acc, !BWD ? p : (!CHECK || left > u * G ? p * w[u] : 0.f), x);
+        }
+    }
+    template <bool CHECK>
+    __device__ __forceinline__ void add(const int32_t *ids, int cnt) {
+        held.next(acc);                                          // sums are blocked per window
+        float dpart = 0.f;
+        const int32_t *sp = ids + ln.g;
+        if (!CHECK) {                                            // a full window
+#pragma unroll kUnroll
+            for (int e = 0; e < 32; e += G * kFull) step<kFull, false>(sp + e, 0, dpart);
+            den += dpart;
+            return;
+        }
+#pragma unroll 1
+        for (; cnt >= G * kFull; cnt -= G * kFull, sp += G * kFull) step<kFull, false>(sp, 0, dpart);
+#pragma unroll 1
+        for (; CHECK && cnt > 0; cnt -= G * kPart, sp += G * kPart) step<kPart, true>(sp, cnt - ln.g, dpart);
+        den += dpart;
+    }
+    template <class Get>
+    __device__ __forceinline__ void fold(Get get) {
+        const float m2 = get(m, VEC), mm = fmaxf(m, m2);
+        const float sa = dw_rescale(m, mm), sb = dw_rescale(m2, mm);
+        den = den * sa + get(den, VEC + 1) * sb;
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) acc[i] = acc[i] * sa + get(acc[i], i) * sb;
+        m = mm;
+    }
+    __device__ __forceinline__ void join() {
+        held.last(acc);
+#pragma unroll
+        for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return __shfl_xor_sync(kFull, mine, o); });
+    }
+    __device__ __forceinline__ void merge(const float *slot) {
+        fold([&](float, int i) { return slot[i * LPR + ln.sub]; });
+    }
+    __device__ __forceinline__ void park(float *slot) const {
+        if (ln.g != 0) return;
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) slot[i * LPR + ln.sub] = acc[i];
+        slot[VEC * LPR + ln.sub] = m;
+        slot[(VEC + 1) * LPR + ln.sub] = den;
+    }
+    __device__ __forceinline__ void close(int32_t t, int32_t beg, int32_t end, bool shared) {
+        const bool any = end > beg;
+        if (ln.g == 0 && ln.own) {
+            if constexpr (BWD) {
+                dw_store(a.grad_q + ln.at(t), acc, any ? a.scale / den : 0.f);
+                if (ln.sub % ln.lh == 0)
+                    a.stats[ln.stat(static_cast<uint32_t>(t), a.heads)] =
+                        make_float4(m, any ? 1.f / den : 0.f, beta, 0.f);
+            } else {
+                float r[VEC];
+#pragma unroll
+                for (int i = 0; i < VEC; ++i) r[i] = any ? acc[i] / den : 0.f;
+                dw_store(a.out + ln.at(t), r, 1.f);
+            }
+        }
+        if (!BWD && a.alpha) {
+            const int warp = threadIdx.x >> 5;
+            __syncwarp();
+            if (ln.g == 0 && ln.sub % ln.lh == 0) statistics(warp)[ln.sub / ln.lh] = make_float2(m, den);
+            __syncwarp();
+            if (!shared) weights(warp, t, beg, end, ln.g, G);
+        }
+    }
+    // alpha: every logit again, one writer per (edge, head); a row that several
+    // warps held is done by all warps of the CTA
+    __device__ __forceinline__ float2 *statistics(int w) const { return scratch + w * LPR; }
+    __device__ __forceinline__ bool wants_after() const { return !BWD && a.alpha != nullptr; }
+    __device__ __forceinline__ void after(int w, int32_t t, int32_t beg, int32_t end) {
+        load_query(t);
+        weights(w, t, beg, end, (threadIdx.x >> 5) * G + ln.g, kWarps * G);
+    }
+    __device__ __forceinline__ void weights(int w, int32_t, int32_t beg, int32_t end, int first, int stride) {
+        const float2 st = statistics(w)[ln.sub / ln.lh];
+        const int64_t steps = (static_cast<int64_t>(end) - beg + stride - 1) / stride;   // the same for every lane
+        for (int64_t i = 0; i < steps; ++i) {
+            const int64_t e = beg + i * stride + first;
+            const bool ok = e < end;
+            const uint32_t src = ok ? static_cast<uint32_t>(__ldg(a.col + e)) : 0u;
+            float x[VEC];
+            V::load(ln.row(kb, src), x);
+            const float l = ln.head_sum(dw_dot(qv, x)) * a.scale2;
+            if (ok && ln.own && ln.sub % ln.lh == 0) a.alpha[e * a.heads + ln.head] = exp2f(l - st.x) / st.y;
+        }
+    }
+};
+
+// Backward by source (CSR by source: ids are targets), from the targets'
+// statistics: grad_k = scale sum of alpha (dalpha - beta) q[t], grad_v = sum of
+// alpha grad_out[t].
+template <typename XT, int VEC, int LPR, int LH>
+struct DotBySource {
+    using L = DotLane<XT, VEC, LPR, LH>;
+    using V = VecLoad<XT, VEC>;
+    static constexpr int kWarps = TFG_DW_SRC_WARPS, kLpr = LPR, G = 32 / LPR;
+    static constexpr int kTile = LPR * VEC, kHeadsPerLane = 1;
+    static constexpr int kState = 2 * VEC, kHeld = 2 * VEC;
+    static constexpr int kFull = TFG_DW_DEPTH * G > 32 ? 32 / G : TFG_DW_DEPTH;
+    static constexpr int kPart = walk_part(G) < kFull ? walk_part(G) : kFull;
+    const DotArgs &a;
+    L ln;
+    const char *qb, *gb;
+    DotHeld<2 * VEC> held;
+    float ks[VEC], vs[VEC], dkv[2 * VEC];  // grad_k's and grad_v's sums
+
+    __device__ __forceinline__ DotBySource(const DotArgs &args, uint32_t ft, float *hold, float *)
+        : a(args), ln(args, ft), held(hold) {
+        qb = ln.base(a.q);
+        gb = reinterpret_cast<const char *>(a.grad_out + ln.f0);
+    }
+    __device__ __forceinline__ void clear() {
+        dw_clear(dkv);
+        held.clear();
+    }
+    __device__ __forceinline__ void open(int32_t s) {
+        V::load(static_cast<const XT *>(a.k) + ln.at(s), ks);
+        V::load(static_cast<const XT *>(a.v) + ln.at(s), vs);
+        clear();
+    }
+    template <int D, bool CHECK>
+    __device__ __forceinline__ void step(const int32_t *sp, int left) {
+        typename V::Raw rq[D];
+        float gr[D][VEC];
+        float4 st[D];
+#pragma unroll
+        for (int u = 0; u < D; ++u) {
+            const uint32_t id = static_cast<uint32_t>(sp[u * G]);
+            const bool ok = !CHECK || left > u * G;
+            const float *gp = reinterpret_cast<const float *>(gb + static_cast<uint64_t>(id) * (ln.f * 4u));
+            rq[u] = ok ? V::raw(ln.row(qb, id)) : V::zero();
+#pragma unroll
+            for (int i = 0; i < VEC; i += 4) {
+                const float4 g4 = ok ? __ldg(reinterpret_cast<const float4 *>(gp + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                gr[u][i] = g4.x; gr[u][i + 1] = g4.y; gr[u][i + 2] = g4.z; gr[u][i + 3] = g4.w;
+            }
+            st[u] = ok ? __ldg(a.stats + ln.stat(id, a.heads)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        float *pk = dkv, *pv = dkv + VEC;
+#pragma unroll
+        for (int u = 0; u < D; ++u) {
+            float qv[VEC];
+            V::widen(rq[u], qv);
+            const float l = ln.head_sum(dw_dot(qv, ks)) * a.scale2;
+            const float da = ln.head_sum(dw_dot(gr[u], vs));
+            const bool ok = !CHECK || left > u * G;
+            const float al = ok ? exp2f(l - st[u].x) * st[u].y : 0.f;
+            const float wk = ok ? al * (da - st[u].z) : 0.f;
+            const float2 wk2 = make_float2(wk, wk), al2 = make_float2(al, al);
+#pragma unroll
+            for (int i = 0; i < VEC; i += 2) {
+                const float2 x = fma2(make_float2(qv[i], qv[i + 1]), wk2, make_float2(pk[i], pk[i + 1]));
+                const float2 y = fma2(make_float2(gr[u][i], gr[u][i + 1]), al2, make_float2(pv[i], pv[i + 1]));
+                pk[i] = x.x; pk[i + 1] = x.y;
+                pv[i] = y.x; pv[i + 1] = y.y;
+            }
+        }
+    }
+    template <bool CHECK>
+    __device__ __forceinline__ void add(const int32_t *ids, int cnt) {
+        held.next(dkv);
+        const int32_t *sp = ids + ln.g;
+#pragma unroll 1
+        for (; cnt >= G * kFull; cnt -= G * kFull, sp += G * kFull) step<kFull, false>(sp, 0);
+#pragma unroll 1
+        for (; CHECK && cnt > 0; cnt -= G * kPart, sp += G * kPart) step<kPart, true>(sp, cnt - ln.g);
+    }
+    template <class Get>
+    __device__ __forceinline__ void fold(Get get) {
+#pragma unroll
+        for (int i = 0; i < 2 * VEC; ++i) dkv[i] += get(dkv[i], i);
+    }
+    __device__ __forceinline__ void join() {
+        held.last(dkv);
+#pragma unroll
+        for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return __shfl_xor_sync(kFull, mine, o); });
+    }
+    __device__ __forceinline__ void merge(const float *slot) {
+        fold([&](float, int i) { return slot[i * LPR + ln.sub]; });
+    }
+    __device__ __forceinline__ void park(float *slot) const {
+        if (ln.g != 0) return;
+#pragma unroll
+        for (int i = 0; i < 2 * VEC; ++i) slot[i * LPR + ln.sub] = dkv[i];
+    }
+    __device__ __forceinline__ bool wants_after() const { return false; }
+    __device__ __forceinline__ void after(int, int32_t, int32_t, int32_t) {}
+    __device__ __forceinline__ void close(int32_t s, int32_t, int32_t, bool) {
+        if (ln.g != 0 || !ln.own) return;
+        float dk[VEC], dv[VEC];
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) {
+            dk[i] = dkv[i];
+            dv[i] = dkv[VEC + i];
+        }
+        dw_store(a.grad_k + ln.at(s), dk, a.scale);
+        dw_store(a.grad_v + ln.at(s), dv, 1.f);
+    }
+};
+
+// lh (a power of two up to 32, at most the lanes of a row) picks the kernel with
+// that many lanes per head.  PASS<XT, VEC, LPR, LH> is the policy.
+template <template <typename, int, int, int> class PASS, typename XT, int VEC, int LPR>
+cudaError_t launch_dot_lanes(const DotArgs &a, cudaStream_t s) {
+    switch (a.lh) {
+        case 1: return launch_walk<PASS<XT, VEC, LPR, 1>>(a, s);
+        case 2: return launch_walk<PASS<XT, VEC, LPR, 2>>(a, s);
+        case 4: return launch_walk<PASS<XT, VEC, LPR, 4>>(a, s);
+        case 8: return launch_walk<PASS<XT, VEC, LPR, 8>>(a, s);
+        default: return launch_walk<PASS<XT, VEC, LPR, 0>>(a, s);
+    }
+}
+template <template <typename, int, int, int> class PASS, typename XT, int VEC>
+cudaError_t launch_dot_pass(const DotArgs &a, cudaStream_t s) {
+    const int64_t slices = static_cast<int64_t>(a.heads) * a.channels / VEC;
+    if (slices > 16 || a.lh > 16) return launch_dot_lanes<PASS, XT, VEC, 32>(a, s);
+    if (slices > 8 || a.lh > 8) return launch_dot_lanes<PASS, XT, VEC, 16>(a, s);
+    return launch_dot_lanes<PASS, XT, VEC, 8>(a, s);
+}
+
+}  // namespace
+}  // namespace tfg

@@ -1,0 +1,12 @@
+// Backward of the dot-product attention by source (dot_walk.cuh): grad_k and
+// grad_v from the targets' statistics.
+#include "dot_walk.cuh"
+
+namespace tfg {
+
+cudaError_t launch_dot_walk_sources(const DotArgs &a, int x_dtype, cudaStream_t s) {
+    if (x_dtype == TFG_BF16) return launch_dot_pass<DotBySource, uint16_t, 8>(a, s);
+    return launch_dot_pass<DotBySource, float, 4>(a, s);
+}
+
+}  // namespace tfg

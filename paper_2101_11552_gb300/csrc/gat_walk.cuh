@@ -135,7 +135,7 @@ struct GatByTarget {
     using V = VecLoad<XT, VEC>;
     static constexpr int kWarps = TFG_GW_WARPS, kLpr = LPR, G = 32 / LPR;
     static constexpr int kTile = LPR * VEC * T, kHeadsPerLane = T;
-    static constexpr int kState = T * VEC + NH * (TARGET_BWD ? 3 : 2);
+    static constexpr int kState = T * VEC + NH * (TARGET_BWD ? 3 : 2), kHeld = 0;
     static constexpr int D = TFG_GW_DEPTH * G > 32 ? 32 / G : TFG_GW_DEPTH;   // gathers in flight per lane
     const GatArgs &a;
     GatLane<VEC, LPR, T, NH> at;
@@ -144,7 +144,7 @@ struct GatByTarget {
     float *scratch;                      // [warp][heads of the tile] (m, den), for alpha
     float sd[NH], m[NH], den[NH], phi[NH], acc[T][VEC];
 
-    __device__ __forceinline__ GatByTarget(const GatArgs &args, uint32_t ft, float *scr) : a(args), scratch(scr) {
+    __device__ __forceinline__ GatByTarget(const GatArgs &args, uint32_t ft, float *, float *scr) : a(args), scratch(scr) {
         at.place(ft, a.heads, a.channels);
         xb = reinterpret_cast<const char *>(static_cast<const XT *>(a.x) + (at.own > 0 ? at.f0 : 0));
         row_bytes = at.f * static_cast<uint32_t>(sizeof(XT));
@@ -413,7 +413,7 @@ struct GatBySource {
     using V = VecLoad<float, VEC>;
     static constexpr int kWarps = TFG_GW_SRC_WARPS, kLpr = LPR, G = 32 / LPR;
     static constexpr int kTile = LPR * VEC * T, kHeadsPerLane = T;
-    static constexpr int kState = 2 * T * VEC + NH;
+    static constexpr int kState = 2 * T * VEC + NH, kHeld = 0;
     static constexpr int D = TFG_GW_SRC_DEPTH * G > 32 ? 32 / G : TFG_GW_SRC_DEPTH;
     static constexpr int kUnroll = 32 / (G * D) < TFG_GW_SRC_UNROLL ? 32 / (G * D) : TFG_GW_SRC_UNROLL;
     const GatArgs &a;
@@ -422,7 +422,7 @@ struct GatBySource {
     uint32_t row_bytes;
     float ss[NH], sb[NH], P[T][VEC], Q[T][VEC];
 
-    __device__ __forceinline__ GatBySource(const GatArgs &args, uint32_t ft, float *) : a(args) {
+    __device__ __forceinline__ GatBySource(const GatArgs &args, uint32_t ft, float *, float *) : a(args) {
         at.place(ft, a.heads, a.channels);
         gb = reinterpret_cast<const char *>(a.grad_out + (at.own > 0 ? at.f0 : 0));
         row_bytes = at.f * 4u;
@@ -564,34 +564,6 @@ struct GatBySource {
         }
     }
 };
-
-template <class Policy>
-__global__ void __launch_bounds__(Policy::kWarps * 32, 1) gat_walk(GatArgs a) {
-    extern __shared__ __align__(16) float s_parts[];
-    __shared__ WalkShared<Policy::kWarps> s_walk;
-    const uint32_t f = static_cast<uint32_t>(a.heads) * static_cast<uint32_t>(a.channels);
-    for (uint32_t ft = blockIdx.y * Policy::kTile; ft < f; ft += gridDim.y * Policy::kTile) {
-        Policy p(a, ft, s_parts + 2 * Policy::kWarps * Policy::kState * Policy::kLpr);
-        walk_rows<Policy::kWarps>(a.rowptr, a.col, a.n, p, s_walk, s_parts);
-        __syncthreads();                   // before the next tile reuses the shared memory
-    }
-}
-
-template <class Policy>
-cudaError_t launch_walk(const GatArgs &a, cudaStream_t s) {
-    constexpr int parts = 2 * Policy::kWarps * Policy::kState * Policy::kLpr * static_cast<int>(sizeof(float));
-    constexpr int stats = Policy::kWarps * Policy::kLpr * Policy::kHeadsPerLane * static_cast<int>(sizeof(float2));
-    const int smem = parts + (a.alpha ? stats : 0);
-    if (smem > 32 * 1024) {   // with the static part above the 48 KB every launch may use
-        const cudaError_t err = cudaFuncSetAttribute(gat_walk<Policy>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     parts + stats);
-        if (err != cudaSuccess) return err;
-    }
-    const int64_t tiles = (static_cast<int64_t>(a.heads) * a.channels + Policy::kTile - 1) / Policy::kTile;
-    const dim3 grid(static_cast<unsigned>(min64(a.n, static_cast<int64_t>(sm_count()))), static_cast<unsigned>(min64(tiles, 65535)));
-    gat_walk<Policy><<<grid, Policy::kWarps * 32, smem, s>>>(a);
-    return cudaGetLastError();
-}
 
 }  // namespace
 }  // namespace tfg

@@ -33,6 +33,11 @@ struct WalkShared {
 
 constexpr int kWalkMinWork = 8;   // work (edges + kRowCost per row) a warp should have, at least
 
+// Gathers in flight per lane in a partial window of G lane groups: about 8 edges
+// a step, so that a row of a few edges does not pay for empty slots (100,000
+// nodes, 4 x 8 bf16, G = 4: 138 us with 4, 108 with 2).
+__host__ __device__ constexpr int walk_part(int g) { return g >= 8 ? 1 : (g >= 4 ? 2 : 4); }
+
 // parts: [2 * WARPS][kState * kLpr] floats of shared memory
 template <int WARPS, class P>
 __device__ __forceinline__ void walk_rows(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col,
@@ -117,6 +122,41 @@ __device__ __forceinline__ void walk_rows(const int32_t *__restrict__ rowptr, co
             if (r >= 0) p.after(w, r, __ldg(rowptr + r), __ldg(rowptr + r + 1));
         }
     }
+}
+
+// One CTA per SM of a policy's warps, a column of CTAs per feature tile.  Args has
+// rowptr, col, n, heads, channels and alpha (null: no attention weights wanted);
+// a policy is built from (args, the tile's first feature, kHeld floats a lane of
+// its warp's shared memory, the warps' statistics in shared memory).
+template <class Policy, class Args>
+__global__ void __launch_bounds__(Policy::kWarps * 32, 1) row_walk(Args a) {
+    extern __shared__ __align__(16) float s_parts[];
+    __shared__ WalkShared<Policy::kWarps> s_walk;
+    const uint32_t f = static_cast<uint32_t>(a.heads) * static_cast<uint32_t>(a.channels);
+    for (uint32_t ft = blockIdx.y * Policy::kTile; ft < f; ft += gridDim.y * Policy::kTile) {
+        float *held = s_parts + 2 * Policy::kWarps * Policy::kState * Policy::kLpr;
+        Policy p(a, ft, held + (threadIdx.x >> 5) * 32 * Policy::kHeld, held + Policy::kWarps * 32 * Policy::kHeld);
+        walk_rows<Policy::kWarps>(a.rowptr, a.col, a.n, p, s_walk, s_parts);
+        __syncthreads();                   // before the next tile reuses the shared memory
+    }
+}
+
+template <class Policy, class Args>
+cudaError_t launch_walk(const Args &a, cudaStream_t s) {
+    constexpr int parts = Policy::kWarps * (2 * Policy::kState * Policy::kLpr + 32 * Policy::kHeld) *
+                          static_cast<int>(sizeof(float));
+    constexpr int stats = Policy::kWarps * Policy::kLpr * Policy::kHeadsPerLane * static_cast<int>(sizeof(float2));
+    const int smem = parts + (a.alpha ? stats : 0);
+    if (smem > 32 * 1024) {   // with the static part above the 48 KB every launch may use
+        const cudaError_t err = cudaFuncSetAttribute(row_walk<Policy, Args>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     parts + stats);
+        if (err != cudaSuccess) return err;
+    }
+    const int64_t tiles = (static_cast<int64_t>(a.heads) * a.channels + Policy::kTile - 1) / Policy::kTile;
+    const dim3 grid(static_cast<unsigned>(min64(a.n, static_cast<int64_t>(sm_count()))),
+                    static_cast<unsigned>(min64(tiles, 65535)));
+    row_walk<Policy, Args><<<grid, Policy::kWarps * 32, smem, s>>>(a);
+    return cudaGetLastError();
 }
 
 }  // namespace tfg

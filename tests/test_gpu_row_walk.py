@@ -8,7 +8,7 @@ import torch
 
 import oracle
 from _helpers import (KAPPA_GAT, TOL_F32, assert_alpha_close, assert_exact_f32, assert_scaled_close,
-                      csr_rows, dev, features, gat_logit_mag, host_features)
+                      csr_rows, dev, dot_logit_mag, features, gat_logit_mag, host_features, kappa_dot)
 from paper_2101_11552_gb300 import graphgen as gg
 from paper_2101_11552_gb300 import tfg
 
@@ -105,3 +105,39 @@ def test_gat_layouts(heads, channels, dtype, more):
     tol = TOL_F32 + KAPPA_GAT * float(np.max(lam + lam_max[row]))
     for name, a, b, sc in zip(("grad_x", "grad_a_src", "grad_a_dst"), got, want[:3], want[3]):
         assert_scaled_close(a.cpu().numpy(), b, sc, tol, f"{name} {what}")
+
+
+@pytest.mark.parametrize("more", [0, 1000])     # mean in-degree 72 and 6
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("heads,channels", [(1, 8), (4, 8), (5, 8), (2, 16), (8, 16), (3, 32), (2, 64),
+                                            (1, 128), (1, 256), (16, 16)])
+def test_dot_layouts(heads, channels, dtype, more):
+    f = heads * channels
+    ei, n = graph(f + 1, more)
+    rng = np.random.default_rng(3000 + f)
+    wls = [gg.Workload("walk", n, ei, x, x_bf16=gg.bf16_bits_rne(x))
+           for x in rng.standard_normal((3, n, f), dtype=np.float32)]
+    (q, k, v), (qh, kh, vh) = ([features(w, dtype) for w in wls], [host_features(w, dtype) for w in wls])
+    scale = float(np.float32(1.0 / np.sqrt(channels)))
+    csr = tfg.tfg_build_csr(dev(ei), n)
+    out, alpha = tfg.tfg_dot_edge_softmax_aggregate(csr.rowptr, csr.col, q, k, v, heads, channels, scale,
+                                                    want_alpha=True)
+    ref, ref_alpha, sc = oracle.dot_softmax(ei, n, qh, kh, vh, heads, channels, scale)
+    what = f"{dtype} H={heads} C={channels} more={more}"
+    assert_scaled_close(out.cpu().numpy(), ref, sc, TOL_F32, "out " + what)
+    rowptr, col, perm, _ = oracle.build_csr(ei, n)
+    row = csr_rows(rowptr)
+    lam = dot_logit_mag(oracle.widen(qh), oracle.widen(kh), col, row, heads, channels, scale)
+    assert_alpha_close(alpha.cpu().numpy(), ref_alpha[perm], lam, row, kappa_dot(channels), "alpha " + what)
+    if not (32 % channels == 0 if channels <= 32 else channels % 32 == 0):
+        return
+    src = tfg.tfg_build_csr_by_source(dev(ei), n)
+    g = rng.standard_normal((n, f)).astype(np.float32)
+    got = tfg.tfg_dot_edge_softmax_aggregate_backward(csr.rowptr, csr.col, src.rowptr, src.col, q, k, v,
+                                                      heads, channels, scale, out, dev(g))
+    want = oracle.dot_softmax_backward(ei, n, qh, kh, vh, heads, channels, scale, g)
+    lam_max = np.zeros((n, heads))
+    np.maximum.at(lam_max, row, lam)
+    tol = TOL_F32 + kappa_dot(channels) * float(np.max(lam + lam_max[row]))
+    for name, a, b, s in zip(("grad_q", "grad_k", "grad_v"), got, want[:3], want[3]):
+        assert_scaled_close(a.cpu().numpy(), b, s, tol, f"{name} {what}")
