@@ -23,6 +23,9 @@ cudaError_t launch_kind(const AggArgs &a, int kind, cudaStream_t s) {
 
 }  // namespace
 
+cudaError_t launch_max_packed(const int32_t *rowptr, const int32_t *col, const void *x, int64_t n, int64_t f,
+                              float *out, cudaStream_t s);
+
 cudaError_t launch_aggregate(int mode, const int32_t *rowptr, const int32_t *col, const float *w,
                              const float *dinv, const void *x, int x_dtype, int64_t n, int64_t f,
                              int add_self, float fill, float *out, cudaStream_t s) {
@@ -32,6 +35,8 @@ cudaError_t launch_aggregate(int mode, const int32_t *rowptr, const int32_t *col
     const bool aligned = (reinterpret_cast<uintptr_t>(x) % 16 == 0) &&
                          (reinterpret_cast<uintptr_t>(out) % 16 == 0);
     if (x_dtype == TFG_BF16) {
+        if (kind == kMax && w == nullptr && aligned && f % 8 == 0)
+            return launch_max_packed(rowptr, col, x, n, f, out, s);
         if (aligned && f % 8 == 0) return launch_kind<uint16_t, 8>(a, kind, s);
         return launch_kind<uint16_t, 1>(a, kind, s);
     }

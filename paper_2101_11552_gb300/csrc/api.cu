@@ -35,11 +35,6 @@ struct NvtxRange {
 // win marks (backward.cu).
 namespace tfg {
 size_t max_backward_workspace_bytes(int64_t n, int64_t e, int64_t f);
-cudaError_t launch_max_backward_marked(const int32_t *rowptr_src, const int32_t *col_src,
-                                       const int32_t *perm_src, const int32_t *argmax,
-                                       const float *edge_weight, const float *grad_out, int64_t n,
-                                       int64_t e, int64_t f, float *grad_x, void *ws,
-                                       cudaStream_t s);
 cudaError_t launch_build_csr32(const int32_t *edge_index, int64_t e, int64_t n, int32_t *rowptr,
                                int32_t *col, int32_t *perm, int32_t *in_degree, void *ws,
                                int32_t *status, cudaStream_t s, bool by_source);
@@ -553,11 +548,8 @@ int tfg_aggregate_max_backward(const int32_t *rowptr_src, const int32_t *col_src
     const int32_t *col = num_edges > 0 ? col_src : nullptr;
     const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     return cuda_result(
-        need ? tfg::launch_max_backward_marked(rowptr_src, col, perm_src, argmax, edge_weight,
-                                               grad_out, num_nodes, num_edges, num_features, grad_x,
-                                               workspace, s)
-             : tfg::launch_max_backward(rowptr_src, col, perm_src, argmax, edge_weight, grad_out,
-                                        num_nodes, num_features, grad_x, s),
+        tfg::launch_max_backward(rowptr_src, col, perm_src, argmax, edge_weight, grad_out, num_nodes,
+                                 num_edges, num_features, grad_x, need ? workspace : nullptr, s),
         fn);
 }
 

@@ -22,6 +22,8 @@ struct DotArgs {
     const float *fwd_out, *grad_out;      // backward
     float4 *stats;                        // [N, H]: (m, 1 / den, beta, 0)
     float *grad_q, *grad_k, *grad_v;
+    __host__ __device__ uint32_t width() const { return static_cast<uint32_t>(heads) * static_cast<uint32_t>(channels); }
+    __host__ __device__ bool statistics() const { return alpha != nullptr; }
 };
 
 namespace {
@@ -205,7 +207,7 @@ struct DotByTarget {
         V::load(static_cast<const XT *>(a.q) + ln.at(t), qv);
         if (!ln.own) dw_clear(qv);
     }
-    __device__ __forceinline__ void open(int32_t t) {
+    __device__ __forceinline__ void open(int32_t t, int32_t, int32_t) {
         load_query(t);
         if constexpr (BWD) {
             float ov[VEC];
@@ -372,7 +374,7 @@ struct DotBySource {
         dw_clear(dkv);
         held.clear();
     }
-    __device__ __forceinline__ void open(int32_t s) {
+    __device__ __forceinline__ void open(int32_t s, int32_t, int32_t) {
         V::load(static_cast<const XT *>(a.k) + ln.at(s), ks);
         V::load(static_cast<const XT *>(a.v) + ln.at(s), vs);
         clear();

@@ -24,6 +24,8 @@ struct GatArgs {
     float4 *stats;                       // [N, H]: (s_dst, m, 1 / den, beta)
     float *ds_dst, *ds_src, *grad_x;
     const float *a_src, *a_dst;          // backward by source
+    __host__ __device__ uint32_t width() const { return static_cast<uint32_t>(heads) * static_cast<uint32_t>(channels); }
+    __host__ __device__ bool statistics() const { return alpha != nullptr; }
 };
 
 namespace {
@@ -160,7 +162,7 @@ struct GatByTarget {
 #pragma unroll
             for (int q = 0; q < VEC; ++q) acc[i][q] = 0.f;
     }
-    __device__ __forceinline__ void open(int32_t t) {
+    __device__ __forceinline__ void open(int32_t t, int32_t, int32_t) {
 #pragma unroll
         for (int i = 0; i < NH; ++i)
             sd[i] = __ldg(a.s_dst + static_cast<uint64_t>(static_cast<uint32_t>(t)) * a.heads + at.head[i]);
@@ -435,7 +437,7 @@ struct GatBySource {
 #pragma unroll
             for (int q = 0; q < VEC; ++q) P[i][q] = Q[i][q] = 0.f;
     }
-    __device__ __forceinline__ void open(int32_t s) {
+    __device__ __forceinline__ void open(int32_t s, int32_t, int32_t) {
 #pragma unroll
         for (int i = 0; i < NH; ++i)
             ss[i] = __ldg(a.s_src + static_cast<uint64_t>(static_cast<uint32_t>(s)) * a.heads + at.head[i]);

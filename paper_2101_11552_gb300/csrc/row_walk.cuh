@@ -7,7 +7,9 @@
 //
 // A policy P holds one lane's state of one row and provides
 //   kLpr, kState          lanes per row, floats a lane parks for another warp
-//   open(t)               start row t (loads what the row needs, clears the state)
+//   open(t, k, beg)       start row t at edge k; its first edge is beg (loads what the
+//                         row needs, clears the state)
+//   clear()               the empty state
 //   add<CHECK>(ids, cnt)  edges ids[0 .. cnt) (whole warp; ids in shared memory,
 //                         readable up to 32 entries past them)
 //   join()                combine the warp's lane groups (every lane ends with
@@ -76,7 +78,7 @@ __device__ __forceinline__ void walk_rows(const int32_t *__restrict__ rowptr, co
         int rem = rend - k;
         k = rend;
         if (closes || rem > 0) {
-            p.open(t);
+            p.open(t, rend - rem, rbeg);
             while (rem > 0) {
                 if (j == 32) {
                     next_window();
@@ -110,10 +112,11 @@ __device__ __forceinline__ void walk_rows(const int32_t *__restrict__ rowptr, co
     if (hr >= 0) {                                          // earlier parts in warp order, then ours
         int first = warp;
         while (first > 0 && s.tail_row[first - 1] == hr) --first;
-        p.open(hr);
+        const int32_t beg = __ldg(rowptr + hr);
+        p.open(hr, beg, beg);
         for (int w = first; w < warp; ++w) p.merge(parts + w * kSlot);
         p.merge(parts + (WARPS + warp) * kSlot);
-        p.close(hr, __ldg(rowptr + hr), __ldg(rowptr + hr + 1), true);
+        p.close(hr, beg, __ldg(rowptr + hr + 1), true);
     }
     if (p.wants_after()) {
         __syncthreads();
@@ -125,17 +128,21 @@ __device__ __forceinline__ void walk_rows(const int32_t *__restrict__ rowptr, co
 }
 
 // One CTA per SM of a policy's warps, a column of CTAs per feature tile.  Args has
-// rowptr, col, n, heads, channels and alpha (null: no attention weights wanted);
-// a policy is built from (args, the tile's first feature, kHeld floats a lane of
-// its warp's shared memory, the warps' statistics in shared memory).
+// rowptr, col, n, width() (features of a row) and statistics() (whether the warps'
+// statistics are wanted).  A policy is built from (args, the tile's first feature,
+// kHeld floats a lane of its warp's shared memory or, when kHeld is 0, the warp's
+// parking slot, which is free until the walk ends, the warps' statistics in
+// shared memory).
 template <class Policy, class Args>
 __global__ void __launch_bounds__(Policy::kWarps * 32, 1) row_walk(Args a) {
     extern __shared__ __align__(16) float s_parts[];
     __shared__ WalkShared<Policy::kWarps> s_walk;
-    const uint32_t f = static_cast<uint32_t>(a.heads) * static_cast<uint32_t>(a.channels);
+    const uint32_t f = a.width();
     for (uint32_t ft = blockIdx.y * Policy::kTile; ft < f; ft += gridDim.y * Policy::kTile) {
         float *held = s_parts + 2 * Policy::kWarps * Policy::kState * Policy::kLpr;
-        Policy p(a, ft, held + (threadIdx.x >> 5) * 32 * Policy::kHeld, held + Policy::kWarps * 32 * Policy::kHeld);
+        const int warp = threadIdx.x >> 5;
+        float *own = Policy::kHeld > 0 ? held + warp * 32 * Policy::kHeld : s_parts + warp * Policy::kState * Policy::kLpr;
+        Policy p(a, ft, own, held + Policy::kWarps * 32 * Policy::kHeld);
         walk_rows<Policy::kWarps>(a.rowptr, a.col, a.n, p, s_walk, s_parts);
         __syncthreads();                   // before the next tile reuses the shared memory
     }
@@ -146,13 +153,13 @@ cudaError_t launch_walk(const Args &a, cudaStream_t s) {
     constexpr int parts = Policy::kWarps * (2 * Policy::kState * Policy::kLpr + 32 * Policy::kHeld) *
                           static_cast<int>(sizeof(float));
     constexpr int stats = Policy::kWarps * Policy::kLpr * Policy::kHeadsPerLane * static_cast<int>(sizeof(float2));
-    const int smem = parts + (a.alpha ? stats : 0);
+    const int smem = parts + (a.statistics() ? stats : 0);
     if (smem > 32 * 1024) {   // with the static part above the 48 KB every launch may use
         const cudaError_t err = cudaFuncSetAttribute(row_walk<Policy, Args>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                      parts + stats);
         if (err != cudaSuccess) return err;
     }
-    const int64_t tiles = (static_cast<int64_t>(a.heads) * a.channels + Policy::kTile - 1) / Policy::kTile;
+    const int64_t tiles = (static_cast<int64_t>(a.width()) + Policy::kTile - 1) / Policy::kTile;
     const dim3 grid(static_cast<unsigned>(min64(a.n, static_cast<int64_t>(sm_count()))),
                     static_cast<unsigned>(min64(tiles, 65535)));
     row_walk<Policy, Args><<<grid, Policy::kWarps * 32, smem, s>>>(a);

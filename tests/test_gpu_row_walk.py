@@ -141,3 +141,37 @@ def test_dot_layouts(heads, channels, dtype, more):
     tol = TOL_F32 + kappa_dot(channels) * float(np.max(lam + lam_max[row]))
     for name, a, b, s in zip(("grad_q", "grad_k", "grad_v"), got, want[:3], want[3]):
         assert_scaled_close(a.cpu().numpy(), b, s, tol, f"{name} {what}")
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("f", [3, 8, 16, 24, 40, 41, 64, 72, 100, 128, 136, 256, 264])
+def test_max_argmax_widths(f, dtype):
+    """Argmax where the layout changes, weighted and not, with values that tie."""
+    ei, n = graph(f + 2, 300)
+    rng = np.random.default_rng(4000 + f)
+    x = np.round(rng.standard_normal((n, f), dtype=np.float32) * 4) / 4
+    wl = gg.Workload("walk", n, ei, x, x_bf16=gg.bf16_bits_rne(x))
+    csr = tfg.tfg_build_csr(dev(ei), n)
+    for ew in (None, rng.uniform(-1.5, 1.5, ei.shape[1]).astype(np.float32)):
+        w = None if ew is None else dev(ew).index_select(0, csr.perm)
+        out, arg = tfg.tfg_aggregate_max_argmax(csr, features(wl, dtype), w)
+        ref, ref_arg = oracle.max_argmax(ei, n, host_features(wl, dtype), ew)
+        assert np.array_equal(arg.cpu().numpy(), ref_arg), f"argmax F={f}"
+        assert_exact_f32(out.cpu().numpy(), ref, f"max F={f}")
+
+
+def test_max_argmax_of_a_row_past_16_bit_positions():
+    """A target of 3,000,000 edges: each warp's share exceeds the 65,000 edges that
+    16-bit positions cover; the maximum sits first, last and twice in the row."""
+    n, e, f = 40, 3_000_000, 24
+    rng = np.random.default_rng(5)
+    ei = np.stack([rng.integers(8, n, size=e), np.zeros(e, np.int64)])
+    ei[0, [0, e // 3, e - 1]] = [1, 2, 3]
+    x = rng.standard_normal((n, f), dtype=np.float32)
+    x[1, :6], x[2, 4:12], x[3, 8:18] = 9.0, 9.0, 9.0
+    wl = gg.Workload("star", n, ei, x, x_bf16=gg.bf16_bits_rne(x))
+    csr = tfg.tfg_build_csr(dev(ei), n)
+    out, arg = tfg.tfg_aggregate_max_argmax(csr, features(wl, "bf16"))
+    ref, ref_arg = oracle.max_argmax(ei, n, host_features(wl, "bf16"), None)
+    assert np.array_equal(arg.cpu().numpy(), ref_arg)
+    assert_exact_f32(out.cpu().numpy(), ref)
