@@ -565,9 +565,20 @@ cudaError_t walk_targets(const GatArgs &a, cudaStream_t s) {
     if (slices <= 16) return launch_walk<GatByTarget<XT, VEC, 16, 1, 1, true>>(a, s);
     return launch_walk<GatByTarget<XT, VEC, 32, 1, 1, true>>(a, s);
 }
+// 32-byte gradient slices pay on long rows only: they take fewer, register-rich
+// warps.  8 x 16 bf16, 32- / 16-byte slices, us: mean degree 492 (114.6M edges) 4685 /
+// 5418, 100 (20M) 1025 / 1018, 50 664 / 594, 16 367 / 272; 4 x 16 fp32 at 100 566 / 586,
+// at 50 399 / 394.
+#ifndef TFG_GW_WIDE_DEGREE
+#define TFG_GW_WIDE_DEGREE 128
+#endif
 template <typename XT>
-cudaError_t walk_sources(const GatArgs &a, cudaStream_t s) {
+cudaError_t walk_sources(const GatArgs &a, int64_t e, cudaStream_t s) {
     const int slices = a.heads * a.channels / 4;
+    if (e >= TFG_GW_WIDE_DEGREE * a.n && slices > 8 && a.channels % 8 == 0 && reinterpret_cast<uintptr_t>(a.grad_out) % 32 == 0) {
+        if (slices <= 16) return launch_walk<GatBySource<XT, 8, 8, 1, 1>>(a, s);
+        return launch_walk<GatBySource<XT, 8, 16, 1, 1>>(a, s);
+    }
     if (slices <= 8) return launch_walk<GatBySource<XT, 4, 8, 1, 1>>(a, s);
     if (slices <= 16) return launch_walk<GatBySource<XT, 4, 16, 1, 1>>(a, s);
     return launch_walk<GatBySource<XT, 4, 32, 1, 1>>(a, s);
@@ -698,7 +709,7 @@ cudaError_t launch_edge_softmax_backward(const int32_t *rowptr, const int32_t *c
         if (err != cudaSuccess) return err;
         ga.rowptr = rowptr_src;
         ga.col = col_src;
-        err = bf16 ? walk_sources<uint16_t>(ga, s) : walk_sources<float>(ga, s);
+        err = bf16 ? walk_sources<uint16_t>(ga, e, s) : walk_sources<float>(ga, e, s);
         if (err != cudaSuccess) return err;
         if (bf16)
             return launch_vectors(static_cast<const uint16_t *>(x), n, heads, channels, buf[7], buf[6],

@@ -65,6 +65,29 @@ __device__ __forceinline__ uint4 ld_row16(const void *p) {
 #endif
 }
 
+// A 32-byte slice of a gathered fp32 row (p 32-byte aligned) in one load, so that
+// lanes side by side fill whole 128-byte lines; zeros where ok is false.
+struct Row32 {
+    float v[8];
+};
+__device__ __forceinline__ Row32 ld_row32(const float *p) {
+    Row32 r;
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3]), "=f"(r.v[4]), "=f"(r.v[5]), "=f"(r.v[6]), "=f"(r.v[7])
+        : "l"(p));
+    return r;
+}
+__device__ __forceinline__ Row32 ld_row32(bool ok, const float *p) {
+    Row32 r;
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %9, 0;\n\t"
+        "mov.b32 %0, 0;\n\tmov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\tmov.b32 %3, 0;\n\t"
+        "mov.b32 %4, 0;\n\tmov.b32 %5, 0;\n\tmov.b32 %6, 0;\n\tmov.b32 %7, 0;\n\t"
+        "@p ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t}"
+        : "=&f"(r.v[0]), "=&f"(r.v[1]), "=&f"(r.v[2]), "=&f"(r.v[3]), "=&f"(r.v[4]), "=&f"(r.v[5]), "=&f"(r.v[6]), "=&f"(r.v[7])
+        : "l"(p), "r"(static_cast<int>(ok)));
+    return r;
+}
+
 // VEC consecutive features of one row: a raw load (kept packed in registers
 // while the load is in flight) and its widening to fp32.
 template <typename XT, int VEC> struct VecLoad;
@@ -81,6 +104,22 @@ template <> struct VecLoad<float, 4> {
         v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
     }
     static __device__ __forceinline__ void load(const float *p, float (&v)[4]) { widen(raw(p), v); }
+};
+template <> struct VecLoad<float, 8> {
+    using Raw = Row32;
+    static __device__ __forceinline__ Raw raw(const float *p) { return ld_row32(p); }   // p 32-byte aligned
+    static __device__ __forceinline__ Raw raw(bool ok, const float *p) { return ld_row32(ok, p); }
+    static __device__ __forceinline__ void widen(const Raw &q, float (&v)[8]) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = q.v[i];
+    }
+    static __device__ __forceinline__ void load(const float *p, float (&v)[8]) {        // p 16-byte aligned
+#pragma unroll
+        for (int i = 0; i < 8; i += 4) {
+            const float4 q = __ldg(reinterpret_cast<const float4 *>(p + i));
+            v[i] = q.x; v[i + 1] = q.y; v[i + 2] = q.z; v[i + 3] = q.w;
+        }
+    }
 };
 template <> struct VecLoad<float, 1> {
     using Raw = float;

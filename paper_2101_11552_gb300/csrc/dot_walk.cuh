@@ -183,6 +183,7 @@ struct DotByTarget {
     static constexpr int kTile = LPR * VEC, kHeadsPerLane = 1;
     static constexpr int kState = VEC + 2, kHeld = VEC;
     static constexpr int kFull = TFG_DW_DEPTH * G > 32 ? 32 / G : TFG_DW_DEPTH, kUnroll = TFG_DW_UNROLL;
+    static_assert(32 % (G * kFull) == 0, "a full window is read in whole steps");
     static constexpr int kPart = walk_part(G) < kFull ? walk_part(G) : kFull;
     const DotArgs &a;
     L ln;
@@ -350,14 +351,17 @@ struct DotByTarget {
 // Backward by source (CSR by source: ids are targets), from the targets'
 // statistics: grad_k = scale sum of alpha (dalpha - beta) q[t], grad_v = sum of
 // alpha grad_out[t].
-template <typename XT, int VEC, int LPR, int LH>
-struct DotBySource {
+// WIDE (VEC = 8): 32-byte gradient slices, one load each instead of two that each
+// touch every sector: 114.6M edges 7.49 ms against 7.59.
+template <typename XT, int VEC, int LPR, int LH, bool WIDE>
+struct DotSource {
     using L = DotLane<XT, VEC, LPR, LH>;
     using V = VecLoad<XT, VEC>;
     static constexpr int kWarps = TFG_DW_SRC_WARPS, kLpr = LPR, G = 32 / LPR;
     static constexpr int kTile = LPR * VEC, kHeadsPerLane = 1;
     static constexpr int kState = 2 * VEC, kHeld = 2 * VEC;
     static constexpr int kFull = TFG_DW_DEPTH * G > 32 ? 32 / G : TFG_DW_DEPTH;
+    static_assert(32 % (G * kFull) == 0, "a full window is read in whole steps");
     static constexpr int kPart = walk_part(G) < kFull ? walk_part(G) : kFull;
     const DotArgs &a;
     L ln;
@@ -365,7 +369,7 @@ struct DotBySource {
     DotHeld<2 * VEC> held;
     float ks[VEC], vs[VEC], dkv[2 * VEC];  // grad_k's and grad_v's sums
 
-    __device__ __forceinline__ DotBySource(const DotArgs &args, uint32_t ft, float *hold, float *)
+    __device__ __forceinline__ DotSource(const DotArgs &args, uint32_t ft, float *hold, float *)
         : a(args), ln(args, ft), held(hold) {
         qb = ln.base(a.q);
         gb = reinterpret_cast<const char *>(a.grad_out + ln.f0);
@@ -390,6 +394,11 @@ struct DotBySource {
             const bool ok = !CHECK || left > u * G;
             const float *gp = reinterpret_cast<const float *>(gb + static_cast<uint64_t>(id) * (ln.f * 4u));
             rq[u] = ok ? V::raw(ln.row(qb, id)) : V::zero();
+            if constexpr (WIDE) {
+                const Row32 g8 = CHECK ? ld_row32(ok, gp) : ld_row32(gp);
+#pragma unroll
+                for (int i = 0; i < VEC; ++i) gr[u][i] = g8.v[i];
+            } else
 #pragma unroll
             for (int i = 0; i < VEC; i += 4) {
                 const float4 g4 = ok ? __ldg(reinterpret_cast<const float4 *>(gp + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -458,6 +467,12 @@ struct DotBySource {
         dw_store(a.grad_v + ln.at(s), dv, 1.f);
     }
 };
+
+template <typename XT, int VEC, int LPR, int LH>
+using DotBySource = DotSource<XT, VEC, LPR, LH, VEC == 8>;
+// gradient rows that are not 32-byte aligned: one kernel a row width, heads at run time
+template <typename XT, int VEC, int LPR, int LH>
+using DotBySourceNarrow = DotSource<XT, VEC, LPR, 0, false>;
 
 // lh (a power of two up to 32, at most the lanes of a row) picks the kernel with
 // that many lanes per head.  PASS<XT, VEC, LPR, LH> is the policy.

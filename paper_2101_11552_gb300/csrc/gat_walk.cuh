@@ -33,7 +33,8 @@ namespace {
 // What bounds it: instructions on short rows (169,343 nodes, mean in-degree 6.9, 8
 // x 16 fp32: forward 145, by target 164, by source 161 us, against 36-45 us for
 // the gathered bytes at the L2 rate), the gathers and the weights' arithmetic on
-// long ones (by source at 114.6M edges: 640 bytes an edge, 5.43 ms, 13.5 TB/s;
+// long ones (by source at 114.6M edges: 640 bytes an edge, 4.69 ms, 15.6 TB/s;
+// 5.42 ms with 16-byte slices;
 // 7.93 ms when each edge's dot product was finished by a butterfly).  One head of
 // 41 channels on the first graph, alpha written: 1,753 us in a row-per-warp
 // kernel whose hub rows one warp walked, 196 us.
@@ -56,6 +57,15 @@ namespace {
 // 5.53 ms, 2: 6.12, 8: 5.43 at 114.6M edges).
 #ifndef TFG_GW_SRC_DEPTH
 #define TFG_GW_SRC_DEPTH 4
+#endif
+// By source with 32-byte gradient slices (VEC = 8: half the lanes a row, so an edge's
+// weight is formed by half as many lanes, and twice the bytes a load): 114.6M edges
+// 4.69 ms with 16 warps and 4 in flight, 20 and 4 4.86, 24 and 2 5.98, 12 and 4 5.45.
+#ifndef TFG_GW_SRC8_WARPS
+#define TFG_GW_SRC8_WARPS 16
+#endif
+#ifndef TFG_GW_SRC8_DEPTH
+#define TFG_GW_SRC8_DEPTH 4
 #endif
 #ifndef TFG_GW_SRC_UNROLL
 #define TFG_GW_SRC_UNROLL 8
@@ -139,6 +149,7 @@ struct GatByTarget {
     static constexpr int kTile = LPR * VEC * T, kHeadsPerLane = T;
     static constexpr int kState = T * VEC + NH * (TARGET_BWD ? 3 : 2), kHeld = 0;
     static constexpr int D = TFG_GW_DEPTH * G > 32 ? 32 / G : TFG_GW_DEPTH;   // gathers in flight per lane
+    static_assert(32 % (G * D) == 0, "a full window is read in whole steps");
     const GatArgs &a;
     GatLane<VEC, LPR, T, NH> at;
     const char *xb;
@@ -413,10 +424,12 @@ struct GatByTarget {
 template <typename XT, int VEC, int LPR, int T, int NH>
 struct GatBySource {
     using V = VecLoad<float, VEC>;
-    static constexpr int kWarps = TFG_GW_SRC_WARPS, kLpr = LPR, G = 32 / LPR;
+    static constexpr int kWarps = VEC == 8 ? TFG_GW_SRC8_WARPS : TFG_GW_SRC_WARPS, kLpr = LPR, G = 32 / LPR;
     static constexpr int kTile = LPR * VEC * T, kHeadsPerLane = T;
     static constexpr int kState = 2 * T * VEC + NH, kHeld = 0;
-    static constexpr int D = TFG_GW_SRC_DEPTH * G > 32 ? 32 / G : TFG_GW_SRC_DEPTH;
+    static constexpr int kDepth = VEC == 8 ? TFG_GW_SRC8_DEPTH : TFG_GW_SRC_DEPTH;
+    static constexpr int D = kDepth * G > 32 ? 32 / G : kDepth;
+    static_assert(32 % (G * D) == 0, "a full window is read in whole steps");
     static constexpr int kUnroll = 32 / (G * D) < TFG_GW_SRC_UNROLL ? 32 / (G * D) : TFG_GW_SRC_UNROLL;
     const GatArgs &a;
     GatLane<VEC, LPR, T, NH> at;
@@ -468,8 +481,11 @@ struct GatBySource {
                     st[u][i] = ok ? __ldg(a.stats + static_cast<uint64_t>(id) * a.heads + at.head[i])
                                   : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                for (int i = 0; i < T; ++i)
-                    raw[u][i] = (T == 1 ? ok : ok && i < at.own) ? V::raw(row + i * LPR * VEC) : V::zero();
+                for (int i = 0; i < T; ++i) {
+                    const bool on = T == 1 ? ok : ok && i < at.own;
+                    if constexpr (VEC == 8) raw[u][i] = CHECK || T > 1 ? V::raw(on, row + i * LPR * VEC) : V::raw(row + i * LPR * VEC);
+                    else raw[u][i] = on ? V::raw(row + i * LPR * VEC) : V::zero();
+                }
             }
 #pragma unroll
             for (int u = 0; u < D; ++u) {

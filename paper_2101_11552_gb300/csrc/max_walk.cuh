@@ -73,6 +73,7 @@ struct MaxByTarget {
     static constexpr int kTile = LPR * VEC * T, kHeadsPerLane = T;
     static constexpr int kState = (ARG ? 2 : 1) * T * VEC, kHeld = 0;
     static constexpr int kFull = TFG_MW_DEPTH * G > 32 ? 32 / G : TFG_MW_DEPTH;
+    static_assert(32 % (G * kFull) == 0, "a full window is read in whole steps");
     static constexpr int kPart = walk_part(G) < kFull ? walk_part(G) : kFull;
     static constexpr int kPairs = PACKED ? VEC / 2 : 1;
     static constexpr int kReach = 65000;          // edges that 16-bit positions cover
@@ -358,6 +359,7 @@ struct MaxBwdArgs {
 template <int VEC, int T>
 struct MaxBySource {
     static constexpr int kWarps = T > 2 ? 28 : TFG_MXA_WARPS, kLpr = 32, D = TFG_MXA_DEPTH;
+    static_assert(32 % D == 0, "a full window is read in whole steps");
     static constexpr int kTile = 32 * VEC * T, kHeadsPerLane = 1;
     static constexpr int kState = T * VEC, kHeld = 0;
     const MaxBwdArgs &a;

@@ -175,3 +175,49 @@ def test_max_argmax_of_a_row_past_16_bit_positions():
     ref, ref_arg = oracle.max_argmax(ei, n, host_features(wl, "bf16"), None)
     assert np.array_equal(arg.cpu().numpy(), ref_arg)
     assert_exact_f32(out.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("offset", [0, 4, 8])   # floats before grad_out: 32-byte aligned, 16, 32
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("heads,channels", [(4, 8), (5, 8), (8, 8), (3, 16), (8, 16), (1, 64), (1, 128)])
+def test_gradient_slices_of_32_bytes(heads, channels, dtype, offset):
+    """Backward by source of both attentions on rows of mean degree 206, with
+    gradients that 32-byte loads may and may not read."""
+    f = heads * channels
+    rng = np.random.default_rng(6000 + f)
+    deg = np.array(DEGREES[:16] + [3, 0, 7] * 10)
+    n = len(deg)
+    ei = np.stack([np.repeat(np.arange(n), deg), rng.integers(0, n, size=deg.sum())]).astype(np.int64)
+    wls = [gg.Workload("walk", n, ei, x, x_bf16=gg.bf16_bits_rne(x))
+           for x in rng.standard_normal((3, n, f), dtype=np.float32)]
+    (q, k, v), (qh, kh, vh) = ([features(w, dtype) for w in wls], [host_features(w, dtype) for w in wls])
+    a_s, a_d = (0.5 * rng.standard_normal((2, f))).astype(np.float32)
+    g = rng.standard_normal((n, f)).astype(np.float32)
+    gd = torch.empty(offset + n * f, device="cuda")[offset:].view(n, f)
+    gd.copy_(dev(g))
+    csr, src = tfg.tfg_build_csr(dev(ei), n), tfg.tfg_build_csr_by_source(dev(ei), n)
+    rowptr, col, _, _ = oracle.build_csr(ei, n)
+    row = csr_rows(rowptr)
+
+    def check(names, got, want, lam, kappa):
+        lam_max = np.zeros((n, heads))
+        np.maximum.at(lam_max, row, lam)
+        tol = TOL_F32 + kappa * float(np.max(lam + lam_max[row]))
+        for name, a, b, s in zip(names, got, want[:3], want[3]):
+            assert_scaled_close(a.cpu().numpy(), b, s, tol, f"{name} {dtype} H={heads} C={channels}")
+
+    out, _ = tfg.tfg_edge_softmax_aggregate(csr.rowptr, csr.col, q, heads, channels, dev(a_s), dev(a_d), 0.2,
+                                            want_alpha=True)
+    got = tfg.tfg_edge_softmax_aggregate_backward(csr.rowptr, csr.col, src.rowptr, src.col, q, heads,
+                                                  channels, dev(a_s), dev(a_d), 0.2, out, gd)
+    check(("grad_x", "grad_a_src", "grad_a_dst"), got,
+          oracle.edge_softmax_backward(ei, n, qh, heads, channels, a_s, a_d, 0.2, g),
+          gat_logit_mag(oracle.widen(qh), col, row, heads, channels, a_s, a_d), KAPPA_GAT)
+    scale = float(np.float32(1.0 / np.sqrt(channels)))
+    out, _ = tfg.tfg_dot_edge_softmax_aggregate(csr.rowptr, csr.col, q, k, v, heads, channels, scale,
+                                                want_alpha=True)
+    got = tfg.tfg_dot_edge_softmax_aggregate_backward(csr.rowptr, csr.col, src.rowptr, src.col, q, k, v,
+                                                      heads, channels, scale, out, gd)
+    check(("grad_q", "grad_k", "grad_v"), got,
+          oracle.dot_softmax_backward(ei, n, qh, kh, vh, heads, channels, scale, g),
+          dot_logit_mag(oracle.widen(qh), oracle.widen(kh), col, row, heads, channels, scale), kappa_dot(channels))
