@@ -197,18 +197,6 @@ __device__ __forceinline__ int64_t first_row_at(const int32_t *rowptr, int64_t n
     return lo;
 }
 
-// Last t in [lo, hi] with rowptr[t] + t <= q (rowptr[lo] + lo <= q holds):
-// the row open at merge coordinate q; q - t is the CSR position reached.
-__device__ __forceinline__ int32_t last_row_at(const int32_t *rowptr, int32_t lo, int32_t hi,
-                                               int64_t q) {
-    while (lo < hi) {
-        const int32_t mid = lo + (hi - lo + 1) / 2;
-        if (static_cast<int64_t>(__ldg(rowptr + mid)) + mid <= q) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
 __device__ __forceinline__ void balanced_rows(const int32_t *rowptr, int64_t n, int64_t nb,
                                               int64_t b, int64_t &r0, int64_t &r1) {
     const int64_t total = static_cast<int64_t>(__ldg(rowptr + n)) + n;

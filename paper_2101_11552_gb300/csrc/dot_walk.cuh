@@ -30,7 +30,7 @@ namespace {
 
 // What bounds it: instructions on short rows (169,343 nodes, mean in-degree 6.9, 8
 // x 16 fp32: forward 166, by target 206, by source 253 us); on long ones (114.6M
-// edges, 8 x 16 bf16) the gathers, 896 bytes an edge by source (7.6 ms, 13.5 TB/s)
+// edges, 8 x 16 bf16) the gathers, 896 bytes an edge by source (7.5 ms, 13.7 TB/s)
 // and 512 by target (5.4 ms, 11 TB/s), with one CTA of few, register-rich warps.
 // Before: a row per warp, the lanes of a head a run-time count and every slot
 // tested, 141 instructions for two edges by source: 12.4 ms, by target 8.9 ms.

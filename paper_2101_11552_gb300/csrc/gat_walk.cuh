@@ -33,11 +33,10 @@ namespace {
 // What bounds it: instructions on short rows (169,343 nodes, mean in-degree 6.9, 8
 // x 16 fp32: forward 145, by target 164, by source 161 us, against 36-45 us for
 // the gathered bytes at the L2 rate), the gathers and the weights' arithmetic on
-// long ones (by source at 114.6M edges: 640 bytes an edge, 4.69 ms, 15.6 TB/s;
-// 5.42 ms with 16-byte slices;
-// 7.93 ms when each edge's dot product was finished by a butterfly).  One head of
-// 41 channels on the first graph, alpha written: 1,753 us in a row-per-warp
-// kernel whose hub rows one warp walked, 196 us.
+// long ones (by source at 114.6M edges: 640 bytes an edge, 4.69 ms, 15.6 TB/s, 5.42
+// ms with 16-byte slices, 7.93 ms when each edge's dot product was finished by a
+// butterfly).  One head of 41 channels on the first graph, alpha written: 196 us;
+// 1,753 in a row-per-warp kernel whose hub rows one warp walked.
 //
 // Tuning knobs.  Warps per CTA (one CTA per SM), measured on the two graphs:
 // by target 28 (forward 146 us / 2.68 ms), 24 160 / 2.84, 32 136 / 2.64; by source

@@ -334,7 +334,7 @@ struct MaxBwdArgs {
     const float *grad_out;
     int64_t n, f, e;
     float *grad_x;
-    const uint8_t *mark;                  // bit j of mark[e]: edge e wins a feature of group j (null: no marks)
+    const uint8_t *mark;                  // max_bwd_kernel: bit j of mark[e] when edge e wins a feature of group j
     int group;                            // features per group, a multiple of 4
     __host__ __device__ uint32_t width() const { return static_cast<uint32_t>(f); }
     __host__ __device__ bool statistics() const { return false; }
