@@ -62,7 +62,12 @@ def csr_passes(n: int) -> int:
 
 def launches_per_step(n: int, e: int) -> int:
     """Kernels libtfg launches in one step (fixed by the launch plan)."""
-    build = (csr_passes(n) * 5 if e > 0 else 0) + 2   # per pass: upsweep, 3 scan, downsweep
+    # per pass: upsweep, 2 scan kernels (3 above 1,024 chunks of counters), downsweep
+    bits = max(1, (n - 1).bit_length())
+    width = -(-bits // csr_passes(n))
+    chunks = -(-(-(-e // 4096) << width) // 4096)
+    large = chunks > 1024                             # scan_top and degree_from_rowptr of their own
+    build = (csr_passes(n) * (4 + large) if e > 0 else 0) + 1 + large
     norm = 1                                          # dinv only
     gcn = 1
     softmax = 2                                       # node scores + aggregate

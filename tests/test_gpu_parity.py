@@ -452,3 +452,19 @@ def test_deterministic_bitwise():
                                                dev(np.ones(128, np.float32)), 0.2, want_alpha=True)
         runs.append([np_(t).tobytes() for t in (csr.col, csr.perm, dinv, a, b, al)])
     assert runs[0] == runs[1]
+
+
+@pytest.mark.parametrize("n,e", [(1, 7), (254, 900), (255, 900), (256, 900), (510, 40), (300, 70_000),
+                                 (600, 8_380_000), (600, 8_400_000)])
+def test_csr_scan_and_row_ends(n, e):
+    """Row counts around a CTA's 255 rows, and counters around the 1,024 chunks
+    that the scan sums without a kernel of its own (10-bit digits: 8.39M edges)."""
+    rng = np.random.default_rng(n + e)
+    ei = rng.integers(0, n, size=(2, e)).astype(np.int64)
+    csr = tfg.tfg_build_csr(torch.from_numpy(ei).cuda(), n)
+    order = np.argsort(ei[1], kind="stable")
+    deg = np.bincount(ei[1], minlength=n)
+    assert np.array_equal(csr.perm.cpu().numpy(), order)
+    assert np.array_equal(csr.col.cpu().numpy(), ei[0][order])
+    assert np.array_equal(csr.in_degree.cpu().numpy(), deg)
+    assert np.array_equal(csr.rowptr.cpu().numpy(), np.concatenate([[0], np.cumsum(deg)]))
