@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kAggThreads, 1) aggregate_rows(AggArgs a) {
         };
         for (;;) {
             const bool closes = t < tb;
-            const int32_t rend = closes ? __shfl_sync(kFull, rwin, tl) : kb;
+            const int32_t rend = closes ? lane_get(rwin, tl) : kb;
             typename V::Raw xt[T];
             typename V0::Raw x0t[T];
             if (S::kGcnLike) load(xt, row(static_cast<uint32_t>(t)), self && closes);   // what the row end
@@ -348,10 +348,10 @@ __global__ void __launch_bounds__(kAggThreads, 1) aggregate_rows(AggArgs a) {
                 for (int i = 0; i < T; ++i)
 #pragma unroll
                     for (int q = 0; q < VEC; ++q)
-                        acc[i][q] = S::combine(acc[i][q], __shfl_xor_sync(kFull, acc[i][q], s));
+                        acc[i][q] = S::combine(acc[i][q], lane_xor(acc[i][q], s));
             if (!closes) break;
             float c1f = 0.f, c2f = 1.f;
-            if (S::kGcnLike) S::factors(a, __shfl_sync(kFull, dwin, tl), c1f, c2f);
+            if (S::kGcnLike) S::factors(a, lane_get(dwin, tl), c1f, c2f);
             if (t == sh.ta && sh.head_split) {             // parts of it sit with earlier warps
                 if (g == 0) {
 #pragma unroll

@@ -52,12 +52,12 @@ __device__ __forceinline__ void head_sums(float (&v)[NT], int channels) {
     if (channels <= 32) {
 #pragma unroll
         for (int i = 0; i < NT; ++i)
-            for (int o = 1; o < channels; o <<= 1) v[i] += __shfl_xor_sync(kFull, v[i], o);
+            for (int o = 1; o < channels; o <<= 1) v[i] += lane_xor(v[i], o);
     } else {
 #pragma unroll
         for (int i = 0; i < NT; ++i)
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) v[i] += __shfl_xor_sync(kFull, v[i], o);
+            for (int o = 1; o < 32; o <<= 1) v[i] += lane_xor(v[i], o);
         const int per = channels / 32;             // tiles per head
         float tot[NT];
 #pragma unroll
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kBwThreads) bwd_targets(BwArgs a) {
             float l[kBwUnroll][NT];
 #pragma unroll
             for (int u = 0; u < kBwUnroll; ++u) {
-                const int64_t s = __shfl_sync(kFull, c, (j + u) & 31);
+                const int64_t s = lane_get(c, (j + u) & 31);
 #pragma unroll
                 for (int i = 0; i < NT; ++i)
                     l[u][i] = bw_leaky(__ldg(a.s_src + s * a.heads + hd[i]) + sd[i], a.slope);
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(kBwThreads) bwd_targets(BwArgs a) {
             float d[kBwUnroll][NT], z[kBwUnroll][NT];
 #pragma unroll
             for (int u = 0; u < kBwUnroll; ++u) {
-                const int64_t s = __shfl_sync(kFull, c, (j + u) & 31);
+                const int64_t s = lane_get(c, (j + u) & 31);
 #pragma unroll
                 for (int i = 0; i < NT; ++i) {
                     float xv[1] = {0.f};
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kBwThreads) bwd_sources(BwArgs a) {
                 dt[kBwUnrollSrc][NT], bt[kBwUnrollSrc][NT];
 #pragma unroll
             for (int u = 0; u < kBwUnrollSrc; ++u) {
-                const int64_t t = __shfl_sync(kFull, c, (j + u) & 31);
+                const int64_t t = lane_get(c, (j + u) & 31);
 #pragma unroll
                 for (int i = 0; i < NT; ++i) {
                     const int64_t th = t * a.heads + hd[i];

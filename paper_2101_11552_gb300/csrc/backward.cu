@@ -127,7 +127,7 @@ struct MaxBwd {
             const float wc = weight_of(a, mk, ec);
             const bool win = mk != 0;
             // the chunk's edges that may contribute, D at a time in chunk order
-            for (uint32_t m = __ballot_sync(kFull, win); m != 0;) {
+            for (uint32_t m = lane_ballot(win); m != 0;) {
                 int at[D];                                  // the edges' lanes in the chunk
                 int32_t am[D][VEC];                         // -2: no edge's id
                 float gv[D][VEC];
@@ -136,8 +136,8 @@ struct MaxBwd {
                     const bool any = m != 0;
                     at[d] = any ? __ffs(m) - 1 : 0;
                     m &= m - 1;
-                    const uint32_t t = static_cast<uint32_t>(__shfl_sync(kFull, c, at[d]));
-                    const bool ok = any && (__shfl_sync(kFull, mk, at[d]) & my_bit) != 0;   // per lane
+                    const uint32_t t = static_cast<uint32_t>(lane_get(c, at[d]));
+                    const bool ok = any && (lane_get(mk, at[d]) & my_bit) != 0;   // per lane
                     const uint64_t from = static_cast<uint64_t>(t) * f + fl;
                     if constexpr (VEC == 4) {
                         const int4 v = ok ? __ldg(reinterpret_cast<const int4 *>(a.argmax + from)) : make_int4(-2, -2, -2, -2);
@@ -152,8 +152,8 @@ struct MaxBwd {
                 }
 #pragma unroll
                 for (int d = 0; d < D; ++d) {
-                    const int32_t ed = __shfl_sync(kFull, ec, at[d]);
-                    const float we = a.w ? __shfl_sync(kFull, wc, at[d]) : 1.f;
+                    const int32_t ed = lane_get(ec, at[d]);
+                    const float we = a.w ? lane_get(wc, at[d]) : 1.f;
 #pragma unroll
                     for (int q = 0; q < VEC; ++q)
                         if (am[d][q] == ed) acc[q] = fmaf(we, gv[d][q], acc[q]);
@@ -225,13 +225,13 @@ __global__ void __launch_bounds__(kMxThreads, MASKED ? TFG_MXB_MINB : 4) max_bwd
     for (;;) {
         int i = 0;
         if (lane == 0) i = atomicAdd(&s_next, 1);
-        i = __shfl_sync(kFull, i, 0);
+        i = lane_get(i, 0);
         if (i >= nrows) break;
         const int64_t s = r0 + i;
         if (a.col != nullptr && a.rowptr[s + 1] - a.rowptr[s] > kMxHeavyDeg) {
             int slot = 0;
             if (lane == 0) slot = atomicAdd(&s_nheavy, 1);
-            slot = __shfl_sync(kFull, slot, 0);
+            slot = lane_get(slot, 0);
             if (slot < kMxMaxHeavy) {
                 if (lane == 0) s_heavy[slot] = s;
                 continue;

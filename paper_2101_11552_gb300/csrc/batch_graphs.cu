@@ -44,7 +44,7 @@ scan_counts(const int64_t *__restrict__ node_counts, const int64_t *__restrict__
         for (int a = 0; a < 2; ++a) {
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int64_t y = __shfl_up_sync(kFull, incl[a], o);
+                const int64_t y = lane_up(incl[a], o);
                 if (lane >= o) incl[a] += y;
             }
             if (lane == 31) s_w[a][warp] = incl[a];
@@ -57,7 +57,7 @@ scan_counts(const int64_t *__restrict__ node_counts, const int64_t *__restrict__
                 int64_t si = s;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
-                    const int64_t y = __shfl_up_sync(kFull, si, o);
+                    const int64_t y = lane_up(si, o);
                     if (lane >= o) si += y;
                 }
                 s_w[a][lane] = si - s;

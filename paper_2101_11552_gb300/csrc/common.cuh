@@ -8,7 +8,19 @@
 
 namespace tfg {
 
-constexpr unsigned kFull = 0xffffffffu;
+constexpr unsigned kAllLanes = 0xffffffffu;
+
+// Exchanges between all 32 lanes of a warp.  The mask is named here and nowhere else: a
+// call that passed one by name would take a constant of its own class before this one,
+// and an exchange that leaves executing lanes out of its mask is undefined.
+template <typename T>
+__device__ __forceinline__ T lane_get(T v, int from) { return __shfl_sync(kAllLanes, v, from); }
+template <typename T>
+__device__ __forceinline__ T lane_xor(T v, int mask) { return __shfl_xor_sync(kAllLanes, v, mask); }
+template <typename T>
+__device__ __forceinline__ T lane_up(T v, unsigned by) { return __shfl_up_sync(kAllLanes, v, by); }
+__device__ __forceinline__ unsigned lane_ballot(bool v) { return __ballot_sync(kAllLanes, v); }
+__device__ __forceinline__ bool lane_any(bool v) { return __any_sync(kAllLanes, v) != 0; }
 
 // First error wins: a kernel that finds bad data records its code once.
 __device__ __forceinline__ void set_status(int32_t *status, int32_t code) {
@@ -218,7 +230,7 @@ __device__ __forceinline__ void for_each_row(const int32_t *rowptr, int64_t n, R
     for (;;) {
         int i = 0;
         if (lane == 0) i = atomicAdd(&s_next, 1);
-        i = __shfl_sync(kFull, i, 0);
+        i = lane_get(i, 0);
         if (i >= r1 - r0) break;
         fn(r0 + i, lane);
     }

@@ -24,7 +24,7 @@
 namespace tfg {
 namespace {
 
-constexpr int kTile = 4096;                       // edges per CTA tile
+constexpr int kSortTile = 4096;                   // edges per CTA tile
 constexpr int kMaxDigitBits = 10;
 constexpr int kUpThreads = 256;
 constexpr int kScanThreads = 256;
@@ -72,8 +72,8 @@ radix_upsweep(const IdT *__restrict__ dst64, const uint32_t *__restrict__ key32,
     const int radix = 1 << width;
     for (int d = threadIdx.x; d < radix; d += kUpThreads) s_cnt[d] = 0;
     __syncthreads();
-    const int64_t base = static_cast<int64_t>(blockIdx.x) * kTile;
-    const int64_t stop = min64(e, base + kTile);
+    const int64_t base = static_cast<int64_t>(blockIdx.x) * kSortTile;
+    const int64_t stop = min64(e, base + kSortTile);
     for (int64_t i = base + threadIdx.x; i < stop; i += kUpThreads) {
         uint32_t key = FIRST ? checked_id(__ldg(dst64 + i), n, status) : __ldg(key32 + i);
         atomicAdd(&s_cnt[(key >> shift) & (radix - 1)], 1);
@@ -98,7 +98,7 @@ __device__ int32_t block_exclusive_scan(int32_t v, int32_t *total) {
     int32_t incl = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const int32_t y = __shfl_up_sync(kFull, incl, o);
+        const int32_t y = lane_up(incl, o);
         if (lane >= o) incl += y;
     }
     if (lane == 31) warp_sums[warp] = incl;
@@ -108,7 +108,7 @@ __device__ int32_t block_exclusive_scan(int32_t v, int32_t *total) {
         int32_t si = s;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(kFull, si, o);
+            const int32_t y = lane_up(si, o);
             if (lane >= o) si += y;
         }
         if (lane < kScanThreads / 32) warp_sums[lane] = si - s;
@@ -130,7 +130,7 @@ scan_reduce(const int32_t *__restrict__ data, int64_t m, int32_t *__restrict__ s
         if (k < m) s += data[k];
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+    for (int o = 16; o > 0; o >>= 1) s += lane_xor(s, o);
     __shared__ int32_t ws[kScanThreads / 32];
     if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
     __syncthreads();
@@ -163,7 +163,7 @@ __device__ int32_t block_sum(const int32_t *__restrict__ sums, int n) {
     int32_t s = 0;
     for (int k = threadIdx.x; k < n; k += kScanThreads) s += __ldg(sums + k);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+    for (int o = 16; o > 0; o >>= 1) s += lane_xor(s, o);
     if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
     __syncthreads();
     s = 0;
@@ -211,7 +211,7 @@ scan_down(int32_t *data, int64_t m, const int32_t *__restrict__ sums) {
 
 // chunks of the counters of e edges at a digit width
 int64_t scan_chunks(int64_t e, int width) {
-    return (((e + kTile - 1) / kTile << width) + kScanChunk - 1) / kScanChunk;
+    return (((e + kSortTile - 1) / kSortTile << width) + kScanChunk - 1) / kScanChunk;
 }
 
 cudaError_t exclusive_scan(int32_t *data, int64_t m, int32_t *sums, cudaStream_t s) {
@@ -247,10 +247,10 @@ cudaError_t exclusive_scan(int32_t *data, int64_t m, int32_t *sums, cudaStream_t
 constexpr bool kDsFullTiles = TFG_DS_FULL_TILES != 0;
 constexpr int kDsWarps = 16;
 constexpr int kDsThreads = kDsWarps * 32;
-constexpr int kDsItems = kTile / kDsThreads;   // 8 per lane
+constexpr int kDsItems = kSortTile / kDsThreads;   // 8 per lane
 
 size_t downsweep_smem(int radix) {
-    return sizeof(uint32_t) * 3 * kTile + sizeof(int32_t) * kDsWarps * radix +
+    return sizeof(uint32_t) * 3 * kSortTile + sizeof(int32_t) * kDsWarps * radix +
            sizeof(int32_t) * 2 * radix + sizeof(int32_t) * 32;
 }
 
@@ -258,20 +258,20 @@ size_t downsweep_smem(int radix) {
 // 2^bits: one ballot per bit (measured faster here than __match_any_sync).
 __device__ __forceinline__ unsigned peers_from_bit(unsigned peers, uint32_t dig, int b) {
     const bool set = (dig >> b) & 1u;
-    const unsigned bal = __ballot_sync(kFull, set);
+    const unsigned bal = lane_ballot(set);
     return peers & (set ? bal : ~bal);
 }
 
 template <int BITS>   // bit count known at compile time: the loop unrolls
 __device__ __forceinline__ unsigned same_digit_lanes(uint32_t dig) {
-    unsigned peers = kFull;
+    unsigned peers = kAllLanes;
 #pragma unroll
     for (int b = 0; b < BITS; ++b) peers = peers_from_bit(peers, dig, b);
     return peers;
 }
 
 __device__ __forceinline__ unsigned same_digit_lanes(uint32_t dig, int bits) {
-    unsigned peers = kFull;
+    unsigned peers = kAllLanes;
 #pragma unroll 1
     for (int b = 0; b < bits; ++b) peers = peers_from_bit(peers, dig, b);
     return peers;
@@ -291,15 +291,15 @@ radix_downsweep(const IdT *__restrict__ src64, const IdT *__restrict__ dst64,
     const int width = W > 0 ? W : width_arg;
     const int radix = 1 << width;
     uint32_t *s_key = reinterpret_cast<uint32_t *>(smem);                 // [tile]
-    int32_t *s_src = reinterpret_cast<int32_t *>(s_key + kTile);           // [tile]
-    int32_t *s_eid = s_src + kTile;                                        // [tile]
-    int32_t *s_cnt = s_eid + kTile;                                        // [warp][digit]
+    int32_t *s_src = reinterpret_cast<int32_t *>(s_key + kSortTile);       // [tile]
+    int32_t *s_eid = s_src + kSortTile;                                    // [tile]
+    int32_t *s_cnt = s_eid + kSortTile;                                        // [warp][digit]
     int32_t *s_tstart = s_cnt + kDsWarps * radix;                          // [digit]
     int32_t *s_delta = s_tstart + radix;                                   // [digit]
     int32_t *s_chunk = s_delta + radix;                                    // [32]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t tile0 = static_cast<int64_t>(blockIdx.x) * kTile;
-    const int count = static_cast<int>(min64(kTile, e - tile0));
+    const int64_t tile0 = static_cast<int64_t>(blockIdx.x) * kSortTile;
+    const int count = static_cast<int>(min64(kSortTile, e - tile0));
     // every tile but the last is full: its copy of the code has no bounds tests
     auto run = [&](auto full_tag) {
         constexpr bool FULL = decltype(full_tag)::value;
@@ -351,7 +351,7 @@ radix_downsweep(const IdT *__restrict__ src64, const IdT *__restrict__ dst64,
                 base = mine[dig];
                 mine[dig] = base + __popc(peers);
             }
-            base = __shfl_sync(kFull, base, leader);
+            base = lane_get(base, leader);
             const uint32_t rk = static_cast<uint32_t>(base + __popc(peers & lower));
             if (r < 4) rank_lo |= rk << (8 * r);
             else rank_hi |= rk << (8 * (r - 4));
@@ -380,7 +380,7 @@ radix_downsweep(const IdT *__restrict__ src64, const IdT *__restrict__ dst64,
             int32_t incl = v;
     #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int32_t y = __shfl_up_sync(kFull, incl, o);
+                const int32_t y = lane_up(incl, o);
                 if (lane >= o) incl += y;
             }
             if (d < radix) s_tstart[d] = incl - v;
@@ -392,7 +392,7 @@ radix_downsweep(const IdT *__restrict__ src64, const IdT *__restrict__ dst64,
             int32_t incl = v;
     #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int32_t y = __shfl_up_sync(kFull, incl, o);
+                const int32_t y = lane_up(incl, o);
                 if (lane >= o) incl += y;
             }
             if (lane < chunks) s_chunk[lane] = incl - v;
@@ -434,7 +434,7 @@ radix_downsweep(const IdT *__restrict__ src64, const IdT *__restrict__ dst64,
             }
         }
     };
-    if (kDsFullTiles && count == kTile) run(std::true_type{});
+    if (kDsFullTiles && count == kSortTile) run(std::true_type{});
     else run(std::false_type{});
 }
 
@@ -496,7 +496,7 @@ DownsweepFn<IdT> downsweep_for(int width) {
 size_t csr_workspace_bytes(int64_t n, int64_t e) {
     if (e <= 0) return 256;
     const SortPlan p = plan_for(n);
-    const int64_t tiles = ceil_div(e, kTile);
+    const int64_t tiles = ceil_div(e, kSortTile);
     const int64_t radix = int64_t(1) << p.width;
     const size_t a = align256(sizeof(int32_t) * 3 * size_t(e));
     const size_t b = align256(sizeof(int32_t) * (p.passes >= 3 ? 3 : 1) * size_t(e));
@@ -515,7 +515,7 @@ cudaError_t build_csr_impl(const IdT *edge_index, int64_t e, int64_t n, int32_t 
     const uint32_t *sorted_keys = nullptr;
     if (e > 0) {
         const SortPlan p = plan_for(n);
-        const int tiles = ceil_div(e, kTile);
+        const int tiles = ceil_div(e, kSortTile);
         const int radix = 1 << p.width;
         char *w = static_cast<char *>(ws);
         struct Buf { uint32_t *key; int32_t *src; int32_t *eid; } buf[2];

@@ -61,7 +61,7 @@ __device__ __forceinline__ void dot_rows(const int32_t *rowptr, int64_t n, RowFn
     for (;;) {
         int i = 0;
         if (lane == 0) i = atomicAdd(&s_next, 1);
-        i = __shfl_sync(kFull, i, 0);
+        i = lane_get(i, 0);
         if (i >= r1 - r0) break;
         fn(r0 + i, lane);
     }
@@ -132,7 +132,7 @@ __device__ __forceinline__ void dot_fast_row(const DotArgs &a, int lh_arg, int64
                 for (int u = 0; u < kDotUnroll; ++u) {
                     const int k = j + u * G + g;
                     const uint64_t off = static_cast<uint64_t>(
-                        static_cast<uint32_t>(__shfl_sync(kFull, c, k & 31))) * row_bytes;
+                        static_cast<uint32_t>(lane_get(c, k & 31))) * row_bytes;
                     ok[u] = FULL || k < cnt;
                     rk[u] = ok[u] ? V::raw(reinterpret_cast<const XT *>(kb + off)) : V::zero();
                     rv[u] = ok[u] ? V::raw(reinterpret_cast<const XT *>(vb + off)) : V::zero();
@@ -145,7 +145,7 @@ __device__ __forceinline__ void dot_fast_row(const DotArgs &a, int lh_arg, int64
                     V::widen(rk[u], kv);
                     float d = dw_dot(qv, kv);
 #pragma unroll
-                    for (int o = 1; o < lh; o <<= 1) d += __shfl_xor_sync(kFull, d, o);
+                    for (int o = 1; o < lh; o <<= 1) d += lane_xor(d, o);
                     l[u] = ok[u] ? d * a.scale2 : -CUDART_INF_F;
                     mc = fmaxf(mc, l[u]);
                 }
@@ -185,14 +185,14 @@ __device__ __forceinline__ void dot_fast_row(const DotArgs &a, int lh_arg, int64
         // merge the G groups' states in a fixed butterfly order
 #pragma unroll
         for (int s = LPR; s < 32; s <<= 1) {
-            const float mo = __shfl_xor_sync(kFull, m, s);
-            const float dn = __shfl_xor_sync(kFull, den, s);
+            const float mo = lane_xor(m, s);
+            const float dn = lane_xor(den, s);
             const float mm = fmaxf(m, mo);
             const float x = dw_rescale(m, mm), y = dw_rescale(mo, mm);
             den = den * x + dn * y;
 #pragma unroll
             for (int q = 0; q < VEC; ++q) {
-                const float ao = __shfl_xor_sync(kFull, acc[q], s);
+                const float ao = lane_xor(acc[q], s);
                 acc[q] = acc[q] * x + ao * y;
             }
             m = mm;
@@ -212,7 +212,7 @@ __device__ __forceinline__ void dot_fast_row(const DotArgs &a, int lh_arg, int64
                 float kv[VEC];
                 V::load(kp + src * f + fl, kv);
                 float d = dw_dot(qv, kv);
-                for (int o = 1; o < lh; o <<= 1) d += __shfl_xor_sync(kFull, d, o);
+                for (int o = 1; o < lh; o <<= 1) d += lane_xor(d, o);
                 if (ok && fok && sub % lh == 0)
                     a.alpha[k * a.heads + h] = exp2f(d * a.scale2 - m) / den;
             }
@@ -250,7 +250,7 @@ __device__ __forceinline__ void dot_general_row(const DotArgs &a, int64_t t, int
 #pragma unroll
             for (int j = 0; j < NCH; ++j) part[j] = 0.f;
             for (int e = 0; e < cnt; ++e) {
-                const int64_t src = __shfl_sync(kFull, c, e);
+                const int64_t src = lane_get(c, e);
                 float kv[NCH], vv[NCH];
 #pragma unroll
                 for (int j = 0; j < NCH; ++j) {
@@ -267,7 +267,7 @@ __device__ __forceinline__ void dot_general_row(const DotArgs &a, int64_t t, int
 #pragma unroll
                 for (int j = 0; j < NCH; ++j) d = fmaf(qv[j], kv[j], d);
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) d += __shfl_xor_sync(kFull, d, o);
+                for (int o = 1; o < 32; o <<= 1) d += lane_xor(d, o);
                 const float l = d * a.scale2;
                 if (l > m) {
                     const float sc = dot_rescale(m, l);
@@ -306,7 +306,7 @@ __device__ __forceinline__ void dot_general_row(const DotArgs &a, int64_t t, int
                     d = fmaf(qv[j], x[0], d);
                 }
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) d += __shfl_xor_sync(kFull, d, o);
+                for (int o = 1; o < 32; o <<= 1) d += lane_xor(d, o);
                 if (lane == 0) a.alpha[k * a.heads + h] = exp2f(d * a.scale2 - m) / den;
             }
         }

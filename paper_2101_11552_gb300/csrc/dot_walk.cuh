@@ -116,9 +116,9 @@ struct DotLane {
     __device__ __forceinline__ float head_sum(float v) const {
         if constexpr (LH > 0) {
 #pragma unroll
-            for (int o = 1; o < LH; o <<= 1) v += __shfl_xor_sync(kFull, v, o);
+            for (int o = 1; o < LH; o <<= 1) v += lane_xor(v, o);
         } else {
-            for (int o = 1; o < lh; o <<= 1) v += __shfl_xor_sync(kFull, v, o);
+            for (int o = 1; o < lh; o <<= 1) v += lane_xor(v, o);
         }
         return v;
     }
@@ -182,9 +182,9 @@ struct DotByTarget {
     static constexpr int kWarps = BWD ? TFG_DW_TGT_WARPS : TFG_DW_FWD_WARPS, kLpr = LPR, G = 32 / LPR;
     static constexpr int kTile = LPR * VEC, kHeadsPerLane = 1;
     static constexpr int kState = VEC + 2, kHeld = VEC;
-    static constexpr int kFull = TFG_DW_DEPTH * G > 32 ? 32 / G : TFG_DW_DEPTH, kUnroll = TFG_DW_UNROLL;
-    static_assert(32 % (G * kFull) == 0, "a full window is read in whole steps");
-    static constexpr int kPart = walk_part(G) < kFull ? walk_part(G) : kFull;
+    static constexpr int kStepFull = TFG_DW_DEPTH * G > 32 ? 32 / G : TFG_DW_DEPTH, kUnroll = TFG_DW_UNROLL;
+    static_assert(32 % (G * kStepFull) == 0, "a full window is read in whole steps");
+    static constexpr int kStepPart = walk_part(G) < kStepFull ? walk_part(G) : kStepFull;
     const DotArgs &a;
     L ln;
     const char *kb, *vb;
@@ -268,14 +268,14 @@ struct DotByTarget {
         const int32_t *sp = ids + ln.g;
         if (!CHECK) {                                            // a full window
 #pragma unroll kUnroll
-            for (int e = 0; e < 32; e += G * kFull) step<kFull, false>(sp + e, 0, dpart);
+            for (int e = 0; e < 32; e += G * kStepFull) step<kStepFull, false>(sp + e, 0, dpart);
             den += dpart;
             return;
         }
 #pragma unroll 1
-        for (; cnt >= G * kFull; cnt -= G * kFull, sp += G * kFull) step<kFull, false>(sp, 0, dpart);
+        for (; cnt >= G * kStepFull; cnt -= G * kStepFull, sp += G * kStepFull) step<kStepFull, false>(sp, 0, dpart);
 #pragma unroll 1
-        for (; CHECK && cnt > 0; cnt -= G * kPart, sp += G * kPart) step<kPart, true>(sp, cnt - ln.g, dpart);
+        for (; CHECK && cnt > 0; cnt -= G * kStepPart, sp += G * kStepPart) step<kStepPart, true>(sp, cnt - ln.g, dpart);
         den += dpart;
     }
     template <class Get>
@@ -290,7 +290,7 @@ struct DotByTarget {
     __device__ __forceinline__ void join() {
         held.last(acc);
 #pragma unroll
-        for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return __shfl_xor_sync(kFull, mine, o); });
+        for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return lane_xor(mine, o); });
     }
     __device__ __forceinline__ void merge(const float *slot) {
         fold([&](float, int i) { return slot[i * LPR + ln.sub]; });
@@ -360,9 +360,9 @@ struct DotSource {
     static constexpr int kWarps = TFG_DW_SRC_WARPS, kLpr = LPR, G = 32 / LPR;
     static constexpr int kTile = LPR * VEC, kHeadsPerLane = 1;
     static constexpr int kState = 2 * VEC, kHeld = 2 * VEC;
-    static constexpr int kFull = TFG_DW_DEPTH * G > 32 ? 32 / G : TFG_DW_DEPTH;
-    static_assert(32 % (G * kFull) == 0, "a full window is read in whole steps");
-    static constexpr int kPart = walk_part(G) < kFull ? walk_part(G) : kFull;
+    static constexpr int kStepFull = TFG_DW_DEPTH * G > 32 ? 32 / G : TFG_DW_DEPTH;
+    static_assert(32 % (G * kStepFull) == 0, "a full window is read in whole steps");
+    static constexpr int kStepPart = walk_part(G) < kStepFull ? walk_part(G) : kStepFull;
     const DotArgs &a;
     L ln;
     const char *qb, *gb;
@@ -431,9 +431,9 @@ struct DotSource {
         held.next(dkv);
         const int32_t *sp = ids + ln.g;
 #pragma unroll 1
-        for (; cnt >= G * kFull; cnt -= G * kFull, sp += G * kFull) step<kFull, false>(sp, 0);
+        for (; cnt >= G * kStepFull; cnt -= G * kStepFull, sp += G * kStepFull) step<kStepFull, false>(sp, 0);
 #pragma unroll 1
-        for (; CHECK && cnt > 0; cnt -= G * kPart, sp += G * kPart) step<kPart, true>(sp, cnt - ln.g);
+        for (; CHECK && cnt > 0; cnt -= G * kStepPart, sp += G * kStepPart) step<kStepPart, true>(sp, cnt - ln.g);
     }
     template <class Get>
     __device__ __forceinline__ void fold(Get get) {
@@ -443,7 +443,7 @@ struct DotSource {
     __device__ __forceinline__ void join() {
         held.last(dkv);
 #pragma unroll
-        for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return __shfl_xor_sync(kFull, mine, o); });
+        for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return lane_xor(mine, o); });
     }
     __device__ __forceinline__ void merge(const float *slot) {
         fold([&](float, int i) { return slot[i * LPR + ln.sub]; });

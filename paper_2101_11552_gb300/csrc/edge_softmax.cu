@@ -178,7 +178,7 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
         typename V::Raw raw0[kSmUnroll];
 #pragma unroll
         for (int u = 0; u < kSmUnroll; ++u)
-            raw0[u] = gather(static_cast<uint32_t>(__shfl_sync(kFull, c, (u * G + g) & 31)));
+            raw0[u] = gather(static_cast<uint32_t>(lane_get(c, (u * G + g) & 31)));
         float p[R];
         float cm = -CUDART_INF_F;
 #pragma unroll
@@ -187,19 +187,19 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
 #if TFG_SM_PREFETCH >= 2
             const float ss = sv[r];                  // gathered during the previous chunk
 #else
-            const float ss = __ldg(s_src + static_cast<int64_t>(__shfl_sync(kFull, c, k)) * H + sh);
+            const float ss = __ldg(s_src + static_cast<int64_t>(lane_get(c, k)) * H + sh);
 #endif
             p[r] = (FULL || k < cnt) ? leaky(ss + sd, slope) : -CUDART_INF_F;
             cm = fmaxf(cm, p[r]);
         }
 #pragma unroll
-        for (int o = H; o < 32; o <<= 1) cm = fmaxf(cm, __shfl_xor_sync(kFull, cm, o));
+        for (int o = H; o < 32; o <<= 1) cm = fmaxf(cm, lane_xor(cm, o));
         const bool rises = cm > m;
-        if (__any_sync(kFull, rises)) {   // warp-uniform; rare after the first chunks
+        if (lane_any(rises)) {   // warp-uniform; rare after the first chunks
             const float sc = rises ? (m == -CUDART_INF_F ? 0.f : exp2f(m - cm)) : 1.f;
             den *= sc;
             if (BWD) ph *= sc;
-            const float fsc = __shfl_sync(kFull, sc, fh);   // lane fh scores head fh
+            const float fsc = lane_get(sc, fh);   // lane fh scores head fh
 #pragma unroll
             for (int q = 0; q < VEC; ++q) acc[q] *= fsc;
             m = fmaxf(m, cm);
@@ -221,7 +221,7 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
         // the next chunk's node scores, requested before this chunk's rows
 #pragma unroll
         for (int r = 0; r < R; ++r)
-            sv[r] = __ldg(s_src + static_cast<int64_t>(__shfl_sync(kFull, cnext, r * ES + se)) * H + sh);
+            sv[r] = __ldg(s_src + static_cast<int64_t>(lane_get(cnext, r * ES + se)) * H + sh);
 #endif
         float part[VEC];
 #pragma unroll
@@ -236,9 +236,9 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
                 const int k0 = e + u * G;              // edge of group 0 in this step
                 const int k = k0 + g;
                 // p of (edge k, head fh) sits in lane (k % ES) * H + fh, register k / ES
-                pw[u] = __shfl_sync(kFull, p[k0 / ES], ((k0 % ES) + g) * H + fh);
+                pw[u] = lane_get(p[k0 / ES], ((k0 % ES) + g) * H + fh);
                 if (e == 0) raw[u] = raw0[u];
-                else raw[u] = gather(static_cast<uint32_t>(__shfl_sync(kFull, c, k & 31)));
+                else raw[u] = gather(static_cast<uint32_t>(lane_get(c, k & 31)));
             }
 #pragma unroll
             for (int u = 0; u < kSmUnroll; ++u) {
@@ -269,7 +269,7 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
 #if TFG_SM_PREFETCH >= 2
 #pragma unroll
     for (int r = 0; r < R; ++r)
-        sv[r] = __ldg(s_src + static_cast<int64_t>(__shfl_sync(kFull, cnext, r * ES + se)) * H + sh);
+        sv[r] = __ldg(s_src + static_cast<int64_t>(lane_get(cnext, r * ES + se)) * H + sh);
 #endif
     for (int64_t base = beg; base < end; base += 32) {
         const int cnt = static_cast<int>(min64(32, end - base));
@@ -283,16 +283,16 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
         else chunk(std::false_type{}, c, cnt);
     }
 #pragma unroll
-    for (int o = H; o < 32; o <<= 1) den += __shfl_xor_sync(kFull, den, o);
+    for (int o = H; o < 32; o <<= 1) den += lane_xor(den, o);
 #pragma unroll
     for (int o = LPR; o < 32; o <<= 1)
 #pragma unroll
-        for (int q = 0; q < VEC; ++q) acc[q] += __shfl_xor_sync(kFull, acc[q], o);
-    const float dh = __shfl_sync(kFull, den, fh);   // lane fh holds head fh's denominator
+        for (int q = 0; q < VEC; ++q) acc[q] += lane_xor(acc[q], o);
+    const float dh = lane_get(den, fh);   // lane fh holds head fh's denominator
     if constexpr (BWD) {
 #pragma unroll
-        for (int o = H; o < 32; o <<= 1) ph += __shfl_xor_sync(kFull, ph, o);
-        const float phh = __shfl_sync(kFull, ph, fh), mh = __shfl_sync(kFull, m, fh), sdh = __shfl_sync(kFull, sd, fh);
+        for (int o = H; o < 32; o <<= 1) ph += lane_xor(ph, o);
+        const float phh = lane_get(ph, fh), mh = lane_get(m, fh), sdh = lane_get(sd, fh);
         float b = 0.f, d = 0.f;
         if (fok) {
             float gv[VEC], ov[VEC];
@@ -305,8 +305,8 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
             }
         }
         for (int o = 1; o < channels / VEC; o <<= 1) {
-            b += __shfl_xor_sync(kFull, b, o);
-            d += __shfl_xor_sync(kFull, d, o);
+            b += lane_xor(b, o);
+            d += lane_xor(d, o);
         }
         if (lane < LPR && fok && f0 % channels == 0) {
             ds_dst[t * H + fh] = end > beg ? (d - b * phh) / dh : 0.f;
@@ -326,7 +326,7 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 const int k = r * ES + se;
-                const int src = __shfl_sync(kFull, c, k);
+                const int src = lane_get(c, k);
                 if (k < cnt) {
                     const float l = leaky(__ldg(s_src + static_cast<int64_t>(src) * H + sh) + sd, slope);
                     alpha[(base + k) * H + sh] = exp2f(l - m) / den;

@@ -288,7 +288,7 @@ struct GatByTarget {
     }
     __device__ __forceinline__ void join() {
 #pragma unroll
-        for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return __shfl_xor_sync(kFull, mine, o); });
+        for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return lane_xor(mine, o); });
     }
     __device__ __forceinline__ void merge(const float *slot) {
         fold([&](float, int q) { return slot[q * LPR + at.sub]; });
@@ -344,8 +344,8 @@ struct GatByTarget {
                     }
                 }
                 for (int o = 1; o < hl; o <<= 1) {
-                    b += __shfl_xor_sync(kFull, b, o);
-                    d += __shfl_xor_sync(kFull, d, o);
+                    b += lane_xor(b, o);
+                    d += lane_xor(d, o);
                 }
                 if (at.g == 0 && i < at.own && (at.f0 + i * LPR * VEC) % a.channels == 0) {
                     const int k = NH > 1 ? i : 0;
@@ -533,7 +533,7 @@ struct GatBySource {
     }
     __device__ __forceinline__ void join() {
 #pragma unroll
-        for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return __shfl_xor_sync(kFull, mine, o); });
+        for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return lane_xor(mine, o); });
     }
     __device__ __forceinline__ void merge(const float *slot) {
         fold([&](float, int q) { return slot[q * LPR + at.sub]; });
@@ -565,7 +565,7 @@ struct GatBySource {
 #pragma unroll
                 for (int q = 0; q < VEC; ++q) d = fmaf(xs[q], Q[i][q], d);
             }
-            for (int o = 1; o < hl; o <<= 1) d += __shfl_xor_sync(kFull, d, o);
+            for (int o = 1; o < hl; o <<= 1) d += lane_xor(d, o);
             if (at.g == 0 && i < at.own) {
                 const uint32_t fi = at.f0 + i * LPR * VEC;
                 const int h = static_cast<int>(fi / a.channels);

@@ -60,7 +60,7 @@ gather_xor_kernel(const int32_t *__restrict__ col, int64_t e, const uint4 *__res
 #pragma unroll
             for (int u = 0; u < kDepth; ++u) {
                 const int k = (j + u) * G + g;
-                const uint32_t src = static_cast<uint32_t>(__shfl_sync(kFull, src_l, k));
+                const uint32_t src = static_cast<uint32_t>(lane_get(src_l, k));
                 raw[u] = k < cnt ? ld_row16(x + static_cast<uint64_t>(src) * LPR + sub)
                                  : make_uint4(0u, 0u, 0u, 0u);
             }
@@ -76,10 +76,10 @@ gather_xor_kernel(const int32_t *__restrict__ col, int64_t e, const uint4 *__res
     // fold the lane groups, then the CTA's warps, then the CTAs (atomics)
 #pragma unroll
     for (int s = LPR; s < 32; s <<= 1) {
-        acc.x ^= __shfl_xor_sync(kFull, acc.x, s);
-        acc.y ^= __shfl_xor_sync(kFull, acc.y, s);
-        acc.z ^= __shfl_xor_sync(kFull, acc.z, s);
-        acc.w ^= __shfl_xor_sync(kFull, acc.w, s);
+        acc.x ^= lane_xor(acc.x, s);
+        acc.y ^= lane_xor(acc.y, s);
+        acc.z ^= lane_xor(acc.z, s);
+        acc.w ^= lane_xor(acc.w, s);
     }
     if (lane < LPR) s_fold[warp][lane] = acc;
     __syncthreads();

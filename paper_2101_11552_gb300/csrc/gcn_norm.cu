@@ -34,7 +34,7 @@ __global__ void dinv_weighted(const int32_t *__restrict__ rowptr, const int32_t 
     float s = 0.f;
     for (int64_t k = rowptr[t] + lane; k < rowptr[t + 1]; k += 32) s += __ldg(ew + perm[k]);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+    for (int o = 16; o > 0; o >>= 1) s += lane_xor(s, o);
     if (lane == 0) dinv[t] = inv_sqrt_or_zero(s + (add_self ? fill : 0.f));
 }
 

@@ -72,9 +72,9 @@ struct MaxByTarget {
     static constexpr int kWarps = PACKED ? TFG_MW_PACKED_WARPS : TFG_MW_WARPS, kLpr = LPR, G = 32 / LPR;
     static constexpr int kTile = LPR * VEC * T, kHeadsPerLane = T;
     static constexpr int kState = (ARG ? 2 : 1) * T * VEC, kHeld = 0;
-    static constexpr int kFull = TFG_MW_DEPTH * G > 32 ? 32 / G : TFG_MW_DEPTH;
-    static_assert(32 % (G * kFull) == 0, "a full window is read in whole steps");
-    static constexpr int kPart = walk_part(G) < kFull ? walk_part(G) : kFull;
+    static constexpr int kStepFull = TFG_MW_DEPTH * G > 32 ? 32 / G : TFG_MW_DEPTH;
+    static_assert(32 % (G * kStepFull) == 0, "a full window is read in whole steps");
+    static constexpr int kStepPart = walk_part(G) < kStepFull ? walk_part(G) : kStepFull;
     static constexpr int kPairs = PACKED ? VEC / 2 : 1;
     static constexpr int kReach = 65000;          // edges that 16-bit positions cover
     static constexpr uint32_t kLowest = 0xff80ff80u, kNone = 0xffffffffu;
@@ -218,13 +218,13 @@ struct MaxByTarget {
         k += cnt;
         if (!CHECK) {                                     // a full window
 #pragma unroll
-            for (int e = 0; e < 32; e += G * kFull) step<kFull, false>(sp + e, 0, at + e);
+            for (int e = 0; e < 32; e += G * kStepFull) step<kStepFull, false>(sp + e, 0, at + e);
             return;
         }
 #pragma unroll 1
-        for (; cnt >= G * kFull; cnt -= G * kFull, sp += G * kFull, at += G * kFull) step<kFull, false>(sp, 0, at);
+        for (; cnt >= G * kStepFull; cnt -= G * kStepFull, sp += G * kStepFull, at += G * kStepFull) step<kStepFull, false>(sp, 0, at);
 #pragma unroll 1
-        for (; cnt > 0; cnt -= G * kPart, sp += G * kPart, at += G * kPart) step<kPart, true>(sp, cnt - g, at);
+        for (; cnt > 0; cnt -= G * kStepPart, sp += G * kStepPart, at += G * kStepPart) step<kStepPart, true>(sp, cnt - g, at);
     }
     template <class GetB, class GetP>
     __device__ __forceinline__ void fold(GetB get_b, GetP get_p) {
@@ -256,8 +256,8 @@ struct MaxByTarget {
         }
 #pragma unroll
         for (int o = LPR; o < 32; o <<= 1)
-            fold([&](float mine, int) { return __shfl_xor_sync(kFull, mine, o); },
-                 [&](int32_t mine, int) { return __shfl_xor_sync(kFull, mine, o); });
+            fold([&](float mine, int) { return lane_xor(mine, o); },
+                 [&](int32_t mine, int) { return lane_xor(mine, o); });
     }
     __device__ __forceinline__ void spill() {             // warp-uniform, rare
         unpack_and_join();

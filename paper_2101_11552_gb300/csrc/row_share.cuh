@@ -27,7 +27,7 @@ __device__ __forceinline__ int64_t warp_last_row_at(const int32_t *rowptr, int64
         const int64_t step = (hi - lo + 31) / 32;
         const int64_t p = lo + (lane + 1) * step;                   // probes in (lo, hi]
         const bool le = p <= hi && static_cast<int64_t>(__ldg(rowptr + p)) + kRowCost * p <= q;
-        const int c = __popc(__ballot_sync(kFull, le));             // monotone: lanes 0 .. c - 1
+        const int c = __popc(lane_ballot(le));             // monotone: lanes 0 .. c - 1
         const int64_t top = lo + (c + 1) * step - 1;
         lo += c * step;
         hi = top < hi ? top : hi;

@@ -74,7 +74,7 @@ __device__ __forceinline__ void walk_rows(const int32_t *__restrict__ rowptr, co
     int j = 0;                                              // position in the staged window
     for (;;) {
         const bool closes = t < tb;
-        const int32_t rend = closes ? __shfl_sync(kFull, rwin, tl) : kb;
+        const int32_t rend = closes ? lane_get(rwin, tl) : kb;
         int rem = rend - k;
         k = rend;
         if (closes || rem > 0) {
