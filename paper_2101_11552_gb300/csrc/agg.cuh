@@ -25,9 +25,10 @@
 //    row's features with LPR lanes (16-byte slices, or T single features a lane
 //    in rows without 16-byte slices); D gathers are in flight per lane in full
 //    windows, P in partial ones; the groups' sums are combined by a butterfly.
-//  * Sums are blocked per window, so an fp32 chain is at most 32 / G + degree / 32
-//    additions long.  Slots without an edge are not loaded: an infinity in an
-//    unrelated row never meets a zero weight.
+//  * Sums are blocked per window, so an fp32 chain is at most 32 / (G * CH) + degree / 32
+//    additions long, CH the chains a lane keeps: two in rows of 17 to 31 slices, one
+//    otherwise.  Slots without an edge are not loaded: an infinity in an unrelated row
+//    never meets a zero weight.
 //  * GCN mode without w_csr forms the weight on the fly:  out[t] = dinv[t] *
 //    (sum_k dinv[col[k]] * x[col[k]] + fill * dinv[t] * x[t]), so no per-edge
 //    weight array is read.  With w_csr it adds fill * dinv[t]^2 * x[t] to the
@@ -78,7 +79,16 @@ namespace {
 #define TFG_AGG_PART4 2
 #endif
 constexpr int kAggWarps = TFG_AGG_WARPS;
-constexpr int kAggThreads = kAggWarps * 32;
+// 16-byte bf16 rows with two chains, whose registers are short: 24 against 28, GCN of
+// 23.3M edges, F = 136 / 200 / 248: 757 / 867 / 971 us against 835 / 979 / 1100 (one
+// chain 711 / 804 / 886); 169,343 nodes of mean in-degree 6.9: 117 / 138 / 154 us against
+// 123 / 146 / 161 (105 / 123 / 135).
+#ifndef TFG_AGG_WARPS_CHAINS
+#define TFG_AGG_WARPS_CHAINS 24
+#endif
+__host__ __device__ constexpr int agg_warps(int vec, int chains) {
+    return vec == 8 && chains > 1 ? TFG_AGG_WARPS_CHAINS : kAggWarps;
+}
 // Work (edges + kRowCost per row) a warp should have, at least: 8 against 32 on
 // 2,708 nodes and 13,264 edges: 6.4 / 8.0 us.
 constexpr int kAggMinWork = 8;
@@ -144,6 +154,24 @@ struct RowAgg {
         }
     }
 
+    // the sum of the chains of a window, in the first (pairs through fma2: times one is exact)
+    template <int CH>
+    static __device__ __forceinline__ void join_chains(float (&part)[CH][T][VEC]) {
+        if constexpr (CH > 1) {
+            static_assert(CH == 2 && !kIsMax, "one chain or two, of sums");
+            const float2 one = make_float2(1.f, 1.f);
+#pragma unroll
+            for (int i = 0; i < T; ++i)
+#pragma unroll
+                for (int q = 0; q < VEC; q += 2) {
+                    const float2 r = fma2(make_float2(part[1][i][q], part[1][i][q + 1]), one,
+                                          make_float2(part[0][i][q], part[0][i][q + 1]));
+                    part[0][i][q] = r.x;
+                    part[0][i][q + 1] = r.y;
+                }
+        }
+    }
+
     // Final values of VEC features: dt * (acc + fill dt self), with given edge
     // weights acc + fill dt^2 self; acc / deg for a mean; 0 for an empty max.
     static __device__ __forceinline__ void finish(const AggArgs &a, float c1, float c2, int32_t deg, float (&r)[VEC],
@@ -186,17 +214,20 @@ struct RowAgg {
     }
 };
 
-template <typename XT, int VEC, int LPR, int T, int KIND, typename X0T>
-__global__ void __launch_bounds__(kAggThreads, 1) aggregate_rows(AggArgs a) {
+// CH: chains of additions a lane keeps within a window, edge by edge in turn.
+template <typename XT, int VEC, int LPR, int T, int CH, int KIND, typename X0T>
+__global__ void __launch_bounds__(agg_warps(VEC, CH) * 32, 1) aggregate_rows(AggArgs a) {
     using S = RowAgg<XT, VEC, LPR, T, KIND, X0T>;
     using V = typename S::V;
     using V0 = typename S::V0;
     constexpr int G = S::G, D = S::D, P = S::P;
+    constexpr int W = agg_warps(VEC, CH);
+    static_assert(D % CH == 0 && P % CH == 0, "steps give every chain the same number of edges");
     extern __shared__ __align__(16) float s_parts[];          // tails [warp][kTile], heads [warp][kTile]
     __shared__ int64_t s_row[2];
-    __shared__ int32_t s_tail_row[kAggWarps], s_head_row[kAggWarps];
-    __shared__ __align__(16) float2 s_stage[kAggWarps][64];    // a window's (id, weight) pairs, and room to read past them
-    WarpShare<kAggWarps> sh;
+    __shared__ int32_t s_tail_row[W], s_head_row[W];
+    __shared__ __align__(16) float2 s_stage[W][64];    // a window's (id, weight) pairs, and room to read past them
+    WarpShare<W> sh;
     if (!sh.init(a.rowptr, a.n, kAggMinWork, s_row)) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sub = lane % LPR, g = lane / LPR;
@@ -257,7 +288,7 @@ __global__ void __launch_bounds__(kAggThreads, 1) aggregate_rows(AggArgs a) {
         int32_t k = sh.ka, rbeg = __ldg(a.rowptr + t);
         int j = 0;                                         // position in the staged window
         // edges [j, j + cnt) of the staged window into part
-        auto some = [&](float (&part)[T][VEC], int cnt) {
+        auto some = [&](float (&part)[CH][T][VEC], int cnt) {
             const float2 *sp = stage + j + g;
             int m = cnt - g;                               // this group's are sp[0], sp[G], ... below m
 #pragma unroll 1
@@ -274,16 +305,18 @@ __global__ void __launch_bounds__(kAggThreads, 1) aggregate_rows(AggArgs a) {
 #pragma unroll
                 for (int u = 0; u < P; ++u)
 #pragma unroll
-                    for (int i = 0; i < T; ++i) S::template axpy<true>(part[i], w[u], raw[u][i], m > u * G);
+                    for (int i = 0; i < T; ++i) S::template axpy<true>(part[u % CH][i], w[u], raw[u][i], m > u * G);
                 sp += G * P;
                 m -= G * P;
             }
         };
-        auto clear = [&](float (&v)[T][VEC]) {
+        auto clear = [&](float (&v)[CH][T][VEC]) {
 #pragma unroll
-            for (int i = 0; i < T; ++i)
+            for (int c = 0; c < CH; ++c)
 #pragma unroll
-                for (int q = 0; q < VEC; ++q) v[i][q] = S::identity();
+                for (int i = 0; i < T; ++i)
+#pragma unroll
+                    for (int q = 0; q < VEC; ++q) v[c][i][q] = S::identity();
         };
         for (;;) {
             const bool closes = t < tb;
@@ -298,22 +331,32 @@ __global__ void __launch_bounds__(kAggThreads, 1) aggregate_rows(AggArgs a) {
             }
             int rem = rend - k;
             k = rend;
-            clear(acc);
             if (j == 32 && rem > 0) {
                 next_window();
                 j = 0;
             }
             if (rem <= 32 - j) {                           // the rest of the row lies in this window
-                some(acc, rem);
+                float part[CH][T][VEC];
+                clear(part);
+                some(part, rem);
+                S::join_chains(part);
+#pragma unroll
+                for (int i = 0; i < T; ++i)
+#pragma unroll
+                    for (int q = 0; q < VEC; ++q) acc[i][q] = part[0][i][q];
                 j += rem;
             } else {
+#pragma unroll
+                for (int i = 0; i < T; ++i)
+#pragma unroll
+                    for (int q = 0; q < VEC; ++q) acc[i][q] = S::identity();
                 while (rem > 0) {
                     if (j == 32) {
                         next_window();
                         j = 0;
                     }
                     const int cnt = min(rem, 32 - j);
-                    float part[T][VEC];                    // sums are blocked per window
+                    float part[CH][T][VEC];                // sums are blocked per window
                     clear(part);
                     if (cnt == 32) {
 #pragma unroll
@@ -329,15 +372,16 @@ __global__ void __launch_bounds__(kAggThreads, 1) aggregate_rows(AggArgs a) {
 #pragma unroll
                             for (int u = 0; u < D; ++u)
 #pragma unroll
-                                for (int i = 0; i < T; ++i) S::template axpy<false>(part[i], w[u], raw[u][i], true);
+                                for (int i = 0; i < T; ++i) S::template axpy<false>(part[u % CH][i], w[u], raw[u][i], true);
                         }
                     } else {
                         some(part, cnt);
                     }
+                    S::join_chains(part);
 #pragma unroll
                     for (int i = 0; i < T; ++i)
 #pragma unroll
-                        for (int q = 0; q < VEC; ++q) acc[i][q] = S::combine(acc[i][q], part[i][q]);
+                        for (int q = 0; q < VEC; ++q) acc[i][q] = S::combine(acc[i][q], part[0][i][q]);
                     rem -= cnt;
                     j += cnt;
                 }
@@ -358,7 +402,7 @@ __global__ void __launch_bounds__(kAggThreads, 1) aggregate_rows(AggArgs a) {
                     for (int i = 0; i < T; ++i)
 #pragma unroll
                         for (int q = 0; q < VEC; ++q)
-                            s_parts[(kAggWarps + warp) * S::kTile + (i * LPR + sub) * VEC + q] = acc[i][q];
+                            s_parts[(W + warp) * S::kTile + (i * LPR + sub) * VEC + q] = acc[i][q];
                 }
                 if (lane == 0) s_head_row[warp] = t;
             } else if (g == 0) {
@@ -403,7 +447,7 @@ __global__ void __launch_bounds__(kAggThreads, 1) aggregate_rows(AggArgs a) {
 #pragma unroll
                     for (int q = 0; q < VEC; ++q) r[q] = S::combine(r[q], s_parts[s * S::kTile + at + q]);
 #pragma unroll
-                for (int q = 0; q < VEC; ++q) r[q] = S::combine(r[q], s_parts[(kAggWarps + warp) * S::kTile + at + q]);
+                for (int q = 0; q < VEC; ++q) r[q] = S::combine(r[q], s_parts[(W + warp) * S::kTile + at + q]);
                 typename V0::Raw x0t = V0::zero();
                 if (S::kX0) x0t = V0::raw(static_cast<const X0T *>(a.x0) + at0 + i * LPR * VEC);
                 S::finish(a, c1f, c2f, deg, r, xt[i], x0t);
@@ -414,19 +458,20 @@ __global__ void __launch_bounds__(kAggThreads, 1) aggregate_rows(AggArgs a) {
     }
 }
 
-template <typename XT, int VEC, int LPR, int T, int KIND, typename X0T>
+template <typename XT, int VEC, int LPR, int T, int KIND, typename X0T, int CH = 1>
 cudaError_t launch_rows(const AggArgs &a, cudaStream_t s) {
     using S = RowAgg<XT, VEC, LPR, T, KIND, X0T>;
-    auto *kernel = aggregate_rows<XT, VEC, LPR, T, KIND, X0T>;
+    auto *kernel = aggregate_rows<XT, VEC, LPR, T, CH, KIND, X0T>;
     const int64_t tiles = (a.f + S::kTile - 1) / S::kTile;
-    constexpr int smem = 2 * kAggWarps * S::kTile * static_cast<int>(sizeof(float));
+    constexpr int threads = agg_warps(VEC, CH) * 32;
+    constexpr int smem = 2 * agg_warps(VEC, CH) * S::kTile * static_cast<int>(sizeof(float));
     if constexpr (smem > 32 * 1024) {   // with the static part above the 48 KB every launch may use
         const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (err != cudaSuccess) return err;
     }
     const dim3 grid(static_cast<unsigned>(min64(a.n, static_cast<int64_t>(sm_count()))),
                     static_cast<unsigned>(min64(tiles, 65535)));
-    kernel<<<grid, kAggThreads, smem, s>>>(a);
+    kernel<<<grid, threads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -437,6 +482,9 @@ cudaError_t launch_rows_vec(const AggArgs &a, cudaStream_t s) {
     const int64_t slices = a.f / VEC;
     if (slices <= 8) return launch_rows<XT, VEC, 8, 1, KIND, X0T>(a, s);
     if (slices <= 16) return launch_rows<XT, VEC, 16, 1, KIND, X0T>(a, s);
+    if constexpr (KIND != kMax) {
+        if (slices < 32) return launch_rows<XT, VEC, 32, 1, KIND, X0T, 2>(a, s);
+    }
     return launch_rows<XT, VEC, 32, 1, KIND, X0T>(a, s);
 }
 

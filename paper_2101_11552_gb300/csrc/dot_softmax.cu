@@ -353,8 +353,8 @@ void launch_fast_vec(const DotArgs &a, int lh, int grid, cudaStream_t s) {
     else launch_fast_lpr<XT, VEC, 8>(a, lh, grid, s);
 }
 
-template <typename XT, int VEC, int LPR, int LH>
-using DotForward = DotByTarget<XT, VEC, LPR, LH, false>;
+template <typename XT, int VEC, int LPR, int LH, int CH>
+using DotForward = DotByTarget<XT, VEC, LPR, LH, false, CH>;
 
 template <typename XT>
 void launch_general(const DotArgs &a, int grid, cudaStream_t s) {

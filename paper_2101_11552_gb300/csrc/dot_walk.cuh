@@ -48,6 +48,15 @@ namespace {
 #ifndef TFG_DW_SRC_WARPS
 #define TFG_DW_SRC_WARPS 16
 #endif
+// The same in bf16 rows with two chains, whose registers are short: forward and
+// backward of 6 x 32 over 10M edges 3689 us with 20 and 16, by target 16 3501, by
+// source 12 3639, 14 3849 (one chain 3291); 169,343 nodes 987 / 961 / 945 / 1027 (839).
+#ifndef TFG_DW_TGT_WARPS_CHAINS
+#define TFG_DW_TGT_WARPS_CHAINS 16
+#endif
+#ifndef TFG_DW_SRC_WARPS_CHAINS
+#define TFG_DW_SRC_WARPS_CHAINS 12
+#endif
 #ifndef TFG_DW_DEPTH
 #define TFG_DW_DEPTH 4        // edges in flight per lane group, full windows
 #endif
@@ -136,6 +145,18 @@ struct DotLane {
     }
 };
 
+// Within a window a lane adds its edges in CH chains, edge by edge in turn: two in rows
+// of 17 to 31 slices, whose 32 lanes leave one lane group.  The chains' sum, in the first.
+template <int CH, int N>
+__device__ __forceinline__ void dw_join_chains(float (&acc)[CH][N]) {
+    if constexpr (CH > 1) {
+        static_assert(CH == 2, "one chain or two");
+#pragma unroll
+        for (int i = 0; i < N; ++i) acc[0][i] += acc[1][i];
+        dw_clear(acc[1]);
+    }
+}
+
 // Sums are blocked per window of 32 edges.  The sums of a row's earlier windows wait
 // in shared memory (element q of a lane at q * 32), so that the registers hold
 // one set of accumulators and more rows in flight; a row of one window never
@@ -175,11 +196,13 @@ struct DotHeld {
 
 // Softmax over the in-edges of a target.  BWD = false: acc = sum of p v[src];
 // BWD = true: acc = sum of p (dalpha - beta) k[src], dalpha = <grad_out[t], v[src]>.
-template <typename XT, int VEC, int LPR, int LH, bool BWD>
+template <typename XT, int VEC, int LPR, int LH, bool BWD, int CH = 1>
 struct DotByTarget {
     using L = DotLane<XT, VEC, LPR, LH>;
     using V = VecLoad<XT, VEC>;
-    static constexpr int kWarps = BWD ? TFG_DW_TGT_WARPS : TFG_DW_FWD_WARPS, kLpr = LPR, G = 32 / LPR;
+    static constexpr int kWarps = !BWD ? TFG_DW_FWD_WARPS
+                                       : (VEC == 8 && CH > 1 ? TFG_DW_TGT_WARPS_CHAINS : TFG_DW_TGT_WARPS);
+    static constexpr int kLpr = LPR, G = 32 / LPR;
     static constexpr int kTile = LPR * VEC, kHeadsPerLane = 1;
     static constexpr int kState = VEC + 2, kHeld = VEC;
     static constexpr int kStepFull = TFG_DW_DEPTH * G > 32 ? 32 / G : TFG_DW_DEPTH, kUnroll = TFG_DW_UNROLL;
@@ -190,7 +213,7 @@ struct DotByTarget {
     const char *kb, *vb;
     float2 *scratch;                      // [warp][heads of the tile] (m, den), for alpha
     DotHeld<VEC> held;                    // the sums of the row's earlier windows
-    float qv[VEC], gt[BWD ? VEC : 1], beta, m, den, acc[VEC];
+    float qv[VEC], gt[BWD ? VEC : 1], beta, m, den, acc[CH][VEC];
 
     __device__ __forceinline__ DotByTarget(const DotArgs &args, uint32_t ft, float *hold, float *scr)
         : a(args), ln(args, ft), scratch(reinterpret_cast<float2 *>(scr)), held(hold) {
@@ -201,7 +224,8 @@ struct DotByTarget {
     __device__ __forceinline__ void clear() {
         m = -CUDART_INF_F;
         den = 0.f;
-        dw_clear(acc);
+#pragma unroll
+        for (int c = 0; c < CH; ++c) dw_clear(acc[c]);
         held.clear();
     }
     __device__ __forceinline__ void load_query(int32_t t) {
@@ -221,7 +245,8 @@ struct DotByTarget {
     }
     // D edges of the group, sp[0], sp[G], ... (CHECK: those below left)
     template <int D, bool CHECK>
-    __device__ __forceinline__ void step(const int32_t *sp, int left, float &dpart) {
+    __device__ __forceinline__ void step(const int32_t *sp, int left, float (&dpart)[CH]) {
+        static_assert(D % CH == 0, "a step gives every chain the same number of edges");
         typename V::Raw rk[D], rv[D];
 #pragma unroll
         for (int u = 0; u < D; ++u) {
@@ -246,37 +271,41 @@ struct DotByTarget {
         if (top > m) {                                           // a new running maximum: rescale the sums so far
             const float sc = dw_rescale(m, top);
             den *= sc;
-            dpart *= sc;
 #pragma unroll
-            for (int i = 0; i < VEC; ++i) acc[i] *= sc;
+            for (int c = 0; c < CH; ++c) {
+                dpart[c] *= sc;
+#pragma unroll
+                for (int i = 0; i < VEC; ++i) acc[c][i] *= sc;
+            }
             held.scale(sc);
             m = top;
         }
 #pragma unroll
         for (int u = 0; u < D; ++u) {
             const float p = !CHECK || left > u * G ? exp2f(l[u] - m) : 0.f;
-            dpart += p;
+            dpart[u % CH] += p;
             float x[VEC];
             V::widen(BWD ? rk[u] : rv[u], x);
-            dw_axpy(acc, !BWD ? p : (!CHECK || left > u * G ? p * w[u] : 0.f), x);
+            dw_axpy(acc[u % CH], !BWD ? p : (!CHECK || left > u * G ? p * w[u] : 0.f), x);
         }
     }
     template <bool CHECK>
     __device__ __forceinline__ void add(const int32_t *ids, int cnt) {
-        held.next(acc);                                          // sums are blocked per window
-        float dpart = 0.f;
+        dw_join_chains(acc);
+        held.next(acc[0]);                                       // sums are blocked per window
+        float dpart[CH] = {};
         const int32_t *sp = ids + ln.g;
         if (!CHECK) {                                            // a full window
 #pragma unroll kUnroll
             for (int e = 0; e < 32; e += G * kStepFull) step<kStepFull, false>(sp + e, 0, dpart);
-            den += dpart;
+            den += CH == 1 ? dpart[0] : dpart[0] + dpart[CH - 1];
             return;
         }
 #pragma unroll 1
         for (; cnt >= G * kStepFull; cnt -= G * kStepFull, sp += G * kStepFull) step<kStepFull, false>(sp, 0, dpart);
 #pragma unroll 1
         for (; CHECK && cnt > 0; cnt -= G * kStepPart, sp += G * kStepPart) step<kStepPart, true>(sp, cnt - ln.g, dpart);
-        den += dpart;
+        den += CH == 1 ? dpart[0] : dpart[0] + dpart[CH - 1];
     }
     template <class Get>
     __device__ __forceinline__ void fold(Get get) {
@@ -284,11 +313,12 @@ struct DotByTarget {
         const float sa = dw_rescale(m, mm), sb = dw_rescale(m2, mm);
         den = den * sa + get(den, VEC + 1) * sb;
 #pragma unroll
-        for (int i = 0; i < VEC; ++i) acc[i] = acc[i] * sa + get(acc[i], i) * sb;
+        for (int i = 0; i < VEC; ++i) acc[0][i] = acc[0][i] * sa + get(acc[0][i], i) * sb;
         m = mm;
     }
     __device__ __forceinline__ void join() {
-        held.last(acc);
+        dw_join_chains(acc);
+        held.last(acc[0]);
 #pragma unroll
         for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return lane_xor(mine, o); });
     }
@@ -298,7 +328,7 @@ struct DotByTarget {
     __device__ __forceinline__ void park(float *slot) const {
         if (ln.g != 0) return;
 #pragma unroll
-        for (int i = 0; i < VEC; ++i) slot[i * LPR + ln.sub] = acc[i];
+        for (int i = 0; i < VEC; ++i) slot[i * LPR + ln.sub] = acc[0][i];
         slot[VEC * LPR + ln.sub] = m;
         slot[(VEC + 1) * LPR + ln.sub] = den;
     }
@@ -306,14 +336,14 @@ struct DotByTarget {
         const bool any = end > beg;
         if (ln.g == 0 && ln.own) {
             if constexpr (BWD) {
-                dw_store(a.grad_q + ln.at(t), acc, any ? a.scale / den : 0.f);
+                dw_store(a.grad_q + ln.at(t), acc[0], any ? a.scale / den : 0.f);
                 if (ln.sub % ln.lh == 0)
                     a.stats[ln.stat(static_cast<uint32_t>(t), a.heads)] =
                         make_float4(m, any ? 1.f / den : 0.f, beta, 0.f);
             } else {
                 float r[VEC];
 #pragma unroll
-                for (int i = 0; i < VEC; ++i) r[i] = any ? acc[i] / den : 0.f;
+                for (int i = 0; i < VEC; ++i) r[i] = any ? acc[0][i] / den : 0.f;
                 dw_store(a.out + ln.at(t), r, 1.f);
             }
         }
@@ -353,11 +383,11 @@ struct DotByTarget {
 // alpha grad_out[t].
 // WIDE (VEC = 8): 32-byte gradient slices, one load each instead of two that each
 // touch every sector: 114.6M edges 7.49 ms against 7.59.
-template <typename XT, int VEC, int LPR, int LH, bool WIDE>
+template <typename XT, int VEC, int LPR, int LH, bool WIDE, int CH = 1>
 struct DotSource {
     using L = DotLane<XT, VEC, LPR, LH>;
     using V = VecLoad<XT, VEC>;
-    static constexpr int kWarps = TFG_DW_SRC_WARPS, kLpr = LPR, G = 32 / LPR;
+    static constexpr int kWarps = VEC == 8 && CH > 1 ? TFG_DW_SRC_WARPS_CHAINS : TFG_DW_SRC_WARPS, kLpr = LPR, G = 32 / LPR;
     static constexpr int kTile = LPR * VEC, kHeadsPerLane = 1;
     static constexpr int kState = 2 * VEC, kHeld = 2 * VEC;
     static constexpr int kStepFull = TFG_DW_DEPTH * G > 32 ? 32 / G : TFG_DW_DEPTH;
@@ -367,7 +397,7 @@ struct DotSource {
     L ln;
     const char *qb, *gb;
     DotHeld<2 * VEC> held;
-    float ks[VEC], vs[VEC], dkv[2 * VEC];  // grad_k's and grad_v's sums
+    float ks[VEC], vs[VEC], dkv[CH][2 * VEC];  // grad_k's and grad_v's sums
 
     __device__ __forceinline__ DotSource(const DotArgs &args, uint32_t ft, float *hold, float *)
         : a(args), ln(args, ft), held(hold) {
@@ -375,7 +405,8 @@ struct DotSource {
         gb = reinterpret_cast<const char *>(a.grad_out + ln.f0);
     }
     __device__ __forceinline__ void clear() {
-        dw_clear(dkv);
+#pragma unroll
+        for (int c = 0; c < CH; ++c) dw_clear(dkv[c]);
         held.clear();
     }
     __device__ __forceinline__ void open(int32_t s, int32_t, int32_t) {
@@ -385,6 +416,7 @@ struct DotSource {
     }
     template <int D, bool CHECK>
     __device__ __forceinline__ void step(const int32_t *sp, int left) {
+        static_assert(D % CH == 0, "a step gives every chain the same number of edges");
         typename V::Raw rq[D];
         float gr[D][VEC];
         float4 st[D];
@@ -406,9 +438,9 @@ struct DotSource {
             }
             st[u] = ok ? __ldg(a.stats + ln.stat(id, a.heads)) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        float *pk = dkv, *pv = dkv + VEC;
 #pragma unroll
         for (int u = 0; u < D; ++u) {
+            float *pk = dkv[u % CH], *pv = dkv[u % CH] + VEC;
             float qv[VEC];
             V::widen(rq[u], qv);
             const float l = ln.head_sum(dw_dot(qv, ks)) * a.scale2;
@@ -428,7 +460,8 @@ struct DotSource {
     }
     template <bool CHECK>
     __device__ __forceinline__ void add(const int32_t *ids, int cnt) {
-        held.next(dkv);
+        dw_join_chains(dkv);
+        held.next(dkv[0]);
         const int32_t *sp = ids + ln.g;
 #pragma unroll 1
         for (; cnt >= G * kStepFull; cnt -= G * kStepFull, sp += G * kStepFull) step<kStepFull, false>(sp, 0);
@@ -438,10 +471,11 @@ struct DotSource {
     template <class Get>
     __device__ __forceinline__ void fold(Get get) {
 #pragma unroll
-        for (int i = 0; i < 2 * VEC; ++i) dkv[i] += get(dkv[i], i);
+        for (int i = 0; i < 2 * VEC; ++i) dkv[0][i] += get(dkv[0][i], i);
     }
     __device__ __forceinline__ void join() {
-        held.last(dkv);
+        dw_join_chains(dkv);
+        held.last(dkv[0]);
 #pragma unroll
         for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return lane_xor(mine, o); });
     }
@@ -451,7 +485,7 @@ struct DotSource {
     __device__ __forceinline__ void park(float *slot) const {
         if (ln.g != 0) return;
 #pragma unroll
-        for (int i = 0; i < 2 * VEC; ++i) slot[i * LPR + ln.sub] = dkv[i];
+        for (int i = 0; i < 2 * VEC; ++i) slot[i * LPR + ln.sub] = dkv[0][i];
     }
     __device__ __forceinline__ bool wants_after() const { return false; }
     __device__ __forceinline__ void after(int, int32_t, int32_t, int32_t) {}
@@ -460,36 +494,37 @@ struct DotSource {
         float dk[VEC], dv[VEC];
 #pragma unroll
         for (int i = 0; i < VEC; ++i) {
-            dk[i] = dkv[i];
-            dv[i] = dkv[VEC + i];
+            dk[i] = dkv[0][i];
+            dv[i] = dkv[0][VEC + i];
         }
         dw_store(a.grad_k + ln.at(s), dk, a.scale);
         dw_store(a.grad_v + ln.at(s), dv, 1.f);
     }
 };
 
-template <typename XT, int VEC, int LPR, int LH>
-using DotBySource = DotSource<XT, VEC, LPR, LH, VEC == 8>;
+template <typename XT, int VEC, int LPR, int LH, int CH>
+using DotBySource = DotSource<XT, VEC, LPR, LH, VEC == 8, CH>;
 // gradient rows that are not 32-byte aligned: one kernel a row width, heads at run time
-template <typename XT, int VEC, int LPR, int LH>
-using DotBySourceNarrow = DotSource<XT, VEC, LPR, 0, false>;
+template <typename XT, int VEC, int LPR, int LH, int CH>
+using DotBySourceNarrow = DotSource<XT, VEC, LPR, 0, false, CH>;
 
 // lh (a power of two up to 32, at most the lanes of a row) picks the kernel with
-// that many lanes per head.  PASS<XT, VEC, LPR, LH> is the policy.
-template <template <typename, int, int, int> class PASS, typename XT, int VEC, int LPR>
+// that many lanes per head.  PASS<XT, VEC, LPR, LH, CH> is the policy.
+template <template <typename, int, int, int, int> class PASS, typename XT, int VEC, int LPR, int CH = 1>
 cudaError_t launch_dot_lanes(const DotArgs &a, cudaStream_t s) {
     switch (a.lh) {
-        case 1: return launch_walk<PASS<XT, VEC, LPR, 1>>(a, s);
-        case 2: return launch_walk<PASS<XT, VEC, LPR, 2>>(a, s);
-        case 4: return launch_walk<PASS<XT, VEC, LPR, 4>>(a, s);
-        case 8: return launch_walk<PASS<XT, VEC, LPR, 8>>(a, s);
-        default: return launch_walk<PASS<XT, VEC, LPR, 0>>(a, s);
+        case 1: return launch_walk<PASS<XT, VEC, LPR, 1, CH>>(a, s);
+        case 2: return launch_walk<PASS<XT, VEC, LPR, 2, CH>>(a, s);
+        case 4: return launch_walk<PASS<XT, VEC, LPR, 4, CH>>(a, s);
+        case 8: return launch_walk<PASS<XT, VEC, LPR, 8, CH>>(a, s);
+        default: return launch_walk<PASS<XT, VEC, LPR, 0, CH>>(a, s);
     }
 }
-template <template <typename, int, int, int> class PASS, typename XT, int VEC>
+template <template <typename, int, int, int, int> class PASS, typename XT, int VEC>
 cudaError_t launch_dot_pass(const DotArgs &a, cudaStream_t s) {
     const int64_t slices = static_cast<int64_t>(a.heads) * a.channels / VEC;
-    if (slices > 16 || a.lh > 16) return launch_dot_lanes<PASS, XT, VEC, 32>(a, s);
+    if (slices >= 32) return launch_dot_lanes<PASS, XT, VEC, 32>(a, s);
+    if (slices > 16 || a.lh > 16) return launch_dot_lanes<PASS, XT, VEC, 32, 2>(a, s);
     if (slices > 8 || a.lh > 8) return launch_dot_lanes<PASS, XT, VEC, 16>(a, s);
     return launch_dot_lanes<PASS, XT, VEC, 8>(a, s);
 }

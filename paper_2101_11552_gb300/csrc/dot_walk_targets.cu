@@ -4,8 +4,8 @@
 
 namespace tfg {
 namespace {
-template <typename XT, int VEC, int LPR, int LH>
-using DotTargets = DotByTarget<XT, VEC, LPR, LH, true>;
+template <typename XT, int VEC, int LPR, int LH, int CH>
+using DotTargets = DotByTarget<XT, VEC, LPR, LH, true, CH>;
 }  // namespace
 
 cudaError_t launch_dot_walk_targets(const DotArgs &a, int x_dtype, cudaStream_t s) {

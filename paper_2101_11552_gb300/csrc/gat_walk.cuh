@@ -141,14 +141,16 @@ struct GatLane {
 // phi the LeakyReLU's slope at the edge, dalpha = <grad_out[t], x[src]>: the sum
 // of the weighted rows is taken first, so an edge costs what it does in the
 // forward and the dot products are taken once per row.
-template <typename XT, int VEC, int LPR, int T, int NH, bool TARGET_BWD>
+// CH: chains of additions a lane keeps within a window, edge by edge in turn: two in
+// rows of 17 to 31 slices, whose 32 lanes leave one lane group.
+template <typename XT, int VEC, int LPR, int T, int NH, bool TARGET_BWD, int CH = 1>
 struct GatByTarget {
     using V = VecLoad<XT, VEC>;
     static constexpr int kWarps = TFG_GW_WARPS, kLpr = LPR, G = 32 / LPR;
     static constexpr int kTile = LPR * VEC * T, kHeadsPerLane = T;
     static constexpr int kState = T * VEC + NH * (TARGET_BWD ? 3 : 2), kHeld = 0;
     static constexpr int D = TFG_GW_DEPTH * G > 32 ? 32 / G : TFG_GW_DEPTH;   // gathers in flight per lane
-    static_assert(32 % (G * D) == 0, "a full window is read in whole steps");
+    static_assert(32 % (G * D) == 0 && D % CH == 0, "a full window is read in whole steps");
     const GatArgs &a;
     GatLane<VEC, LPR, T, NH> at;
     const char *xb;
@@ -180,13 +182,16 @@ struct GatByTarget {
     }
     template <bool CHECK>
     __device__ __forceinline__ void add(const int32_t *ids, int cnt) {
-        float part[T][VEC], dpart[NH], ppart[NH];           // sums are blocked per window
+        float part[CH][T][VEC], dpart[CH][NH], ppart[NH];   // sums are blocked per window
 #pragma unroll
-        for (int i = 0; i < T; ++i)
+        for (int c = 0; c < CH; ++c) {
 #pragma unroll
-            for (int q = 0; q < VEC; ++q) part[i][q] = 0.f;
+            for (int i = 0; i < T; ++i)
 #pragma unroll
-        for (int i = 0; i < NH; ++i) dpart[i] = ppart[i] = 0.f;
+                for (int q = 0; q < VEC; ++q) part[c][i][q] = 0.f;
+#pragma unroll
+            for (int i = 0; i < NH; ++i) dpart[c][i] = ppart[i] = 0.f;
+        }
         const int32_t *sp = ids + at.g;
         int left = cnt - at.g;                              // this group's edges: sp[0], sp[G], ... below left
 #pragma unroll 1
@@ -219,7 +224,8 @@ struct GatByTarget {
                 if (top > m[i]) {                           // a new running maximum: rescale the sums so far
                     const float sc = gw_rescale(m[i], top);
                     den[i] *= sc;
-                    dpart[i] *= sc;
+#pragma unroll
+                    for (int c = 0; c < CH; ++c) dpart[c][i] *= sc;
                     if (TARGET_BWD) {
                         phi[i] *= sc;
                         ppart[i] *= sc;
@@ -230,7 +236,8 @@ struct GatByTarget {
 #pragma unroll
                         for (int q = 0; q < VEC; ++q) {
                             acc[j][q] *= sc;
-                            part[j][q] *= sc;
+#pragma unroll
+                            for (int c = 0; c < CH; ++c) part[c][j][q] *= sc;
                         }
                     }
                     m[i] = top;
@@ -238,7 +245,7 @@ struct GatByTarget {
 #pragma unroll
                 for (int u = 0; u < D; ++u) {
                     const float p = !CHECK || left > u * G ? exp2f(l[u][i] - m[i]) : 0.f;
-                    dpart[i] += p;
+                    dpart[u % CH][i] += p;
                     w[u][i] = p;
                     if (TARGET_BWD) {
                         w[u][i] = z[u][i] > 0.f ? p : a.slope * p;
@@ -252,20 +259,20 @@ struct GatByTarget {
                 for (int i = 0; i < T; ++i) {
                     float v[VEC];
                     V::widen(raw[u][i], v);
-                    gw_axpy(part[i], w[u][NH > 1 ? i : 0], v);
+                    gw_axpy(part[u % CH][i], w[u][NH > 1 ? i : 0], v);
                 }
             sp += G * D;
             left -= G * D;
         }
 #pragma unroll
         for (int i = 0; i < NH; ++i) {
-            den[i] += dpart[i];
+            den[i] += CH == 1 ? dpart[0][i] : dpart[0][i] + dpart[CH - 1][i];
             if (TARGET_BWD) phi[i] += ppart[i];
         }
 #pragma unroll
         for (int i = 0; i < T; ++i)
 #pragma unroll
-            for (int q = 0; q < VEC; ++q) acc[i][q] += part[i][q];
+            for (int q = 0; q < VEC; ++q) acc[i][q] += CH == 1 ? part[0][i][q] : part[0][i][q] + part[CH - 1][i][q];
     }
     // this state and (m2, den2, phi2, acc2), element by element
     template <class Get>

@@ -221,3 +221,80 @@ def test_gradient_slices_of_32_bytes(heads, channels, dtype, offset):
     check(("grad_q", "grad_k", "grad_v"), got,
           oracle.dot_softmax_backward(ei, n, qh, kh, vh, heads, channels, scale, g),
           dot_logit_mag(oracle.widen(qh), oracle.widen(kh), col, row, heads, channels, scale), kappa_dot(channels))
+
+
+# One row of 32 edges: 2^24, then 31 ones.  A one added to 2^24 in fp32 is lost (half a
+# unit in the last place, ties to even), so one chain over a 32-edge window ends 31 short.
+# With a second lane group or a second chain at most 15 ones meet the large term and the
+# two sums' own addition rounds by at most 1: |error| <= 16.  Rows of 17 to 31 slices have
+# 32 lanes or two tiles of 16.  Enough rows that windows begin at every place in a row.
+BIG, CHAIN_BOUND = 2.0 ** 24, 16.0
+
+
+def chain_graph(rows):
+    src = np.ones((rows, 32), np.int64) + rows        # node rows: the large term, rows + 1: one
+    src[:, 0] = rows
+    return np.stack([src.reshape(-1), np.repeat(np.arange(rows), 32)]), rows + 2
+
+
+def chain_values(n, f, dtype):
+    x = torch.ones(n, f, device="cuda")
+    x[n - 2] = BIG
+    return x.to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+
+
+def assert_short_chains(got, want, bound, what):
+    worst = float((got.double() - want).abs().max())
+    assert worst <= bound, f"{what}: {worst} > {bound}"
+
+
+@pytest.mark.parametrize("f,dtype", [(68, "f32"), (100, "f32"), (124, "f32"), (136, "bf16"), (200, "bf16"),
+                                     (248, "bf16")])
+def test_sums_of_17_to_31_slices_keep_two_chains(f, dtype):
+    rows = 20000
+    ei, n = chain_graph(rows)
+    csr = tfg.tfg_build_csr(dev(ei), n)
+    x = chain_values(n, f, dtype)
+    assert_short_chains(tfg.tfg_aggregate_sum(csr.rowptr, csr.col, x)[:rows], BIG + 31, CHAIN_BOUND, "sum")
+    one = torch.ones(n, device="cuda")                # dinv: the edges' weights and the row's factor
+    gcn = tfg.tfg_gcn_aggregate_sum(csr.rowptr, csr.col, one, x, None, 0, 1.0)[:rows]
+    assert_short_chains(gcn, BIG + 31, CHAIN_BOUND, "gcn")
+    hop = tfg.tfg_sgc_propagate(csr.rowptr, csr.col, one, x, 1)[:rows]
+    assert_short_chains(hop, BIG + 31, CHAIN_BOUND, "hop")
+
+
+@pytest.mark.parametrize("heads,channels,dtype", [(3, 32, "f32"), (5, 16, "f32"), (7, 16, "f32"), (1, 100, "f32"),
+                                                  (3, 64, "bf16"), (5, 32, "bf16")])
+def test_attention_over_17_to_31_slices_keeps_two_chains(heads, channels, dtype):
+    f = heads * channels
+    ei, n = chain_graph(20000)
+    rows = n - 2
+    csr = tfg.tfg_build_csr(dev(ei), n)
+    x, zero = chain_values(n, f, dtype), torch.zeros(f, device="cuda")
+    # equal logits: every weight is 1 / 32, and the division is exact
+    out, _ = tfg.tfg_edge_softmax_aggregate(csr.rowptr, csr.col, x, heads, channels, zero, zero, 0.2)
+    assert_short_chains(out[:rows], (BIG + 31) / 32, CHAIN_BOUND / 32, "gat")
+    if channels & (channels - 1):
+        return
+    none = torch.zeros_like(x)
+    out, _ = tfg.tfg_dot_edge_softmax_aggregate(csr.rowptr, csr.col, none, none, x, heads, channels, 1.0)
+    assert_short_chains(out[:rows], (BIG + 31) / 32, CHAIN_BOUND / 32, "dot")
+    # by target: dalpha = 0 and beta = -1, so grad_q = sum of k / 32
+    src = tfg.tfg_build_csr_by_source(dev(ei), n)
+    g = torch.zeros(n, heads, channels, device="cuda")
+    g[:, :, 0] = 1
+    g = g.view(n, f)
+    gq, _, _ = tfg.tfg_dot_edge_softmax_aggregate_backward(csr.rowptr, csr.col, src.rowptr, src.col, none, x, none,
+                                                           heads, channels, 1.0, -g, g)
+    assert_short_chains(gq[:rows], (BIG + 31) / 32, CHAIN_BOUND / 32, "grad_q")
+    # by source: 32 out-edges, each the only in-edge of its target, so alpha = 1
+    rows = 4000
+    n = 33 * rows
+    ei = np.stack([np.tile(np.arange(rows), 32), np.arange(rows, n)])
+    csr, src = tfg.tfg_build_csr(dev(ei), n), tfg.tfg_build_csr_by_source(dev(ei), n)
+    none = torch.zeros(n, f, device="cuda", dtype=x.dtype)
+    g = torch.ones(n, f, device="cuda")
+    g[rows:2 * rows] = BIG
+    _, _, gv = tfg.tfg_dot_edge_softmax_aggregate_backward(csr.rowptr, csr.col, src.rowptr, src.col, none, none, none,
+                                                           heads, channels, 1.0, none.float(), g)
+    assert_short_chains(gv[:rows], BIG + 31, CHAIN_BOUND, "grad_v")
