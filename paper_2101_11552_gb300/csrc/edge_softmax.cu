@@ -484,8 +484,7 @@ cudaError_t walk_vec(const GatArgs &a, cudaStream_t s) {
     const int64_t slices = static_cast<int64_t>(a.heads) * a.channels / VEC;
     if (slices <= 8) return launch_walk<GatByTarget<XT, VEC, 8, 1, 1, false>>(a, s);
     if (slices <= 16) return launch_walk<GatByTarget<XT, VEC, 16, 1, 1, false>>(a, s);
-    if (slices < 32) return launch_walk<GatByTarget<XT, VEC, 32, 1, 1, false, 2>>(a, s);
-    return launch_walk<GatByTarget<XT, VEC, 32, 1, 1, false>>(a, s);
+    return launch_walk<GatByTarget<XT, VEC, 32, 1, 1, false, 2>>(a, s);
 }
 template <typename XT, int LPR, int T>
 cudaError_t walk_lanes(const GatArgs &a, cudaStream_t s) {

@@ -142,7 +142,11 @@ struct GatLane {
 // of the weighted rows is taken first, so an edge costs what it does in the
 // forward and the dot products are taken once per row.
 // CH: chains of additions a lane keeps within a window, edge by edge in turn: two in
-// rows of 17 to 31 slices, whose 32 lanes leave one lane group.
+// rows of more than 16 slices, whose 32 lanes leave one lane group.  softmax_fast adds a
+// window's weights on 32 / H score lanes and rescales once a window, a lane here after every
+// step of D edges; with one chain the walk's error against 64 bits was 1-5 % above
+// it, with two it is 1-4 % below, and the walk is faster: 8 x 16 fp32 on 169,343 nodes 157
+// us against 186, on 100,000 nodes of mean in-degree 24 168 against 188.
 template <typename XT, int VEC, int LPR, int T, int NH, bool TARGET_BWD, int CH = 1>
 struct GatByTarget {
     using V = VecLoad<XT, VEC>;

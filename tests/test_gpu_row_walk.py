@@ -226,8 +226,8 @@ def test_gradient_slices_of_32_bytes(heads, channels, dtype, offset):
 # One row of 32 edges: 2^24, then 31 ones.  A one added to 2^24 in fp32 is lost (half a
 # unit in the last place, ties to even), so one chain over a 32-edge window ends 31 short.
 # With a second lane group or a second chain at most 15 ones meet the large term and the
-# two sums' own addition rounds by at most 1: |error| <= 16.  Rows of 17 to 31 slices have
-# 32 lanes or two tiles of 16.  Enough rows that windows begin at every place in a row.
+# two sums' own addition rounds by at most 1: |error| <= 16.  Rows of 17 and more slices
+# have one lane group.  Enough rows that windows begin at every place in a row.
 BIG, CHAIN_BOUND = 2.0 ** 24, 16.0
 
 
@@ -261,6 +261,18 @@ def test_sums_of_17_to_31_slices_keep_two_chains(f, dtype):
     assert_short_chains(gcn, BIG + 31, CHAIN_BOUND, "gcn")
     hop = tfg.tfg_sgc_propagate(csr.rowptr, csr.col, one, x, 1)[:rows]
     assert_short_chains(hop, BIG + 31, CHAIN_BOUND, "hop")
+
+
+@pytest.mark.parametrize("heads,channels,dtype", [(8, 16, "f32"), (4, 32, "f32"), (1, 128, "f32"), (4, 64, "bf16"),
+                                                  (2, 128, "f32")])
+def test_gat_over_32_slices_keeps_two_chains(heads, channels, dtype):
+    f = heads * channels
+    ei, n = chain_graph(20000)
+    csr = tfg.tfg_build_csr(dev(ei), n)
+    zero = torch.zeros(f, device="cuda")
+    out, _ = tfg.tfg_edge_softmax_aggregate(csr.rowptr, csr.col, chain_values(n, f, dtype), heads, channels, zero,
+                                            zero, 0.2)
+    assert_short_chains(out[:n - 2], (BIG + 31) / 32, CHAIN_BOUND / 32, "gat")
 
 
 @pytest.mark.parametrize("heads,channels,dtype", [(3, 32, "f32"), (5, 16, "f32"), (7, 16, "f32"), (1, 100, "f32"),
