@@ -18,8 +18,7 @@
 //                       backward on long rows, GatByTarget's walk otherwise: one
 //                       online pass gives the softmax statistics and ds_dst
 //   by source           (the same layouts) GatBySource's walk: alpha from the
-//                       statistics, grad_x and ds_src.  Both passes sum weighted
-//                       rows and take the dot products once per row, not per edge.
+//                       statistics, grad_x and ds_src
 //   bwd_targets,        the same two passes for any other layout, one warp per
 //   bwd_sources         row: lanes cover the features in tiles of 32, a head's dot
 //                       products finished by a butterfly over its lanes per edge
@@ -563,25 +562,33 @@ cudaError_t walk_targets(const GatArgs &a, cudaStream_t s) {
     const int slices = a.heads * a.channels / VEC;
     if (slices <= 8) return launch_walk<GatByTarget<XT, VEC, 8, 1, 1, true>>(a, s);
     if (slices <= 16) return launch_walk<GatByTarget<XT, VEC, 16, 1, 1, true>>(a, s);
-    return launch_walk<GatByTarget<XT, VEC, 32, 1, 1, true>>(a, s);
+    return launch_walk<GatByTarget<XT, VEC, 32, 1, 1, true, 2>>(a, s);
 }
-// 32-byte gradient slices pay on long rows only: they take fewer, register-rich
-// warps.  8 x 16 bf16, 32- / 16-byte slices, us: mean degree 492 (114.6M edges) 4685 /
-// 5418, 100 (20M) 1025 / 1018, 50 664 / 594, 16 367 / 272; 4 x 16 fp32 at 100 566 / 586,
-// at 50 399 / 394.
+// 32-byte gradient slices pay on long rows only: they take fewer, register-rich warps.
+// Forward + backward with 32- / 16-byte slices, us: 10M edges of mean degree 100, 8 x 16
+// bf16 1241 / 1287, fp32 1418 / 1470, 4 x 32 bf16 1163 / 1223; 4M edges of mean degree 40
+// 730 / 725, 784 / 788, 693 / 694.
 #ifndef TFG_GW_WIDE_DEGREE
-#define TFG_GW_WIDE_DEGREE 128
+#define TFG_GW_WIDE_DEGREE 64
 #endif
+// lanes of a head: a power of two up to the lanes of a row
+template <typename XT, int VEC, int LPR, int LH = 1>
+cudaError_t walk_sources_lanes(const GatArgs &a, cudaStream_t s) {
+    if constexpr (LH < LPR) {
+        if (a.channels / VEC > LH) return walk_sources_lanes<XT, VEC, LPR, 2 * LH>(a, s);
+    }
+    return launch_walk<GatBySource<XT, VEC, LPR, LH>>(a, s);
+}
 template <typename XT>
 cudaError_t walk_sources(const GatArgs &a, int64_t e, cudaStream_t s) {
     const int slices = a.heads * a.channels / 4;
     if (e >= TFG_GW_WIDE_DEGREE * a.n && slices > 8 && a.channels % 8 == 0 && reinterpret_cast<uintptr_t>(a.grad_out) % 32 == 0) {
-        if (slices <= 16) return launch_walk<GatBySource<XT, 8, 8, 1, 1>>(a, s);
-        return launch_walk<GatBySource<XT, 8, 16, 1, 1>>(a, s);
+        if (slices <= 16) return walk_sources_lanes<XT, 8, 8>(a, s);
+        return walk_sources_lanes<XT, 8, 16>(a, s);
     }
-    if (slices <= 8) return launch_walk<GatBySource<XT, 4, 8, 1, 1>>(a, s);
-    if (slices <= 16) return launch_walk<GatBySource<XT, 4, 16, 1, 1>>(a, s);
-    return launch_walk<GatBySource<XT, 4, 32, 1, 1>>(a, s);
+    if (slices <= 8) return walk_sources_lanes<XT, 4, 8>(a, s);
+    if (slices <= 16) return walk_sources_lanes<XT, 4, 16>(a, s);
+    return walk_sources_lanes<XT, 4, 32>(a, s);
 }
 
 template <typename XT, int NT>

@@ -118,11 +118,10 @@ __device__ __forceinline__ float leaky(float v, float slope) { return v > 0.f ? 
 //    p of its (edge, head) from the score lane holding it with one shuffle,
 //    and accumulates p * x into fp32 per-chunk partials.
 //
-// BWD: the backward by target, as in GatByTarget: the rows are weighted with
-// p times the LeakyReLU's slope at the edge, whose sum the score lanes keep in
-// ph; out is then the forward's output, and grad_out, stats and ds_dst are set
-// (114.6M edges, 8 x 16 bf16: 2.66 ms against 3.46 ms for a pass that finished
-// <grad_out[t], x[src]> per edge with a butterfly).
+// BWD: the backward by target, as in GatByTarget: a feature lane adds p times the
+// LeakyReLU's slope at the edge times its share of dalpha - beta; out is then the
+// forward's output, and grad_out, stats and ds_dst are set (114.6M edges, 8 x 16 bf16: 2.66 ms against 3.46 ms for a pass that
+// finished <grad_out[t], x[src]> per edge with a butterfly).
 template <typename XT, int VEC, int LPR, int H, bool BWD>
 __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
                                          const int32_t *__restrict__ col,
@@ -160,9 +159,20 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
     // chunk's logits, the running maximum m of each head absorbs the chunk's
     // maximum (earlier sums are rescaled by exp(m_old - m_new) when it rises),
     // then p = exp(l - m) weights the chunk's gathered rows
-    float m = -CUDART_INF_F, den = 0.f, ph = 0.f, acc[VEC];
+    float m = -CUDART_INF_F, den = 0.f, acc[VEC];
 #pragma unroll
     for (int q = 0; q < VEC; ++q) acc[q] = 0.f;
+    float gt[VEC], beta = 0.f, dz = 0.f;             // BWD: the lane's slice of grad_out[t], its shares of beta and ds_dst
+    if constexpr (BWD) {
+        float ov[VEC];
+#pragma unroll
+        for (int q = 0; q < VEC; ++q) gt[q] = ov[q] = 0.f;
+        if (fok) {
+            gw_load(grad_out + t * f + f0, gt);
+            gw_load(out + t * f + f0, ov);
+        }
+        beta = gw_dot(gt, ov);
+    }
 #if TFG_SM_PREFETCH
     int cnext = 0;   // the next chunk's column ids (lane j: edge j of that chunk)
 #endif
@@ -198,32 +208,31 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
         if (lane_any(rises)) {   // warp-uniform; rare after the first chunks
             const float sc = rises ? (m == -CUDART_INF_F ? 0.f : exp2f(m - cm)) : 1.f;
             den *= sc;
-            if (BWD) ph *= sc;
             const float fsc = lane_get(sc, fh);   // lane fh scores head fh
+            if constexpr (BWD) {
+                dz *= fsc;
+            } else {
 #pragma unroll
-            for (int q = 0; q < VEC; ++q) acc[q] *= fsc;
+                for (int q = 0; q < VEC; ++q) acc[q] *= fsc;
+            }
             m = fmaxf(m, cm);
         }
-        float den_part = 0.f, ph_part = 0.f;
+        float den_part = 0.f;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int k = r * ES + se;
             p[r] = (FULL || k < cnt) ? exp2f(p[r] - m) : 0.f;
             den_part += p[r];
-            if (BWD) {
-                p[r] = sv[r] + sd > 0.f ? p[r] : slope * p[r];
-                ph_part += p[r];
-            }
+            if (BWD) p[r] = sv[r] + sd > 0.f ? p[r] : slope * p[r];
         }
         den += den_part;
-        if (BWD) ph += ph_part;
 #if TFG_SM_PREFETCH >= 2
         // the next chunk's node scores, requested before this chunk's rows
 #pragma unroll
         for (int r = 0; r < R; ++r)
             sv[r] = __ldg(s_src + static_cast<int64_t>(lane_get(cnext, r * ES + se)) * H + sh);
 #endif
-        float part[VEC];
+        float part[VEC], zpart = 0.f;
 #pragma unroll
         for (int q = 0; q < VEC; ++q) part[q] = 0.f;
 #pragma unroll
@@ -244,7 +253,9 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
             for (int u = 0; u < kSmUnroll; ++u) {
                 float v[VEC];
                 V::widen(raw[u], v);
-                if constexpr (VEC % 2 == 0) {
+                if constexpr (BWD) {
+                    zpart = fmaf(pw[u], gw_dot(gt, v) - beta, zpart);
+                } else if constexpr (VEC % 2 == 0) {
                     const float2 w2 = make_float2(pw[u], pw[u]);
 #pragma unroll
                     for (int q = 0; q < VEC; q += 2) {
@@ -259,8 +270,12 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
                 }
             }
         }
+        if constexpr (BWD) {
+            dz += zpart;
+        } else {
 #pragma unroll
-        for (int q = 0; q < VEC; ++q) acc[q] += part[q];
+            for (int q = 0; q < VEC; ++q) acc[q] += part[q];
+        }
     };
 #if TFG_SM_PREFETCH
     // the next chunk's column ids are requested before this chunk's rows
@@ -285,31 +300,21 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
 #pragma unroll
     for (int o = H; o < 32; o <<= 1) den += lane_xor(den, o);
 #pragma unroll
-    for (int o = LPR; o < 32; o <<= 1)
+    for (int o = LPR; o < 32; o <<= 1) {
+        if constexpr (BWD) {
+            dz += lane_xor(dz, o);
+        } else {
 #pragma unroll
-        for (int q = 0; q < VEC; ++q) acc[q] += lane_xor(acc[q], o);
+            for (int q = 0; q < VEC; ++q) acc[q] += lane_xor(acc[q], o);
+        }
+    }
     const float dh = lane_get(den, fh);   // lane fh holds head fh's denominator
     if constexpr (BWD) {
-#pragma unroll
-        for (int o = H; o < 32; o <<= 1) ph += lane_xor(ph, o);
-        const float phh = lane_get(ph, fh), mh = lane_get(m, fh), sdh = lane_get(sd, fh);
-        float b = 0.f, d = 0.f;
-        if (fok) {
-            float gv[VEC], ov[VEC];
-            gw_load(grad_out + t * f + f0, gv);
-            gw_load(out + t * f + f0, ov);
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) {
-                b = fmaf(gv[q], ov[q], b);
-                d = fmaf(gv[q], acc[q], d);
-            }
-        }
-        for (int o = 1; o < channels / VEC; o <<= 1) {
-            b += lane_xor(b, o);
-            d += lane_xor(d, o);
-        }
+        const float mh = lane_get(m, fh), sdh = lane_get(sd, fh);
+        const int hl = channels / VEC;               // lanes of a head, a power of two
+        const float d = gw_head_sum<0>(dz, hl), b = gw_head_sum<0>(beta, hl);
         if (lane < LPR && fok && f0 % channels == 0) {
-            ds_dst[t * H + fh] = end > beg ? (d - b * phh) / dh : 0.f;
+            ds_dst[t * H + fh] = end > beg ? d / dh : 0.f;
             stats[t * H + fh] = make_float4(sdh, mh, end > beg ? 1.f / dh : 0.f, b);
         }
         return;

@@ -45,7 +45,7 @@ namespace {
 #define TFG_GW_WARPS 28
 #endif
 #ifndef TFG_GW_SRC_WARPS
-#define TFG_GW_SRC_WARPS 24
+#define TFG_GW_SRC_WARPS 28
 #endif
 // Gathers in flight per lane: 4 against 2 (forward 147 us / 3.20 ms) and 8 with
 // 16 warps (239 us / 2.99 ms).
@@ -65,9 +65,6 @@ namespace {
 #endif
 #ifndef TFG_GW_SRC8_DEPTH
 #define TFG_GW_SRC8_DEPTH 4
-#endif
-#ifndef TFG_GW_SRC_UNROLL
-#define TFG_GW_SRC_UNROLL 8
 #endif
 
 template <int VEC>
@@ -112,6 +109,65 @@ __device__ __forceinline__ void gw_store(float *p, const float (&r)[VEC]) {
     }
 }
 
+// A lane's share of a dot product.  Eight features are two fours added, as two lanes of
+// four would be by the first exchange of a head's sum: the sum over a head has the same
+// bits in either slice width (and in gw_spread_sums), so that a difference of two equal
+// products is zero whichever pass formed each.
+template <int VEC>
+__device__ __forceinline__ float gw_dot(const float (&a)[VEC], const float (&b)[VEC]) {
+    static_assert(VEC == 4 || VEC == 8, "whole 16-byte slices");
+    float r[VEC / 4];
+#pragma unroll
+    for (int i = 0; i < VEC / 4; ++i) {
+        float2 d = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 4 * i; q < 4 * i + 4; q += 2)
+            d = fma2(make_float2(a[q], a[q + 1]), make_float2(b[q], b[q + 1]), d);
+        r[i] = d.x + d.y;
+    }
+    return VEC == 8 ? r[0] + r[VEC / 4 - 1] : r[0];
+}
+
+// Sum over the lanes of a head (a power of two: LH, or hl where LH = 0), to each of them.
+template <int LH>
+__device__ __forceinline__ float gw_head_sum(float v, int hl) {
+    if constexpr (LH > 0) {
+#pragma unroll
+        for (int o = 1; o < LH; o <<= 1) v += lane_xor(v, o);
+    } else {
+        for (int o = 1; o < hl; o <<= 1) v += lane_xor(v, o);
+    }
+    return v;
+}
+
+// The head sums of D values, spread over the LH lanes of the head: in log2(LH) exchanges
+// each lane gives away one half of its values and takes its neighbour's other half, so
+// that D - 1 values are exchanged instead of D log2(LH).  The lane ends with the first
+// max(1, D / LH) entries of v complete; w and b follow their values.  lane: the lane's
+// place in the head.  Lanes left with the same value (LH > D): all but the first get w = 0.
+template <int LH, int D>
+__device__ __forceinline__ void gw_spread_sums(float (&v)[D], float (&w)[D], float (&b)[D], int lane) {
+    int n = D;
+#pragma unroll
+    for (int o = 1; o < LH; o <<= 1) {
+        const bool up = (lane & o) != 0;
+        if (n > 1) {
+            n /= 2;
+#pragma unroll
+            for (int i = 0; i < D / 2; ++i) {
+                if (i >= n) continue;
+                const float give = up ? v[i] : v[n + i];
+                v[i] = (up ? v[n + i] : v[i]) + lane_xor(give, o);
+                w[i] = up ? w[n + i] : w[i];
+                b[i] = up ? b[n + i] : b[i];
+            }
+        } else {
+            v[0] += lane_xor(v[0], o);
+            w[0] = up ? 0.f : w[0];
+        }
+    }
+}
+
 // 2^(m_old - m_new) for base-2 maxima; 0 for an empty state (m_old = -inf).
 __device__ __forceinline__ float gw_rescale(float m_old, float m_new) {
     return m_old == -CUDART_INF_F ? 0.f : exp2f(m_old - m_new);
@@ -136,11 +192,14 @@ struct GatLane {
 };
 
 // Softmax passes by target.  TARGET_BWD = false: out = sum of alpha x, and alpha
-// if wanted.  TARGET_BWD = true: the row's statistics for the source pass and
-//   ds_dst = sum of alpha phi (dalpha - beta) = <grad_out[t], sum of alpha phi x> - beta sum of alpha phi,
-// phi the LeakyReLU's slope at the edge, dalpha = <grad_out[t], x[src]>: the sum
-// of the weighted rows is taken first, so an edge costs what it does in the
-// forward and the dot products are taken once per row.
+// if wanted.  TARGET_BWD = true (one slice a lane, T = 1): the row's statistics for the
+// source pass and
+//   ds_dst = sum of alpha phi (dalpha - beta),  dalpha = <grad_out[t], x[src]>,
+// phi the LeakyReLU's slope at the edge.  A lane keeps its own slice's share of dalpha and
+// of beta = <grad_out[t], out[t]>, subtracts them edge by edge, and the shares are added
+// over the lanes of the head once a row: an edge costs what it does in the forward, and
+// the difference, which cancels where an edge has most of its row's weight (to nothing
+// where t has one in-edge), is taken before anything is rounded to a larger sum.
 // CH: chains of additions a lane keeps within a window, edge by edge in turn: two in
 // rows of more than 16 slices, whose 32 lanes leave one lane group.  softmax_fast adds a
 // window's weights on 32 / H score lanes and rescales once a window, a lane here after every
@@ -152,7 +211,9 @@ struct GatByTarget {
     using V = VecLoad<XT, VEC>;
     static constexpr int kWarps = TFG_GW_WARPS, kLpr = LPR, G = 32 / LPR;
     static constexpr int kTile = LPR * VEC * T, kHeadsPerLane = T;
-    static constexpr int kState = T * VEC + NH * (TARGET_BWD ? 3 : 2), kHeld = 0;
+    static constexpr int kSums = TARGET_BWD ? 1 : T * VEC;      // dz, or acc
+    static constexpr int kState = kSums + 2 * NH, kHeld = 0;
+    static_assert(!TARGET_BWD || (T == 1 && NH == 1), "the backward has one slice a lane");
     static constexpr int D = TFG_GW_DEPTH * G > 32 ? 32 / G : TFG_GW_DEPTH;   // gathers in flight per lane
     static_assert(32 % (G * D) == 0 && D % CH == 0, "a full window is read in whole steps");
     const GatArgs &a;
@@ -160,7 +221,8 @@ struct GatByTarget {
     const char *xb;
     uint32_t row_bytes;
     float *scratch;                      // [warp][heads of the tile] (m, den), for alpha
-    float sd[NH], m[NH], den[NH], phi[NH], acc[T][VEC];
+    float sd[NH], m[NH], den[NH], acc[T][VEC];
+    float gt[TARGET_BWD ? VEC : 1], beta, dz;   // backward: this slice of grad_out[t], its share of beta and of the sum
 
     __device__ __forceinline__ GatByTarget(const GatArgs &args, uint32_t ft, float *, float *scr) : a(args), scratch(scr) {
         at.place(ft, a.heads, a.channels);
@@ -171,8 +233,9 @@ struct GatByTarget {
 #pragma unroll
         for (int i = 0; i < NH; ++i) {
             m[i] = -CUDART_INF_F;
-            den[i] = phi[i] = 0.f;
+            den[i] = 0.f;
         }
+        dz = 0.f;
 #pragma unroll
         for (int i = 0; i < T; ++i)
 #pragma unroll
@@ -182,11 +245,22 @@ struct GatByTarget {
 #pragma unroll
         for (int i = 0; i < NH; ++i)
             sd[i] = __ldg(a.s_dst + static_cast<uint64_t>(static_cast<uint32_t>(t)) * a.heads + at.head[i]);
+        if constexpr (TARGET_BWD) {
+            float o[VEC];
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) gt[q] = o[q] = 0.f;
+            if (at.own > 0) {
+                const uint64_t row = static_cast<uint64_t>(static_cast<uint32_t>(t)) * at.f + at.f0;
+                gw_load(a.grad_out + row, gt);
+                gw_load(a.fwd_out + row, o);
+            }
+            beta = gw_dot(gt, o);
+        }
         clear();
     }
     template <bool CHECK>
     __device__ __forceinline__ void add(const int32_t *ids, int cnt) {
-        float part[CH][T][VEC], dpart[CH][NH], ppart[NH];   // sums are blocked per window
+        float part[CH][T][VEC], dpart[CH][NH], zpart[CH];   // sums are blocked per window
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
 #pragma unroll
@@ -194,7 +268,8 @@ struct GatByTarget {
 #pragma unroll
                 for (int q = 0; q < VEC; ++q) part[c][i][q] = 0.f;
 #pragma unroll
-            for (int i = 0; i < NH; ++i) dpart[c][i] = ppart[i] = 0.f;
+            for (int i = 0; i < NH; ++i) dpart[c][i] = 0.f;
+            zpart[c] = 0.f;
         }
         const int32_t *sp = ids + at.g;
         int left = cnt - at.g;                              // this group's edges: sp[0], sp[G], ... below left
@@ -228,15 +303,15 @@ struct GatByTarget {
                 if (top > m[i]) {                           // a new running maximum: rescale the sums so far
                     const float sc = gw_rescale(m[i], top);
                     den[i] *= sc;
+                    dz *= sc;
 #pragma unroll
-                    for (int c = 0; c < CH; ++c) dpart[c][i] *= sc;
-                    if (TARGET_BWD) {
-                        phi[i] *= sc;
-                        ppart[i] *= sc;
+                    for (int c = 0; c < CH; ++c) {
+                        dpart[c][i] *= sc;
+                        zpart[c] *= sc;
                     }
 #pragma unroll
                     for (int j = 0; j < T; ++j) {
-                        if (NH > 1 && j != i) continue;
+                        if (TARGET_BWD || (NH > 1 && j != i)) continue;
 #pragma unroll
                         for (int q = 0; q < VEC; ++q) {
                             acc[j][q] *= sc;
@@ -250,11 +325,7 @@ struct GatByTarget {
                 for (int u = 0; u < D; ++u) {
                     const float p = !CHECK || left > u * G ? exp2f(l[u][i] - m[i]) : 0.f;
                     dpart[u % CH][i] += p;
-                    w[u][i] = p;
-                    if (TARGET_BWD) {
-                        w[u][i] = z[u][i] > 0.f ? p : a.slope * p;
-                        ppart[i] += w[u][i];
-                    }
+                    w[u][i] = TARGET_BWD && z[u][i] <= 0.f ? a.slope * p : p;
                 }
             }
 #pragma unroll
@@ -263,33 +334,42 @@ struct GatByTarget {
                 for (int i = 0; i < T; ++i) {
                     float v[VEC];
                     V::widen(raw[u][i], v);
-                    gw_axpy(part[u % CH][i], w[u][NH > 1 ? i : 0], v);
+                    if constexpr (TARGET_BWD) {
+                        const float diff = gw_dot(gt, v) - beta;
+                        zpart[u % CH] = fmaf(w[u][0], !CHECK || left > u * G ? diff : 0.f, zpart[u % CH]);
+                    } else {
+                        gw_axpy(part[u % CH][i], w[u][NH > 1 ? i : 0], v);
+                    }
                 }
             sp += G * D;
             left -= G * D;
         }
 #pragma unroll
-        for (int i = 0; i < NH; ++i) {
-            den[i] += CH == 1 ? dpart[0][i] : dpart[0][i] + dpart[CH - 1][i];
-            if (TARGET_BWD) phi[i] += ppart[i];
-        }
+        for (int i = 0; i < NH; ++i) den[i] += CH == 1 ? dpart[0][i] : dpart[0][i] + dpart[CH - 1][i];
 #pragma unroll
         for (int i = 0; i < T; ++i)
 #pragma unroll
-            for (int q = 0; q < VEC; ++q) acc[i][q] += CH == 1 ? part[0][i][q] : part[0][i][q] + part[CH - 1][i][q];
+            for (int q = 0; q < VEC; ++q) {
+                if (CH > 1) part[0][i][q] += part[CH - 1][i][q];
+                acc[i][q] += part[0][i][q];
+            }
+        dz += CH == 1 ? zpart[0] : zpart[0] + zpart[CH - 1];
     }
-    // this state and (m2, den2, phi2, acc2), element by element
+    // this state and (sums, m, den) of another, element by element
     template <class Get>
     __device__ __forceinline__ void fold(Get get) {
         float sa[NH], sb[NH];
 #pragma unroll
         for (int i = 0; i < NH; ++i) {
-            const float m2 = get(m[i], T * VEC + i), mm = fmaxf(m[i], m2);
+            const float m2 = get(m[i], kSums + i), mm = fmaxf(m[i], m2);
             sa[i] = gw_rescale(m[i], mm);
             sb[i] = gw_rescale(m2, mm);
-            den[i] = den[i] * sa[i] + get(den[i], T * VEC + NH + i) * sb[i];
-            if (TARGET_BWD) phi[i] = phi[i] * sa[i] + get(phi[i], T * VEC + 2 * NH + i) * sb[i];
+            den[i] = den[i] * sa[i] + get(den[i], kSums + NH + i) * sb[i];
             m[i] = mm;
+        }
+        if constexpr (TARGET_BWD) {
+            dz = dz * sa[0] + get(dz, 0) * sb[0];
+            return;
         }
 #pragma unroll
         for (int i = 0; i < T; ++i)
@@ -306,15 +386,18 @@ struct GatByTarget {
     }
     __device__ __forceinline__ void park(float *slot) const {
         if (at.g != 0) return;
+        if constexpr (TARGET_BWD) {
+            slot[at.sub] = dz;
+        } else {
 #pragma unroll
-        for (int i = 0; i < T; ++i)
+            for (int i = 0; i < T; ++i)
 #pragma unroll
-            for (int q = 0; q < VEC; ++q) slot[(i * VEC + q) * LPR + at.sub] = acc[i][q];
+                for (int q = 0; q < VEC; ++q) slot[(i * VEC + q) * LPR + at.sub] = acc[i][q];
+        }
 #pragma unroll
         for (int i = 0; i < NH; ++i) {
-            slot[(T * VEC + i) * LPR + at.sub] = m[i];
-            slot[(T * VEC + NH + i) * LPR + at.sub] = den[i];
-            if (TARGET_BWD) slot[(T * VEC + 2 * NH + i) * LPR + at.sub] = phi[i];
+            slot[(kSums + i) * LPR + at.sub] = m[i];
+            slot[(kSums + NH + i) * LPR + at.sub] = den[i];
         }
     }
     __device__ __forceinline__ void close(int32_t t, int32_t beg, int32_t end, bool shared) {
@@ -337,33 +420,11 @@ struct GatByTarget {
                 if (!shared) weights(warp, t, beg, end, threadIdx.x & 31, 32);
             }
         } else {
-            // beta = <grad_out[t], out[t]> and <grad_out[t], acc> per head: this
-            // lane's share, then over the lanes of the head (a power of two of them)
-            const int hl = a.channels / VEC;
-            const uint64_t th = static_cast<uint64_t>(static_cast<uint32_t>(t)) * a.heads;
-#pragma unroll
-            for (int i = 0; i < T; ++i) {
-                float b = 0.f, d = 0.f;
-                if (i < at.own) {
-                    float g[VEC], o[VEC];
-                    gw_load(a.grad_out + row + i * LPR * VEC, g);
-                    gw_load(a.fwd_out + row + i * LPR * VEC, o);
-#pragma unroll
-                    for (int q = 0; q < VEC; ++q) {
-                        b = fmaf(g[q], o[q], b);
-                        d = fmaf(g[q], acc[i][q], d);
-                    }
-                }
-                for (int o = 1; o < hl; o <<= 1) {
-                    b += lane_xor(b, o);
-                    d += lane_xor(d, o);
-                }
-                if (at.g == 0 && i < at.own && (at.f0 + i * LPR * VEC) % a.channels == 0) {
-                    const int k = NH > 1 ? i : 0;
-                    const int h = static_cast<int>((at.f0 + i * LPR * VEC) / a.channels);
-                    a.ds_dst[th + h] = any ? (d - b * phi[k]) / den[k] : 0.f;
-                    a.stats[th + h] = make_float4(sd[k], m[k], any ? 1.f / den[k] : 0.f, b);
-                }
+            const float d = gw_head_sum<0>(dz, a.channels / VEC), b = gw_head_sum<0>(beta, a.channels / VEC);
+            if (at.g == 0 && at.own > 0 && at.f0 % a.channels == 0) {
+                const uint64_t th = static_cast<uint64_t>(static_cast<uint32_t>(t)) * a.heads + at.head[0];
+                a.ds_dst[th] = any ? d / den[0] : 0.f;
+                a.stats[th] = make_float4(sd[0], m[0], any ? 1.f / den[0] : 0.f, b);
             }
         }
     }
@@ -425,122 +486,100 @@ struct GatByTarget {
     }
 };
 
-// Backward by source (CSR by source: ids are targets).  With P = sum of alpha
-// grad_out[t] and Q = sum of alpha phi grad_out[t] over the out-edges,
-//   ds_src = sum of alpha phi (dalpha - beta) = <x[s], Q> - sum of alpha phi beta,
-//   grad_x = P + ds_src a_src + ds_dst a_dst:
-// no dot product per edge.  Every lane forms alpha of its head from the target's
-// statistics.
-template <typename XT, int VEC, int LPR, int T, int NH>
+// Backward by source (CSR by source: ids are targets).  grad_x = P + ds_src a_src +
+// ds_dst a_dst with P = sum of alpha grad_out[t] over the out-edges, and
+//   ds_src = sum of alpha phi (dalpha - beta).
+// The lanes of a head finish dalpha edge by edge (gw_spread_sums), so that beta of the
+// target is subtracted before anything is summed, as in the pass by target.  Every lane
+// forms alpha of its head from the target's statistics.  LH: lanes of a head.
+template <typename XT, int VEC, int LPR, int LH>
 struct GatBySource {
     using V = VecLoad<float, VEC>;
     static constexpr int kWarps = VEC == 8 ? TFG_GW_SRC8_WARPS : TFG_GW_SRC_WARPS, kLpr = LPR, G = 32 / LPR;
-    static constexpr int kTile = LPR * VEC * T, kHeadsPerLane = T;
-    static constexpr int kState = 2 * T * VEC + NH, kHeld = 0;
+    static constexpr int kTile = LPR * VEC, kHeadsPerLane = 1;
+    static constexpr int kState = VEC + 1, kHeld = 0;
     static constexpr int kDepth = VEC == 8 ? TFG_GW_SRC8_DEPTH : TFG_GW_SRC_DEPTH;
     static constexpr int D = kDepth * G > 32 ? 32 / G : kDepth;
     static_assert(32 % (G * D) == 0, "a full window is read in whole steps");
-    static constexpr int kUnroll = 32 / (G * D) < TFG_GW_SRC_UNROLL ? 32 / (G * D) : TFG_GW_SRC_UNROLL;
+    static constexpr int kOwnSums = D > LH ? D / LH : 1;         // edges of a step whose sums a lane ends with
+    static constexpr int kUnroll = VEC == 8 ? 32 / (G * D) : 1;      // steps of a full window unrolled
     const GatArgs &a;
-    GatLane<VEC, LPR, T, NH> at;
+    GatLane<VEC, LPR, 1, 1> at;
     const char *gb;
     uint32_t row_bytes;
-    float ss[NH], sb[NH], P[T][VEC], Q[T][VEC];
+    float ss, ds, xs[VEC], P[VEC];           // ds: this lane's share
 
     __device__ __forceinline__ GatBySource(const GatArgs &args, uint32_t ft, float *, float *) : a(args) {
         at.place(ft, a.heads, a.channels);
         gb = reinterpret_cast<const char *>(a.grad_out + (at.own > 0 ? at.f0 : 0));
         row_bytes = at.f * 4u;
     }
+    __device__ __forceinline__ uint64_t element(int32_t s) const {   // feature f0 of row s
+        return static_cast<uint64_t>(static_cast<uint32_t>(s)) * at.f + at.f0;
+    }
     __device__ __forceinline__ void clear() {
+        ds = 0.f;
 #pragma unroll
-        for (int i = 0; i < NH; ++i) sb[i] = 0.f;
-#pragma unroll
-        for (int i = 0; i < T; ++i)
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) P[i][q] = Q[i][q] = 0.f;
+        for (int q = 0; q < VEC; ++q) P[q] = 0.f;
     }
     __device__ __forceinline__ void open(int32_t s, int32_t, int32_t) {
+        ss = __ldg(a.s_src + static_cast<uint64_t>(static_cast<uint32_t>(s)) * a.heads + at.head[0]);
 #pragma unroll
-        for (int i = 0; i < NH; ++i)
-            ss[i] = __ldg(a.s_src + static_cast<uint64_t>(static_cast<uint32_t>(s)) * a.heads + at.head[i]);
+        for (int q = 0; q < VEC; ++q) xs[q] = 0.f;
+        if (at.own > 0) VecLoad<XT, VEC>::load(static_cast<const XT *>(a.x) + element(s), xs);
         clear();
     }
     template <bool CHECK>
     __device__ __forceinline__ void add(const int32_t *ids, int cnt) {
-        float p[T][VEC], r[T][VEC], bpart[NH];
+        float p[VEC], part = 0.f;
 #pragma unroll
-        for (int i = 0; i < T; ++i)
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) p[i][q] = r[i][q] = 0.f;
-#pragma unroll
-        for (int i = 0; i < NH; ++i) bpart[i] = 0.f;
+        for (int q = 0; q < VEC; ++q) p[q] = 0.f;
         const int32_t *sp = ids + at.g;
         int left = cnt - at.g;
 #pragma unroll CHECK ? 1 : kUnroll
         for (int e = 0; e < (CHECK ? cnt : 32); e += G * D) {
-            typename V::Raw raw[D][T];
-            float4 st[D][NH];
+            typename V::Raw raw[D];
+            float4 st[D];
 #pragma unroll
             for (int u = 0; u < D; ++u) {
                 const uint32_t id = static_cast<uint32_t>(sp[u * G]);
                 const bool ok = !CHECK || left > u * G;
                 const float *row = reinterpret_cast<const float *>(gb + static_cast<uint64_t>(id) * row_bytes);
-#pragma unroll
-                for (int i = 0; i < NH; ++i)
-                    st[u][i] = ok ? __ldg(a.stats + static_cast<uint64_t>(id) * a.heads + at.head[i])
-                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int i = 0; i < T; ++i) {
-                    const bool on = T == 1 ? ok : ok && i < at.own;
-                    if constexpr (VEC == 8) raw[u][i] = CHECK || T > 1 ? V::raw(on, row + i * LPR * VEC) : V::raw(row + i * LPR * VEC);
-                    else raw[u][i] = on ? V::raw(row + i * LPR * VEC) : V::zero();
-                }
+                st[u] = ok ? __ldg(a.stats + static_cast<uint64_t>(id) * a.heads + at.head[0])
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+                if constexpr (VEC == 8) raw[u] = CHECK ? V::raw(ok, row) : V::raw(row);
+                else raw[u] = ok ? V::raw(row) : V::zero();
             }
+            float dots[D], af[D], beta[D];
 #pragma unroll
             for (int u = 0; u < D; ++u) {
-                float al[NH], af[NH];
-#pragma unroll
-                for (int i = 0; i < NH; ++i) {
-                    const float z = ss[i] + st[u][i].x;
-                    const float l = z > 0.f ? z : a.slope * z;
-                    al[i] = exp2f(l - st[u][i].y) * st[u][i].z;
-                    if (CHECK) al[i] = left > u * G ? al[i] : 0.f;
-                    af[i] = z > 0.f ? al[i] : a.slope * al[i];
-                    bpart[i] = fmaf(af[i], st[u][i].w, bpart[i]);
-                }
-#pragma unroll
-                for (int i = 0; i < T; ++i) {
-                    float v[VEC];
-                    V::widen(raw[u][i], v);
-                    gw_axpy(p[i], al[NH > 1 ? i : 0], v);
-                    gw_axpy(r[i], af[NH > 1 ? i : 0], v);
-                }
+                const float z = ss + st[u].x;
+                const float l = z > 0.f ? z : a.slope * z;
+                float al = exp2f(l - st[u].y) * st[u].z;
+                if (CHECK) al = left > u * G ? al : 0.f;
+                af[u] = z > 0.f ? al : a.slope * al;
+                beta[u] = st[u].w;
+                float v[VEC];
+                V::widen(raw[u], v);
+                gw_axpy(p, al, v);
+                dots[u] = gw_dot(xs, v);
             }
+            gw_spread_sums<LH>(dots, af, beta, at.sub);
+#pragma unroll
+            for (int u = 0; u < D; ++u)
+                if (u < kOwnSums) part = fmaf(af[u], dots[u] - beta[u], part);
             sp += G * D;
             left -= G * D;
         }
+        ds += part;
 #pragma unroll
-        for (int i = 0; i < NH; ++i) sb[i] += bpart[i];
-#pragma unroll
-        for (int i = 0; i < T; ++i)
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) {
-                P[i][q] += p[i][q];
-                Q[i][q] += r[i][q];
-            }
+        for (int q = 0; q < VEC; ++q) P[q] += p[q];
     }
     template <class Get>
     __device__ __forceinline__ void fold(Get get) {
 #pragma unroll
-        for (int i = 0; i < T; ++i)
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) {
-                P[i][q] += get(P[i][q], i * VEC + q);
-                Q[i][q] += get(Q[i][q], (T + i) * VEC + q);
-            }
-#pragma unroll
-        for (int i = 0; i < NH; ++i) sb[i] += get(sb[i], 2 * T * VEC + i);
+        for (int q = 0; q < VEC; ++q) P[q] += get(P[q], q);
+        ds += get(ds, VEC);
     }
     __device__ __forceinline__ void join() {
 #pragma unroll
@@ -552,44 +591,23 @@ struct GatBySource {
     __device__ __forceinline__ void park(float *slot) const {
         if (at.g != 0) return;
 #pragma unroll
-        for (int i = 0; i < T; ++i)
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) {
-                slot[(i * VEC + q) * LPR + at.sub] = P[i][q];
-                slot[((T + i) * VEC + q) * LPR + at.sub] = Q[i][q];
-            }
-#pragma unroll
-        for (int i = 0; i < NH; ++i) slot[(2 * T * VEC + i) * LPR + at.sub] = sb[i];
+        for (int q = 0; q < VEC; ++q) slot[q * LPR + at.sub] = P[q];
+        slot[VEC * LPR + at.sub] = ds;
     }
     __device__ __forceinline__ bool wants_after() const { return false; }
     __device__ __forceinline__ void after(int, int32_t, int32_t, int32_t) {}
     __device__ __forceinline__ void close(int32_t s, int32_t, int32_t, bool) {
-        const uint64_t row = static_cast<uint64_t>(static_cast<uint32_t>(s)) * at.f + at.f0;
-        const uint64_t sh = static_cast<uint64_t>(static_cast<uint32_t>(s)) * a.heads;
-        const int hl = a.channels / VEC;
+        const float dz = gw_head_sum<LH>(ds, LH);
+        if (at.g != 0 || at.own == 0) return;
+        const uint64_t sh = static_cast<uint64_t>(static_cast<uint32_t>(s)) * a.heads + at.head[0];
+        const float dd = __ldg(a.ds_dst + sh);
+        float as[VEC], ad[VEC], r[VEC];
+        gw_load(a.a_src + at.f0, as);
+        gw_load(a.a_dst + at.f0, ad);
 #pragma unroll
-        for (int i = 0; i < T; ++i) {
-            float d = 0.f;
-            if (i < at.own) {
-                float xs[VEC];
-                VecLoad<XT, VEC>::load(static_cast<const XT *>(a.x) + row + i * LPR * VEC, xs);
-#pragma unroll
-                for (int q = 0; q < VEC; ++q) d = fmaf(xs[q], Q[i][q], d);
-            }
-            for (int o = 1; o < hl; o <<= 1) d += lane_xor(d, o);
-            if (at.g == 0 && i < at.own) {
-                const uint32_t fi = at.f0 + i * LPR * VEC;
-                const int h = static_cast<int>(fi / a.channels);
-                const float ds = d - sb[NH > 1 ? i : 0], dd = __ldg(a.ds_dst + sh + h);
-                float as[VEC], ad[VEC], r[VEC];
-                gw_load(a.a_src + fi, as);
-                gw_load(a.a_dst + fi, ad);
-#pragma unroll
-                for (int q = 0; q < VEC; ++q) r[q] = P[i][q] + ds * as[q] + dd * ad[q];
-                gw_store(a.grad_x + row + i * LPR * VEC, r);
-                if (fi % a.channels == 0) a.ds_src[sh + h] = ds;
-            }
-        }
+        for (int q = 0; q < VEC; ++q) r[q] = P[q] + dz * as[q] + dd * ad[q];
+        gw_store(a.grad_x + element(s), r);
+        if (at.f0 % a.channels == 0) a.ds_src[sh] = dz;
     }
 };
 

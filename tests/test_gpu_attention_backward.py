@@ -143,3 +143,29 @@ def test_gat_backward_is_deterministic_and_rejects_bad_layouts():
         tfg.tfg_edge_softmax_backward_workspace_size(100, 2, 24)     # 24: not a power of two
     with pytest.raises(tfg.TfgError):
         tfg.tfg_edge_softmax_backward_workspace_size(100, 4, 128)    # F = 512 > 256
+
+
+# in-edges of a target, all from one source: the walk; softmax_fast; by source 32-byte slices
+@pytest.mark.parametrize("copies", [1, 32, 128])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("heads,channels", [(8, 16), (4, 8), (1, 64), (3, 32), (1, 128), (16, 4), (5, 8)])
+def test_gat_backward_cancels_where_a_row_has_one_source(heads, channels, dtype, copies):
+    """Then out[t] = x[src] exactly (features of 8 significant bits, so the sums of up to 128
+    copies are exact), dalpha = beta, and every logit's gradient is zero.  dalpha and beta
+    are the same sums in the same order in every slice width, so the difference taken edge
+    by edge is zero exactly; a sum formed before the subtraction leaves its rounding."""
+    n, f = 3000, heads * channels
+    rng = np.random.default_rng(51)
+    src = rng.integers(0, 64, size=n)
+    ei = np.stack([np.repeat(src, copies), np.repeat(np.arange(n), copies)])
+    bits = gg.bf16_bits_rne(rng.standard_normal((n, f)).astype(np.float32))
+    xh = bits if dtype == "bf16" else oracle.widen(bits).astype(np.float32)
+    x = dev(xh.view(np.int16)).view(torch.bfloat16) if dtype == "bf16" else dev(xh)
+    a_s, a_d = rng.standard_normal((2, f)).astype(np.float32)
+    g = rng.standard_normal((n, f)).astype(np.float32)
+    gx, ga, gd, _ = _run(gg.Workload("copies", n, ei, None), x, heads, channels, a_s, a_d, g)
+    rgx, _, _, (sx, _, _) = oracle.edge_softmax_backward(ei, n, xh, heads, channels, a_s, a_d, 0.2, g)
+    what = f"{dtype} H={heads} C={channels} copies={copies}"
+    assert np.array_equal(gd, np.zeros(f, np.float32)), "grad_a_dst " + what
+    assert np.array_equal(ga, np.zeros(f, np.float32)), "grad_a_src " + what
+    assert_scaled_close(gx, rgx, sx, TOL_F32, "grad_x " + what)
