@@ -177,7 +177,7 @@ struct MaxBwd {
 // One row by one warp, feature tiles of 32 * VEC.
 template <int VEC, bool MASKED>
 __device__ void max_warp_row(const MaxBwdArgs &a, int64_t s, int lane) {
-    const int64_t beg = a.rowptr[s], end = a.col ? a.rowptr[s + 1] : beg;
+    const int64_t beg = a.rowptr[s], end = a.rowptr[s + 1];
     for (int64_t f0 = lane * VEC, ft = 0; ft < a.f; ft += 32 * VEC, f0 += 32 * VEC) {
         MaxBwd<VEC, MASKED> st;
         st.init();
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kMxThreads, MASKED ? TFG_MXB_MINB : 4) max_bwd
         i = lane_get(i, 0);
         if (i >= nrows) break;
         const int64_t s = r0 + i;
-        if (a.col != nullptr && a.rowptr[s + 1] - a.rowptr[s] > kMxHeavyDeg) {
+        if (a.rowptr[s + 1] - a.rowptr[s] > kMxHeavyDeg) {
             int slot = 0;
             if (lane == 0) slot = atomicAdd(&s_nheavy, 1);
             slot = lane_get(slot, 0);
