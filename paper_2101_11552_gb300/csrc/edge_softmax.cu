@@ -40,12 +40,6 @@ constexpr int kSmThreads = 256;
 #define TFG_SM_UNROLL 4   // gathers in flight per lane (tuning knob)
 #endif
 constexpr int kSmUnroll = TFG_SM_UNROLL;
-// 1: the next chunk's column ids are requested one chunk ahead; 2: also its
-// node scores s_src, gathered while this chunk's rows are summed (measured on
-// the 114.6M-edge graph: 2.29 ms with 2, 2.40-2.50 ms with 1, 2.44-2.57 ms with 0)
-#ifndef TFG_SM_PREFETCH
-#define TFG_SM_PREFETCH 2
-#endif
 #ifndef TFG_SM_FULL_CHUNKS
 #define TFG_SM_FULL_CHUNKS 1   // separate code for full 32-edge chunks (no slot tests)
 #endif
@@ -173,12 +167,14 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
         }
         beta = gw_dot(gt, ov);
     }
-#if TFG_SM_PREFETCH
-    int cnext = 0;   // the next chunk's column ids (lane j: edge j of that chunk)
-#endif
-#if TFG_SM_PREFETCH >= 2
+    // The next chunk's column ids are requested one chunk ahead, and its node scores
+    // gathered while this chunk's rows are summed (114.6M edges: 2.29 ms; ids alone
+    // ahead 2.40-2.50, neither 2.44-2.57).
+    int cnext = (col && beg + lane < end) ? ld_stream(col + beg + lane) : 0;   // lane j: edge j of the next chunk
     float sv[R];     // s_src of the chunk about to run, for (edge r * ES + se, head sh)
-#endif
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        sv[r] = __ldg(s_src + static_cast<int64_t>(lane_get(cnext, r * ES + se)) * H + sh);
     // one 32-edge chunk with its column ids in c (lane j: edge base + j; any
     // valid id past cnt); FULL chunks (all 32 slots used) skip every slot test
     auto chunk = [&](auto full_tag, int c, int cnt) {
@@ -194,12 +190,7 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int k = r * ES + se;
-#if TFG_SM_PREFETCH >= 2
-            const float ss = sv[r];                  // gathered during the previous chunk
-#else
-            const float ss = __ldg(s_src + static_cast<int64_t>(lane_get(c, k)) * H + sh);
-#endif
-            p[r] = (FULL || k < cnt) ? leaky(ss + sd, slope) : -CUDART_INF_F;
+            p[r] = (FULL || k < cnt) ? leaky(sv[r] + sd, slope) : -CUDART_INF_F;
             cm = fmaxf(cm, p[r]);
         }
 #pragma unroll
@@ -226,12 +217,10 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
             if (BWD) p[r] = sv[r] + sd > 0.f ? p[r] : slope * p[r];
         }
         den += den_part;
-#if TFG_SM_PREFETCH >= 2
         // the next chunk's node scores, requested before this chunk's rows
 #pragma unroll
         for (int r = 0; r < R; ++r)
             sv[r] = __ldg(s_src + static_cast<int64_t>(lane_get(cnext, r * ES + se)) * H + sh);
-#endif
         float part[VEC], zpart = 0.f;
 #pragma unroll
         for (int q = 0; q < VEC; ++q) part[q] = 0.f;
@@ -277,23 +266,10 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
             for (int q = 0; q < VEC; ++q) acc[q] += part[q];
         }
     };
-#if TFG_SM_PREFETCH
-    // the next chunk's column ids are requested before this chunk's rows
-    cnext = (col && beg + lane < end) ? ld_stream(col + beg + lane) : 0;
-#endif
-#if TFG_SM_PREFETCH >= 2
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-        sv[r] = __ldg(s_src + static_cast<int64_t>(lane_get(cnext, r * ES + se)) * H + sh);
-#endif
     for (int64_t base = beg; base < end; base += 32) {
         const int cnt = static_cast<int>(min64(32, end - base));
-#if TFG_SM_PREFETCH
         const int c = cnext;
         cnext = (base + 32 + lane < end) ? ld_stream(col + base + 32 + lane) : 0;
-#else
-        const int c = lane < cnt ? ld_stream(col + base + lane) : 0;
-#endif
         if (kSmFullChunks && cnt == 32) chunk(std::true_type{}, c, 32);
         else chunk(std::false_type{}, c, cnt);
     }
@@ -347,7 +323,10 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
 // 169,343 nodes, mean in-degree 6.9, 8 x 16 fp32: walk 145 us, softmax_fast's
 // earlier merge-path form 164 us; 114.6M edges, mean 492, bf16: walk 2.64-2.68
 // ms, softmax_fast 2.20 ms.
-constexpr int64_t kWalkMaxDegree = 32;
+#ifndef TFG_SM_WALK_DEGREE
+#define TFG_SM_WALK_DEGREE 32
+#endif
+constexpr int64_t kWalkMaxDegree = TFG_SM_WALK_DEGREE;
 
 // Measured on the 114.6M-edge graph (bf16, 8 heads x 16), ids and scores
 // requested one chunk ahead: 3 CTAs per SM with 4 gathers in flight per lane
@@ -382,6 +361,7 @@ softmax_fast_bwd(const int32_t *__restrict__ rowptr, const int32_t *__restrict__
     });
 }
 
+constexpr int kFastBwdHeads = 8;       // the backward's most: 16 score steps a chunk and its sums spill
 constexpr int64_t kSmMinWork = 2048;   // edges + rows per CTA, at least
 
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
@@ -396,11 +376,12 @@ bool launch_fast_lpr(const GatArgs &a, int64_t e, bool bwd, cudaStream_t s) {
 #define TFG_FAST(HH)                                                                              \
     if (a.heads == HH) {                                                                          \
         if constexpr ((32 / HH) % G == 0) {                                                       \
-            if (bwd)                                                                              \
-                softmax_fast_bwd<XT, VEC, LPR, HH><<<grid, kSmThreads, 0, s>>>(                   \
-                    a.rowptr, a.col, xp, a.n, a.channels, a.slope, a.s_src, a.s_dst,              \
-                    const_cast<float *>(a.fwd_out), a.grad_out, a.stats, a.ds_dst);               \
-            else                                                                                  \
+            if (bwd) {                                                                            \
+                if constexpr (HH <= kFastBwdHeads)                                                \
+                    softmax_fast_bwd<XT, VEC, LPR, HH><<<grid, kSmThreads, 0, s>>>(               \
+                        a.rowptr, a.col, xp, a.n, a.channels, a.slope, a.s_src, a.s_dst,          \
+                        const_cast<float *>(a.fwd_out), a.grad_out, a.stats, a.ds_dst);           \
+            } else                                                                                \
                 softmax_fast<XT, VEC, LPR, HH><<<grid, kSmThreads, 0, s>>>(                       \
                     a.rowptr, a.col, xp, a.n, a.channels, a.slope, a.s_src, a.s_dst, a.out, a.alpha); \
             return true;                                                                          \
@@ -420,7 +401,7 @@ template <typename XT, int VEC>
 bool launch_fast(const GatArgs &a, int64_t e, bool bwd, cudaStream_t s) {
     const int64_t f = static_cast<int64_t>(a.heads) * a.channels;
     if (a.channels % VEC != 0 || f > 32 * VEC || e < kWalkMaxDegree * a.n) return false;
-    if (bwd && a.heads > 8) return false;   // 16 score steps a chunk and the backward's sums spill
+    if (bwd && a.heads > kFastBwdHeads) return false;
     const int64_t chunks = f / VEC;
     if (chunks > 16) return launch_fast_lpr<XT, VEC, 32>(a, e, bwd, s);
     if (chunks > 8) return launch_fast_lpr<XT, VEC, 16>(a, e, bwd, s);
