@@ -468,6 +468,7 @@ namespace {
 template <typename XT, int VEC>
 cudaError_t walk_vec(const GatArgs &a, cudaStream_t s) {
     const int64_t slices = static_cast<int64_t>(a.heads) * a.channels / VEC;
+    if (slices <= 4) return launch_walk<GatByTarget<XT, VEC, 4, 1, 1, false>>(a, s);
     if (slices <= 8) return launch_walk<GatByTarget<XT, VEC, 8, 1, 1, false>>(a, s);
     if (slices <= 16) return launch_walk<GatByTarget<XT, VEC, 16, 1, 1, false>>(a, s);
     return launch_walk<GatByTarget<XT, VEC, 32, 1, 1, false, 2>>(a, s);

@@ -209,13 +209,14 @@ struct GatLane {
 template <typename XT, int VEC, int LPR, int T, int NH, bool TARGET_BWD, int CH = 1>
 struct GatByTarget {
     using V = VecLoad<XT, VEC>;
-    static constexpr int kWarps = TFG_GW_WARPS, kLpr = LPR, G = 32 / LPR;
+    static constexpr int kWarps = LPR == 4 ? 32 : TFG_GW_WARPS, kLpr = LPR, G = 32 / LPR;
     static constexpr int kTile = LPR * VEC * T, kHeadsPerLane = T;
     static constexpr int kSums = TARGET_BWD ? 1 : T * VEC;      // dz, or acc
     static constexpr int kState = kSums + 2 * NH, kHeld = 0;
     static_assert(!TARGET_BWD || (T == 1 && NH == 1), "the backward has one slice a lane");
-    static constexpr int D = TFG_GW_DEPTH * G > 32 ? 32 / G : TFG_GW_DEPTH;   // gathers in flight per lane
-    static_assert(32 % (G * D) == 0 && D % CH == 0, "a full window is read in whole steps");
+    static constexpr int kStepFull = TFG_GW_DEPTH * G > 32 ? 32 / G : TFG_GW_DEPTH;   // gathers in flight per lane
+    static_assert(32 % (G * kStepFull) == 0, "a full window is read in whole steps");
+    static constexpr int kStepPart = walk_part(G) < kStepFull ? walk_part(G) : kStepFull;   // the same, a window's rest
     const GatArgs &a;
     GatLane<VEC, LPR, T, NH> at;
     const char *xb;
@@ -258,102 +259,109 @@ struct GatByTarget {
         }
         clear();
     }
+    // a window's sums
+    struct Window {
+        float part[CH][T][VEC], dpart[CH][NH], zpart[CH];
+    };
+    // D edges of the group, sp[0], sp[G], ... (CHECK: those below left)
+    template <int D, bool CHECK>
+    __device__ __forceinline__ void step(const int32_t *sp, int left, Window &s) {
+        static_assert(D % CH == 0, "a step gives every chain the same number of edges");
+        typename V::Raw raw[D][T];
+        float z[D][NH];
+#pragma unroll
+        for (int u = 0; u < D; ++u) {
+            const uint32_t id = static_cast<uint32_t>(sp[u * G]);
+            const bool ok = !CHECK || left > u * G;
+            const XT *row = reinterpret_cast<const XT *>(xb + static_cast<uint64_t>(id) * row_bytes);
+#pragma unroll
+            for (int i = 0; i < NH; ++i)
+                z[u][i] = ok ? __ldg(a.s_src + static_cast<uint64_t>(id) * a.heads + at.head[i]) : 0.f;
+#pragma unroll
+            for (int i = 0; i < T; ++i)
+                raw[u][i] = (T == 1 ? ok : ok && i < at.own) ? V::raw(row + i * LPR * VEC) : V::zero();
+        }
+        float l[D][NH], w[D][NH];
+#pragma unroll
+        for (int i = 0; i < NH; ++i) {
+            float top = m[i];
+#pragma unroll
+            for (int u = 0; u < D; ++u) {
+                z[u][i] += sd[i];
+                l[u][i] = z[u][i] > 0.f ? z[u][i] : a.slope * z[u][i];
+                if (CHECK && left <= u * G) l[u][i] = -CUDART_INF_F;
+                top = fmaxf(top, l[u][i]);
+            }
+            if (top > m[i]) {                           // a new running maximum: rescale the sums so far
+                const float sc = gw_rescale(m[i], top);
+                den[i] *= sc;
+                dz *= sc;
+#pragma unroll
+                for (int c = 0; c < CH; ++c) {
+                    s.dpart[c][i] *= sc;
+                    s.zpart[c] *= sc;
+                }
+#pragma unroll
+                for (int j = 0; j < T; ++j) {
+                    if (TARGET_BWD || (NH > 1 && j != i)) continue;
+#pragma unroll
+                    for (int q = 0; q < VEC; ++q) {
+                        acc[j][q] *= sc;
+#pragma unroll
+                        for (int c = 0; c < CH; ++c) s.part[c][j][q] *= sc;
+                    }
+                }
+                m[i] = top;
+            }
+#pragma unroll
+            for (int u = 0; u < D; ++u) {
+                const float p = !CHECK || left > u * G ? exp2f(l[u][i] - m[i]) : 0.f;
+                s.dpart[u % CH][i] += p;
+                w[u][i] = TARGET_BWD && z[u][i] <= 0.f ? a.slope * p : p;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < D; ++u)
+#pragma unroll
+            for (int i = 0; i < T; ++i) {
+                float v[VEC];
+                V::widen(raw[u][i], v);
+                if constexpr (TARGET_BWD) {
+                    const float diff = gw_dot(gt, v) - beta;
+                    s.zpart[u % CH] = fmaf(w[u][0], !CHECK || left > u * G ? diff : 0.f, s.zpart[u % CH]);
+                } else {
+                    gw_axpy(s.part[u % CH][i], w[u][NH > 1 ? i : 0], v);
+                }
+            }
+    }
     template <bool CHECK>
     __device__ __forceinline__ void add(const int32_t *ids, int cnt) {
-        float part[CH][T][VEC], dpart[CH][NH], zpart[CH];   // sums are blocked per window
+        Window s;                                           // sums are blocked per window
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
 #pragma unroll
             for (int i = 0; i < T; ++i)
 #pragma unroll
-                for (int q = 0; q < VEC; ++q) part[c][i][q] = 0.f;
+                for (int q = 0; q < VEC; ++q) s.part[c][i][q] = 0.f;
 #pragma unroll
-            for (int i = 0; i < NH; ++i) dpart[c][i] = 0.f;
-            zpart[c] = 0.f;
+            for (int i = 0; i < NH; ++i) s.dpart[c][i] = 0.f;
+            s.zpart[c] = 0.f;
         }
         const int32_t *sp = ids + at.g;
-        int left = cnt - at.g;                              // this group's edges: sp[0], sp[G], ... below left
 #pragma unroll 1
-        for (int e = 0; e < cnt; e += G * D) {
-            typename V::Raw raw[D][T];
-            float z[D][NH];
+        for (; cnt >= G * kStepFull; cnt -= G * kStepFull, sp += G * kStepFull) step<kStepFull, false>(sp, 0, s);
+#pragma unroll 1
+        for (; CHECK && cnt > 0; cnt -= G * kStepPart, sp += G * kStepPart) step<kStepPart, true>(sp, cnt - at.g, s);
 #pragma unroll
-            for (int u = 0; u < D; ++u) {
-                const uint32_t id = static_cast<uint32_t>(sp[u * G]);
-                const bool ok = !CHECK || left > u * G;
-                const XT *row = reinterpret_cast<const XT *>(xb + static_cast<uint64_t>(id) * row_bytes);
-#pragma unroll
-                for (int i = 0; i < NH; ++i)
-                    z[u][i] = ok ? __ldg(a.s_src + static_cast<uint64_t>(id) * a.heads + at.head[i]) : 0.f;
-#pragma unroll
-                for (int i = 0; i < T; ++i)
-                    raw[u][i] = (T == 1 ? ok : ok && i < at.own) ? V::raw(row + i * LPR * VEC) : V::zero();
-            }
-            float l[D][NH], w[D][NH];
-#pragma unroll
-            for (int i = 0; i < NH; ++i) {
-                float top = m[i];
-#pragma unroll
-                for (int u = 0; u < D; ++u) {
-                    z[u][i] += sd[i];
-                    l[u][i] = z[u][i] > 0.f ? z[u][i] : a.slope * z[u][i];
-                    if (CHECK && left <= u * G) l[u][i] = -CUDART_INF_F;
-                    top = fmaxf(top, l[u][i]);
-                }
-                if (top > m[i]) {                           // a new running maximum: rescale the sums so far
-                    const float sc = gw_rescale(m[i], top);
-                    den[i] *= sc;
-                    dz *= sc;
-#pragma unroll
-                    for (int c = 0; c < CH; ++c) {
-                        dpart[c][i] *= sc;
-                        zpart[c] *= sc;
-                    }
-#pragma unroll
-                    for (int j = 0; j < T; ++j) {
-                        if (TARGET_BWD || (NH > 1 && j != i)) continue;
-#pragma unroll
-                        for (int q = 0; q < VEC; ++q) {
-                            acc[j][q] *= sc;
-#pragma unroll
-                            for (int c = 0; c < CH; ++c) part[c][j][q] *= sc;
-                        }
-                    }
-                    m[i] = top;
-                }
-#pragma unroll
-                for (int u = 0; u < D; ++u) {
-                    const float p = !CHECK || left > u * G ? exp2f(l[u][i] - m[i]) : 0.f;
-                    dpart[u % CH][i] += p;
-                    w[u][i] = TARGET_BWD && z[u][i] <= 0.f ? a.slope * p : p;
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < D; ++u)
-#pragma unroll
-                for (int i = 0; i < T; ++i) {
-                    float v[VEC];
-                    V::widen(raw[u][i], v);
-                    if constexpr (TARGET_BWD) {
-                        const float diff = gw_dot(gt, v) - beta;
-                        zpart[u % CH] = fmaf(w[u][0], !CHECK || left > u * G ? diff : 0.f, zpart[u % CH]);
-                    } else {
-                        gw_axpy(part[u % CH][i], w[u][NH > 1 ? i : 0], v);
-                    }
-                }
-            sp += G * D;
-            left -= G * D;
-        }
-#pragma unroll
-        for (int i = 0; i < NH; ++i) den[i] += CH == 1 ? dpart[0][i] : dpart[0][i] + dpart[CH - 1][i];
+        for (int i = 0; i < NH; ++i) den[i] += CH == 1 ? s.dpart[0][i] : s.dpart[0][i] + s.dpart[CH - 1][i];
 #pragma unroll
         for (int i = 0; i < T; ++i)
 #pragma unroll
             for (int q = 0; q < VEC; ++q) {
-                if (CH > 1) part[0][i][q] += part[CH - 1][i][q];
-                acc[i][q] += part[0][i][q];
+                if (CH > 1) s.part[0][i][q] += s.part[CH - 1][i][q];
+                acc[i][q] += s.part[0][i][q];
             }
-        dz += CH == 1 ? zpart[0] : zpart[0] + zpart[CH - 1];
+        dz += CH == 1 ? s.zpart[0] : s.zpart[0] + s.zpart[CH - 1];
     }
     // this state and (sums, m, den) of another, element by element
     template <class Get>
@@ -377,9 +385,39 @@ struct GatByTarget {
             for (int q = 0; q < VEC; ++q)
                 acc[i][q] = acc[i][q] * sa[NH > 1 ? i : 0] + get(acc[i][q], i * VEC + q) * sb[NH > 1 ? i : 0];
     }
+    // the lane groups: their largest maximum first, one rescale, then plain sums
     __device__ __forceinline__ void join() {
+        if constexpr (G > 1) {
 #pragma unroll
-        for (int o = LPR; o < 32; o <<= 1) fold([&](float mine, int) { return lane_xor(mine, o); });
+            for (int i = 0; i < NH; ++i) {
+                float top = m[i];
+#pragma unroll
+                for (int o = LPR; o < 32; o <<= 1) top = fmaxf(top, lane_xor(top, o));
+                const float sc = gw_rescale(m[i], top);
+                den[i] *= sc;
+                dz *= sc;
+#pragma unroll
+                for (int j = 0; j < T; ++j) {
+                    if (TARGET_BWD || (NH > 1 && j != i)) continue;
+#pragma unroll
+                    for (int q = 0; q < VEC; ++q) acc[j][q] *= sc;
+                }
+                m[i] = top;
+            }
+#pragma unroll
+            for (int o = LPR; o < 32; o <<= 1) {
+#pragma unroll
+                for (int i = 0; i < NH; ++i) den[i] += lane_xor(den[i], o);
+                if constexpr (TARGET_BWD) {
+                    dz += lane_xor(dz, o);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < T; ++i)
+#pragma unroll
+                        for (int q = 0; q < VEC; ++q) acc[i][q] += lane_xor(acc[i][q], o);
+                }
+            }
+        }
     }
     __device__ __forceinline__ void merge(const float *slot) {
         fold([&](float, int q) { return slot[q * LPR + at.sub]; });

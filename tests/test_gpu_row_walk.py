@@ -69,7 +69,7 @@ def test_widths(f, dtype):
 # layouts of one slice per lane, several features per lane (one head and many),
 # and more than one feature tile; backward where the layout has one
 LAYOUTS = [(1, 3), (1, 41), (1, 100), (3, 5), (2, 9), (5, 13), (1, 130), (7, 20), (8, 16), (4, 8),
-           (1, 32), (2, 64), (3, 4), (16, 4), (6, 32), (12, 4)]
+           (1, 32), (2, 64), (3, 4), (16, 4), (6, 32), (12, 4), (1, 4), (1, 8), (4, 4), (5, 4)]
 
 
 @pytest.mark.parametrize("more", [0, 1000])     # mean in-degree 72 and 6
