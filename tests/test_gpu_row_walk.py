@@ -59,11 +59,15 @@ def test_widths(f, dtype):
         ref, scale = oracle.gcn_aggregate(ei, n, finite, None if w is None else np.abs(w), 1, 1.0)
         assert np.isinf(got[-1]).all()
         assert_scaled_close(got[:-1], ref[:-1], scale[:-1], TOL_F32, f"gcn F={f}")
-    out = tfg.tfg_appnp_propagate(csr.rowptr, csr.col, dinv, dev(finite) if dtype == "f32" else
-                                  dev(finite.view(np.int16)).view(torch.bfloat16), 3, 0.1,
-                                  add_self_loops=1).cpu().numpy()
-    dw = np.abs(ew)
-    assert np.isfinite(out).all() and dw.size       # values: test_gpu_propagate; here every width runs
+    # dinv is that of the weighted graph, so the weights are read from w_csr
+    x0 = dev(finite) if dtype == "f32" else dev(finite.view(np.int16)).view(torch.bfloat16)
+    out = tfg.tfg_appnp_propagate(csr.rowptr, csr.col, dinv, x0, 3, 0.1, w_csr, add_self_loops=1).cpu().numpy()
+    ref, scale = oracle.appnp(ei, n, finite, 3, 0.1, np.abs(ew), add_self_loops=1)
+    assert_scaled_close(out, ref, scale, TOL_F32, f"appnp F={f}")
+    dinv, _ = tfg.tfg_gcn_norm(csr.rowptr, csr.col, csr.perm, n, None, 1, 1.0, want_w_csr=False)
+    out = tfg.tfg_appnp_propagate(csr.rowptr, csr.col, dinv, x0, 3, 0.1, add_self_loops=1).cpu().numpy()
+    ref, scale = oracle.appnp(ei, n, finite, 3, 0.1, add_self_loops=1)
+    assert_scaled_close(out, ref, scale, TOL_F32, f"appnp, weights on the fly, F={f}")
 
 
 # layouts of one slice per lane, several features per lane (one head and many),
@@ -158,6 +162,44 @@ def test_max_argmax_widths(f, dtype):
         ref, ref_arg = oracle.max_argmax(ei, n, host_features(wl, dtype), ew)
         assert np.array_equal(arg.cpu().numpy(), ref_arg), f"argmax F={f}"
         assert_exact_f32(out.cpu().numpy(), ref, f"max F={f}")
+
+
+@pytest.mark.parametrize("f", [8, 64, 72, 128, 136, 264])
+def test_plain_bf16_max_of_special_values(f):
+    """The packed bf16 max passes over NaN and knows the infinities, as the fp32 kernel
+    does on the same values: rows of one value, of NaN only, of -infinity only, a NaN first,
+    last and between, signed zeros, the largest and smallest finite values."""
+    ei, n = graph(f + 3, 300)
+    rng = np.random.default_rng(4500 + f)
+    special = np.array([np.nan, np.inf, -np.inf, 0.0, -0.0, 3.3895e38, -3.3895e38, 1.0, -2.0], np.float32)
+    x = rng.choice(special, size=(n, f), p=[.4, .05, .25, .05, .05, .05, .05, .05, .05])
+    x[:, :2] = np.nan                                  # NaN only
+    x[:, 2:4] = -np.inf
+    xb = torch.from_numpy(x).cuda().to(torch.bfloat16)
+    csr = tfg.tfg_build_csr(dev(ei), n)
+    got = tfg.tfg_aggregate_max(csr.rowptr, csr.col, xb)
+    assert torch.equal(got, tfg.tfg_aggregate_max(csr.rowptr, csr.col, xb.float()))
+    seen = np.where(np.isnan(x), -np.inf, xb.float().cpu().numpy())
+    ref, _ = oracle.aggregate(ei, n, seen.astype(np.float32), "max")
+    assert_exact_f32(got.cpu().numpy(), ref, f"max F={f}")
+
+
+@pytest.mark.parametrize("f", [33, 64, 65, 97, 128, 129, 132, 264])
+def test_max_backward_walk_widths(f):
+    """The backward's row walk where its lanes and feature tiles change, weighted and not,
+    with a source of 9,000 edges that the warps of a CTA share and sources of none."""
+    ei, n = graph(f + 4, 1000)
+    ei = np.ascontiguousarray(ei[::-1])                # the degrees are the sources'
+    rng = np.random.default_rng(4700 + f)
+    x = np.round(rng.standard_normal((n, f), dtype=np.float32) * 4) / 4
+    g = rng.standard_normal((n, f)).astype(np.float32)
+    csr, src = tfg.tfg_build_csr(dev(ei), n), tfg.tfg_build_csr_by_source(dev(ei), n)
+    for ew in (None, rng.uniform(-1.5, 1.5, ei.shape[1]).astype(np.float32)):
+        w = None if ew is None else dev(ew).index_select(0, csr.perm)
+        _, arg = tfg.tfg_aggregate_max_argmax(csr, dev(x), w)
+        got = tfg.tfg_aggregate_max_backward(src, arg, dev(g), None if ew is None else dev(ew))
+        ref, scale = oracle.max_backward(ei, n, arg.cpu().numpy(), g, ew)
+        assert_scaled_close(got.cpu().numpy(), ref, scale, TOL_F32, f"max backward F={f}")
 
 
 def test_max_argmax_of_a_row_past_16_bit_positions():
