@@ -114,8 +114,9 @@ __device__ __forceinline__ float leaky(float v, float slope) { return v > 0.f ? 
 //
 // BWD: the backward by target, as in GatByTarget: a feature lane adds p times the
 // LeakyReLU's slope at the edge times its share of dalpha - beta; out is then the
-// forward's output, and grad_out, stats and ds_dst are set (114.6M edges, 8 x 16 bf16: 2.66 ms against 3.46 ms for a pass that
-// finished <grad_out[t], x[src]> per edge with a butterfly).
+// forward's output, and grad_out, stats and ds_dst are set (114.6M edges, 8 x 16 bf16:
+// 2.74 ms against 3.44 ms for a pass that finished <grad_out[t], x[src]> per edge with a
+// butterfly).
 template <typename XT, int VEC, int LPR, int H, bool BWD>
 __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
                                          const int32_t *__restrict__ col,
@@ -319,10 +320,14 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
 
 // Graphs of a mean in-degree below this take the row walk (gat_walk.cuh), whose
 // warps share hub rows and whose windows cross row ends; longer rows take
-// softmax_fast, whose score lanes evaluate each (edge, head) once.  Measured:
-// 169,343 nodes, mean in-degree 6.9, 8 x 16 fp32: walk 145 us, softmax_fast's
-// earlier merge-path form 164 us; 114.6M edges, mean 492, bf16: walk 2.64-2.68
-// ms, softmax_fast 2.20 ms.
+// softmax_fast, whose score lanes evaluate each (edge, head) once.  Measured, walk /
+// softmax_fast, us a call: block-model graphs of 100,000 nodes, mean degree 16, 32, 64 and
+// 100, 8 x 16 bf16 128 / 140, 179 / 181, 265 / 253, 349 / 333; 8 x 16 fp32 129 / 148, 191 /
+// 208, 302 / 312, 413 / 432; 4 x 8 bf16 100 / 96, 129 / 117, 175 / 160, 226 / 231 (the walk
+// before its rest steps of 8 edges: it is 10-15 % faster now); 114.6M edges, mean 492,
+// 8 x 16 bf16 2.64-2.68 / 2.20 ms.  Where hubs hold a large part of the edges the walk is
+// faster at every degree (preferential attachment, mean 64, 8 x 16 bf16 296 / 661), but E
+// and N do not tell.
 #ifndef TFG_SM_WALK_DEGREE
 #define TFG_SM_WALK_DEGREE 32
 #endif

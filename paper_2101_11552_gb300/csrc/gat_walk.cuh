@@ -31,35 +31,36 @@ struct GatArgs {
 namespace {
 
 // What bounds it: instructions on short rows (169,343 nodes, mean in-degree 6.9, 8
-// x 16 fp32: forward 145, by target 164, by source 161 us, against 36-45 us for
+// x 16 fp32: forward 106, by target 135, by source 168 us, against 36-45 us for
 // the gathered bytes at the L2 rate), the gathers and the weights' arithmetic on
-// long ones (by source at 114.6M edges: 640 bytes an edge, 4.69 ms, 15.6 TB/s, 5.42
-// ms with 16-byte slices, 7.93 ms when each edge's dot product was finished by a
-// butterfly).  One head of 41 channels on the first graph, alpha written: 196 us;
-// 1,753 in a row-per-warp kernel whose hub rows one warp walked.
+// long ones (by source at 114.6M edges, 8 x 16 bf16: 640 bytes an edge, 4.97 ms, 14.8
+// TB/s; 7.9-8.0 ms in a row-per-warp kernel).  One head of 41 channels on the first graph,
+// alpha written: 199 us; 1,753 in a row-per-warp kernel whose hub rows one warp walked.
 //
-// Tuning knobs.  Warps per CTA (one CTA per SM), measured on the two graphs:
-// by target 28 (forward 146 us / 2.68 ms), 24 160 / 2.84, 32 136 / 2.64; by source
-// 24 161 us / 5.43 ms, 28 168 / 5.50, 20 203 / 5.42.
+// Tuning knobs.  Warps per CTA (one CTA per SM).  By target: 28 against 24 and 32 on the
+// first graph, forward 107 / 112 / 100 us, backward 135 / 149 / 131, 3 x 32 fp32 over 10M
+// edges 345 / 353 / 335 (odd widths of several heads, which spill at 28, spill more
+// at 32).  By source: 168 us with 28, 185 with 24, 181 with 32; 4M edges of mean degree
+// 40 245 / 264 / 257.
 #ifndef TFG_GW_WARPS
 #define TFG_GW_WARPS 28
 #endif
 #ifndef TFG_GW_SRC_WARPS
 #define TFG_GW_SRC_WARPS 28
 #endif
-// Gathers in flight per lane: 4 against 2 (forward 147 us / 3.20 ms) and 8 with
-// 16 warps (239 us / 2.99 ms).
+// Gathers in flight per lane: 4 against 2, 8 x 16 fp32 calls on the first graph 143 / 180
+// us; rows of 8 slices and fewer the same with either.
 #ifndef TFG_GW_DEPTH
 #define TFG_GW_DEPTH 4
 #endif
-// The same by source, and how many of its steps unroll in a full window (1:
-// 5.53 ms, 2: 6.12, 8: 5.43 at 114.6M edges).
+// The same by source: 168 / 216 us; over 114.6M edges 4.97 / 8.7 ms.
 #ifndef TFG_GW_SRC_DEPTH
 #define TFG_GW_SRC_DEPTH 4
 #endif
 // By source with 32-byte gradient slices (VEC = 8: half the lanes a row, so an edge's
-// weight is formed by half as many lanes, and twice the bytes a load): 114.6M edges
-// 4.69 ms with 16 warps and 4 in flight, 20 and 4 4.86, 24 and 2 5.98, 12 and 4 5.45.
+// weight is formed by half as many lanes, and twice the bytes a load; its full windows are
+// unrolled, 10.1 ms a call against 10.5 rolled): 114.6M edges 4.98 ms with 16 warps, 20
+// 5.25, 12 5.46.
 #ifndef TFG_GW_SRC8_WARPS
 #define TFG_GW_SRC8_WARPS 16
 #endif
