@@ -40,7 +40,8 @@ namespace {
 // Tuning knobs.  Warps per CTA (one CTA per SM).  By target: 28 against 24 and 32 on the
 // first graph, forward 107 / 112 / 100 us, backward 135 / 149 / 131, 3 x 32 fp32 over 10M
 // edges 345 / 353 / 335 (odd widths of several heads, which spill at 28, spill more
-// at 32).  By source: 168 us with 28, 185 with 24, 181 with 32; 4M edges of mean degree
+// at 32); rows of 4 lanes take 32: 4 x 8 bf16, 100,000 nodes of mean degree 29, 90 us a call
+// against 94.  By source: 168 us with 28, 185 with 24, 181 with 32; 4M edges of mean degree
 // 40 245 / 264 / 257.
 #ifndef TFG_GW_WARPS
 #define TFG_GW_WARPS 28
