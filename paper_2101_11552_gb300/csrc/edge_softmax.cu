@@ -176,8 +176,8 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
 #pragma unroll
     for (int r = 0; r < R; ++r)
         sv[r] = __ldg(s_src + static_cast<int64_t>(lane_get(cnext, r * ES + se)) * H + sh);
-    // one 32-edge chunk with its column ids in c (lane j: edge base + j; any
-    // valid id past cnt); FULL chunks (all 32 slots used) skip every slot test
+    // one 32-edge chunk with its column ids in c (lane j: edge base + j; an id of
+    // the row past cnt); FULL chunks (all 32 slots used) skip every slot test
     auto chunk = [&](auto full_tag, int c, int cnt) {
         constexpr bool FULL = decltype(full_tag)::value;
         // the first step's row gathers need only the column ids: issue them
@@ -271,8 +271,10 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
         const int cnt = static_cast<int>(min64(32, end - base));
         const int c = cnext;
         cnext = (base + 32 + lane < end) ? ld_stream(col + base + 32 + lane) : 0;
+        // slots without an edge have zero weight: they read the row of the chunk's last
+        // edge, since an infinity in another node's row would come through it
         if (kSmFullChunks && cnt == 32) chunk(std::true_type{}, c, 32);
-        else chunk(std::false_type{}, c, cnt);
+        else chunk(std::false_type{}, lane_get(c, min(lane, cnt - 1)), cnt);
     }
 #pragma unroll
     for (int o = H; o < 32; o <<= 1) den += lane_xor(den, o);

@@ -111,6 +111,33 @@ def test_gat_layouts(heads, channels, dtype, more):
         assert_scaled_close(a.cpu().numpy(), b, sc, tol, f"{name} {what}")
 
 
+@pytest.mark.parametrize("more", [0, 1000])     # softmax_fast, the walk
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("heads,channels", [(8, 16), (1, 64), (4, 8), (3, 32)])
+def test_gat_infinity_in_a_node_without_edges(heads, channels, dtype, more):
+    """Slots of a window without an edge hold id 0; node 0 has no edges, so an infinity in
+    its features reaches no output but its own gradient's vectors."""
+    f = heads * channels
+    ei, n = graph(f + 5, more)
+    ei = ei[:, (ei != 0).all(0)]
+    rng = np.random.default_rng(2500 + f)
+    x = rng.standard_normal((n, f)).astype(np.float32)
+    a_s, a_d = (dev((0.5 * rng.standard_normal(f)).astype(np.float32)) for _ in range(2))
+    g = dev(rng.standard_normal((n, f)).astype(np.float32))
+    csr, src = tfg.tfg_build_csr(dev(ei), n), tfg.tfg_build_csr_by_source(dev(ei), n)
+    got = []
+    for first in (0.0, np.inf):
+        x[0] = first
+        xd = dev(x).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+        out, alpha = tfg.tfg_edge_softmax_aggregate(csr.rowptr, csr.col, xd, heads, channels, a_s, a_d, 0.2,
+                                                    want_alpha=True)
+        gx, _, _ = tfg.tfg_edge_softmax_aggregate_backward(csr.rowptr, csr.col, src.rowptr, src.col, xd, heads,
+                                                           channels, a_s, a_d, 0.2, out, g)
+        got.append((out, alpha, gx))
+    for name, a, b in zip(("out", "alpha", "grad_x"), *got):
+        assert torch.isfinite(a).all() and torch.equal(a, b), name
+
+
 @pytest.mark.parametrize("more", [0, 1000])     # mean in-degree 72 and 6
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("heads,channels", [(1, 8), (4, 8), (5, 8), (2, 16), (8, 16), (3, 32), (2, 64),
