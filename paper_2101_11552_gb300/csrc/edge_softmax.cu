@@ -324,12 +324,12 @@ __device__ __forceinline__ void fast_row(const int32_t *__restrict__ rowptr,
 // warps share hub rows and whose windows cross row ends; longer rows take
 // softmax_fast, whose score lanes evaluate each (edge, head) once.  Measured, walk /
 // softmax_fast, us a call: block-model graphs of 100,000 nodes, mean degree 16, 32, 64 and
-// 100, 8 x 16 bf16 128 / 140, 179 / 181, 265 / 253, 349 / 333; 8 x 16 fp32 129 / 148, 191 /
-// 208, 302 / 312, 413 / 432; 4 x 8 bf16 100 / 96, 129 / 117, 175 / 160, 226 / 231 (the walk
-// before its rest steps of 8 edges: it is 10-15 % faster now); 114.6M edges, mean 492,
-// 8 x 16 bf16 2.64-2.68 / 2.20 ms.  Where hubs hold a large part of the edges the walk is
-// faster at every degree (preferential attachment, mean 64, 8 x 16 bf16 296 / 661), but E
-// and N do not tell.
+// 100, 8 x 16 bf16 115 / 140, 155 / 182, 230 / 254, 308 / 334; 8 x 16 fp32 114 / 149, 166 /
+// 208, 270 / 311, 376 / 432; 4 x 8 bf16 79 / 97, 99 / 119, 133 / 172, 163 / 234; 114.6M
+// edges, mean 492, 8 x 16 bf16 2.59 / 2.24 ms.  So the two meet between 100 and 492; the
+// line stands where they met before the walk's partial steps and has not been moved since.
+// Where hubs hold a large part of the edges the walk is faster at every degree
+// (preferential attachment, mean 64, 8 x 16 bf16 247 / 675), but E and N do not tell.
 #ifndef TFG_SM_WALK_DEGREE
 #define TFG_SM_WALK_DEGREE 32
 #endif
